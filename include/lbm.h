@@ -333,7 +333,14 @@ lbm_status lbm_set_launch(lbm_ctx* ctx, int tile_x, int rows);
  *                      finish step s - 1, so no grid-wide step boundary remains.
  *  LBM_PIPELINE_AUTO   (default) BATCHED for contexts of several instances that
  *                      all can use it; otherwise PAIRS where available, else
- *                      ASYNC, else TMA, else PLAIN.
+ *                      ASYNC, else TMA, else PLAIN. Contexts too small to fill
+ *                      the GPU with those kernels' row runs (one 512 x 512
+ *                      domain in FP32, larger in FP64; every nx even or every
+ *                      nx odd) run their unmonitored steps on tiles of at most
+ *                      256 cells instead, up to 256 steps in one cooperative
+ *                      launch in which a tile's step waits (bounded) for the
+ *                      tiles within 3 cells of it only, while the launch shape
+ *                      is the built-in one (lbm_set_launch(ctx, 0, 0)).
  * An instance that cannot use a variant falls back to PLAIN. Takes effect at
  * the next lbm_step. LBM_EINVAL for an unknown mode.
  * D3Q15 contexts: PLAIN runs the unfused step (phi, mu and the collision as
@@ -355,7 +362,9 @@ lbm_status lbm_set_pipeline(lbm_ctx* ctx, int mode);
  * direct launches (so lbm_step can itself be captured into a caller's graph). */
 lbm_status lbm_set_graphs(lbm_ctx* ctx, int enable);
 
-/* Launch index (0 .. lbm_launches_per_step - 1) of one step: strip width,
+/* Launch index (0 .. lbm_launches_per_step - 1) of one step of the row-march
+ * plan (which a context that runs its unmonitored steps on tiles has beside
+ * them, for the monitored ones): strip width,
  * number of thread blocks, and the load path it uses (0 plain, 1 cp.async,
  * 2 TMA, 3 pairs, 4 batched: the one persistent launch, whose blocks count is
  * its grid, one block per resident slot, however many descriptors it takes).
@@ -400,7 +409,8 @@ lbm_status lbm_autotune_shape(lbm_ctx* ctx, int flags, lbm_launch_shape* out);
  * best_tile_x / best_rows may be NULL. Synchronises. */
 lbm_status lbm_autotune(lbm_ctx* ctx, int* best_tile_x, int* best_rows);
 
-/* Kernel launches queued by one lbm_step(1) (for accounting); 0 on error. */
+/* Kernel launches of one step of the row-march plan (for accounting; 0 on error);
+ * a context that runs its steps on tiles (LBM_PIPELINE_AUTO) queues one. */
 int lbm_launches_per_step(const lbm_ctx* ctx);
 
 /* Kernel launches the context's lbm_step calls have queued so far (each kernel

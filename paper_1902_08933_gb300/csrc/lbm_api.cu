@@ -174,6 +174,13 @@ struct lbm_ctx {
     double* d_mon_multi = nullptr; // persistent plan, every step monitored: [64 steps][items][kMonQ] slots
     int* d_mon_multi_cnt = nullptr;   // ... [64 steps][instances][kMonSub + 1] counters
     double* d_mon_multi_sub = nullptr;  // ... and [64 steps][instances][kMonSub][kMonQ] sub-group slots
+    // tile plan (plan_tile): items, neighbours and step counters in one allocation
+    int tile_items = 0, tile_grid = 0, tile_ulog = 0, tile_occ = 0;
+    bool tile_pair = false;
+    void* d_tile = nullptr;
+    WorkItem* d_tile_work = nullptr;
+    int* d_tile_nbr = nullptr;
+    int* d_tile_done = nullptr;
     bool plan_dirty = true;
     // CUDA graph of 2 * graph_pairs steps starting from cur == 0 (built on first use,
     // dropped when the plan changes)
@@ -258,6 +265,7 @@ StepArgs step_args(const lbm_ctx* c, int in) {
     a.wait_limit = lbm::kWaitLimit;
     a.wait_extra = 0;
     a.mon_host = nullptr;
+    a.tile_ulog = 0;
     return a;
 }
 
@@ -323,6 +331,7 @@ void choose(const lbm_ctx* c, const lbm_params& p, bool f_pairs, bool f_async, b
 // or both at their end), from L2 rather than HBM.
 lbm_status plan_d3(lbm_ctx* c);
 lbm_status plan_multi(lbm_ctx* c, int sms);
+lbm_status plan_tile(lbm_ctx* c, int sms);
 lbm_status plan_batched(lbm_ctx* c, bool f_pairs, bool f_async, bool f_tma, int sms);
 lbm_status finish_plan(lbm_ctx* c);
 
@@ -338,6 +347,23 @@ bool use_batched(const lbm_ctx* c, bool f_pairs, bool f_async, bool f_tma) {
         if (variant != lbm::kPairs) return false;
     }
     return true;
+}
+
+// Run length of one domain's row march: least (waves) x (rows a run + 3 for the
+// prologue), waves of `target` blocks counted whole -- one exact wave where the
+// strips allow it; runs of at least 8 rows. *cost: that product.
+int march_rows(int ny, int strips, long long target, long long* cost) {
+    long long best = -1, best_cost = 0;
+    for (long long r = 1; r <= ny; ++r) {
+        const long long rr = (ny + r - 1) / r;
+        if (rr < 8 && r > 1) break;
+        const long long runs = (ny + rr - 1) / rr;
+        const long long waves = (strips * runs + target - 1) / target;
+        const long long k = waves * (rr + 3);
+        if (best < 0 || k < best_cost) { best = rr; best_cost = k; }
+    }
+    if (cost) *cost = best_cost;
+    return (int)best;
 }
 
 lbm_status plan(lbm_ctx* c) {
@@ -358,6 +384,8 @@ lbm_status plan(lbm_ctx* c) {
         f_tma = lbm::has_tma_t<decltype(F)::value>();
         return cudaSuccess;
     });
+    lbm_status ts = plan_tile(c, sms);
+    if (ts != LBM_OK) return ts;
     if (use_batched(c, f_pairs, f_async, f_tma)) return plan_batched(c, f_pairs, f_async, f_tma, sms);
     // Several instances: one run length for all, sized for about four waves of
     // blocks (blocks of different instances differ in width and length, so one
@@ -397,19 +425,7 @@ lbm_status plan(lbm_ctx* c) {
                     occ = lbm::step_occupancy_t<decltype(F)::value>(tx, variant);
                     return cudaSuccess;
                 });
-                // runs per strip: least (waves) x (rows a run + 3 for the prologue),
-                // waves counted whole -- one exact wave where the strips allow it
-                const long long target = (long long)sms * std::max(occ, 1);
-                long long best = -1, best_cost = 0;
-                for (long long r = 1; r <= p.ny; ++r) {
-                    const long long rr = (p.ny + r - 1) / r;
-                    if (rr < 8 && r > 1) break;   // runs of at least 8 rows
-                    const long long runs = (p.ny + rr - 1) / rr;
-                    const long long waves = (strips * runs + target - 1) / target;
-                    const long long cost = waves * (rr + 3);
-                    if (best < 0 || cost < best_cost) { best = rr; best_cost = cost; }
-                }
-                rows = (int)best;
+                rows = march_rows(p.ny, strips, (long long)sms * std::max(occ, 1), nullptr);
             } else {
                 rows = batch_rows;
             }
@@ -607,6 +623,139 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
     return LBM_OK;
 }
 
+// The tile plan (step_kernel_tile, lbm_tile.cuh) of a context under
+// LBM_PIPELINE_AUTO with the built-in launch shape: every instance cut into tiles
+// of at most 128 units (cells; pairs of cells for the FP32-arithmetic forms when
+// every nx is even -- contexts that mix even and odd nx have none), all in one
+// cooperative launch for up to 256 steps. It serves the unmonitored steps; the
+// plan of row marches made beside it serves the monitored ones.
+//
+// Shape: the smallest of 8 x 4, 8 x 8 and 16 x 8 units whose items leave no SM
+// with two (the latency of a step falls with the tile: FP64 64 x 64 15.1 us with
+// 16 x 8, 12.3 with 8 x 4; LBM_F32_C 4.5 and 3.8); beyond that 16 x 8 or 8 x 16,
+// whichever needs fewer rounds of resident blocks.
+// Against the row marches (us a step, tile and march): a march takes about 22 us
+// (FP32) or 100 (FP64) whatever the size until its 8-row runs fill the GPU. FP32
+// pairs: 512 x 512 (2 rounds) 12.9 and 22.9, 130 x 2000 (2) 16.2 and 25.3, 512 x
+// 1024 (4) 26 and 27.5, 1024 x 1024 (7) 58 and 41: up to 3 rounds. One cell a
+// thread in FP32: 513 x 513 (3) 16.5 and 25.0, 517 x 1033 (6) 33 and 31: up to 4.
+// FP64 is bound by its arithmetic either way, so the tile wins by balance: 512 x
+// 512 158 and 188, 517 x 1033 (5 strips of 128 for 4.04) 318 and 410, 1024 x 1024
+// 609 and 607: taken while 1.2 x rounds x blocks stays below the march's waves x
+// (rows + 3) x blocks, both in units of 128 cells.
+lbm_status plan_tile(lbm_ctx* c, int sms) {
+    c->tile_items = 0;
+    if (c->d3 || c->pipeline != LBM_PIPELINE_AUTO || c->tile_req || c->rows_req) return LBM_OK;
+    const bool f64 = c->form == LBM_F64, pair = !f64 && c->params[0].nx % 2 == 0;
+    if (!f64)
+        for (const lbm_params& p : c->params)
+            if ((p.nx % 2 == 0) != pair) return LBM_OK;
+    const int cpt = pair ? 2 : 1;
+    auto count = [&](int u, int r) {
+        long long m = 0;
+        for (const lbm_params& p : c->params) m += (long long)((p.nx / cpt + u - 1) / u) * ((p.ny + r - 1) / r);
+        return m;
+    };
+    auto slots_at = [&](int occ) {
+        int n = 0;
+        by_form(c->form, [&](auto F) {
+            n = lbm::tile_occupancy_t<decltype(F)::value>(pair, occ);
+            return cudaSuccess;
+        });
+        return (long long)sms * n;
+    };
+    int U = 16, R = 8;
+    for (const auto& s : {std::pair<int, int>{8, 4}, {8, 8}, {16, 8}})
+        if (count(s.first, s.second) <= sms) {
+            U = s.first;
+            R = s.second;
+            break;
+        }
+    int occ = f64 ? 2 : pair ? 3 : 5;
+    long long slots = slots_at(occ);
+    if (pair && count(U, R) > slots) slots = slots_at(occ = 4);
+    if (slots <= 0) return LBM_OK;
+    auto rounds = [&](int u, int r) { return (count(u, r) + slots - 1) / slots; };
+    if (rounds(8, 16) < rounds(U, R)) {
+        U = 8;
+        R = 16;
+    }
+    if (!f64) {
+        if (rounds(U, R) > (pair ? 3 : 4)) return LBM_OK;
+    } else if (c->n == 1) {
+        const lbm_params& p = c->params[0];
+        const int tx = default_tile(p.nx);
+        const long long target = (long long)sms * std::max(1, lbm::step_occupancy_t<0>(tx, lbm::kPlain));
+        long long cost = 0;
+        march_rows(p.ny, (p.nx + tx - 1) / tx, target, &cost);
+        if (1.2 * rounds(U, R) * slots * 128 >= (double)cost * target * tx) return LBM_OK;
+    } else if (rounds(U, R) > 16) {
+        return LBM_OK;
+    }
+    int ulog = 0;
+    while ((1 << ulog) < U) ++ulog;
+    // each instance's columns (in units) and rows cut into equal parts, part i
+    // being [cut(i), cut(i + 1)): at least 2 wide and high, so that the items
+    // within the 3 cells a step reaches are at most two away
+    std::vector<WorkItem> items;
+    std::vector<int> nbr;
+    for (int k = 0; k < c->n; ++k) {
+        const lbm_params& p = c->params[k];
+        const int nu = p.nx / cpt, kx = (nu + U - 1) / U, ky = (p.ny + R - 1) / R;
+        auto xcut = [&](int i) { return (int)((long long)nu * i / kx) * cpt; };
+        auto ycut = [&](int i) { return (int)((long long)p.ny * i / ky); };
+        const int first = (int)items.size();
+        // parts within 3 cells of part i along one axis (itself among them)
+        auto near_parts = [](int m, int n, bool periodic, auto&& cut) {
+            std::vector<std::vector<int>> v(m);
+            for (int i = 0; i < m; ++i)
+                for (int j = i - 2; j <= i + 2; ++j) {
+                    if (!periodic && (j < 0 || j >= m)) continue;
+                    const int q = ((j % m) + m) % m, sh = (j - q) / m * n;   // part q, moved by whole periods
+                    if (cut(q) + sh >= cut(i + 1) + 3 || cut(i) - 3 >= cut(q + 1) + sh) continue;
+                    if (std::find(v[i].begin(), v[i].end(), q) == v[i].end()) v[i].push_back(q);
+                }
+            return v;
+        };
+        const auto nearx = near_parts(kx, p.nx, true, xcut);
+        const auto neary = near_parts(ky, p.ny, p.bc_y != LBM_BC_BOUNCEBACK, ycut);
+        for (int j = 0; j < ky; ++j)
+            for (int i = 0; i < kx; ++i) {
+                WorkItem w;
+                w.inst = k;
+                w.x0 = xcut(i);
+                w.dir = xcut(i + 1) - w.x0;   // columns
+                w.ystart = ycut(j);
+                w.nrows = ycut(j + 1) - w.ystart;
+                w.pad = 0;
+                items.push_back(w);
+                const size_t at = nbr.size();
+                for (int jj : neary[j])
+                    for (int ii : nearx[i])
+                        if (ii != i || jj != j) nbr.push_back(first + jj * kx + ii);
+                nbr.resize(at + lbm::kMaxTileNbr, -1);   // at most 5 x 5 - 1
+            }
+    }
+    const size_t wb = (items.size() * sizeof(WorkItem) + 255) & ~size_t(255);
+    const size_t nb = (nbr.size() * sizeof(int) + 255) & ~size_t(255);
+    const size_t db = (items.size() + 1) * sizeof(int);
+    cudaFree(c->d_tile);
+    c->d_tile = nullptr;
+    LBM_CK(c, cudaMalloc(&c->d_tile, wb + nb + db));
+    c->d_tile_work = static_cast<WorkItem*>(c->d_tile);
+    c->d_tile_nbr = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb);
+    c->d_tile_done = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb + nb);
+    LBM_CK(c, cudaMemcpy(c->d_tile_work, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
+    LBM_CK(c, cudaMemcpy(c->d_tile_nbr, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice));
+    LBM_CK(c, cudaMemset(c->d_tile_done, 0, db));
+    c->tile_items = (int)items.size();
+    c->tile_grid = (int)std::min<long long>(c->tile_items, slots);
+    c->tile_occ = occ;
+    c->tile_ulog = ulog;
+    c->tile_pair = pair;
+    return LBM_OK;
+}
+
 // Uploads the work list and sets up the monitor's per-instance item lists.
 lbm_status finish_plan(lbm_ctx* c) {
     if (c->graph) {
@@ -768,6 +917,7 @@ void release(lbm_ctx* c) {
     cudaFree(c->d_done);
     cudaFree(c->d_nbr);
     cudaFree(c->d_multi_done);
+    cudaFree(c->d_tile);
     cudaFree(c->d_mon_multi);
     cudaFree(c->d_mon_multi_cnt);
     cudaFree(c->d_mon_multi_sub);
@@ -1058,6 +1208,31 @@ cudaError_t enqueue_multi(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, in
     });
 }
 
+// Unmonitored steps run on the tile plan.
+bool tile_plan(const lbm_ctx* c) { return !c->d3 && c->tile_items > 0; }
+
+// Queues `nsteps` steps of a tile plan as one launch, the first reading buffer
+// set `in`, after zeroing the per-item step counters and the abort flag;
+// wait_extra / wait_limit as in StepArgs.
+cudaError_t enqueue_tile(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, int wait_limit = lbm::kWaitLimit) {
+    if (nsteps > 1) {
+        cudaError_t e = cudaMemsetAsync(c->d_tile_done, 0, ((size_t)c->tile_items + 1) * sizeof(int), c->stream);
+        if (e != cudaSuccess) return e;
+    }
+    StepArgs a = step_args(c, in);
+    a.work = c->d_tile_work;
+    a.nbr = c->d_tile_nbr;
+    a.done = c->d_tile_done;
+    a.ndesc = c->tile_items;
+    a.nsteps = nsteps;
+    a.wait_extra = wait_extra;
+    a.wait_limit = wait_limit;
+    a.tile_ulog = c->tile_ulog;
+    return by_form(c->form, [&](auto F) {
+        return lbm::launch_tile_t<decltype(F)::value>(c->tile_pair, c->tile_occ, a, c->tile_grid, c->stream);
+    });
+}
+
 // Kernel launches of one directly launched step of the plan.
 int step_kernels(const lbm_ctx* c) {
     if (c->d3) return d3_unfused(c) ? 3 * c->n : 1;
@@ -1170,6 +1345,14 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
     // with the monitor on, the last step runs the monitored kernels
     const bool mon_last = c->monitor && nsteps > 0;
     int left = mon_last ? nsteps - 1 : nsteps;
+    while (left > 0 && tile_plan(c)) {   // launches of up to 256 steps
+        const int n = std::min(left, 256);
+        cudaError_t e = enqueue_tile(c, c->cur, n);
+        if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
+        ++c->step_launches;
+        c->cur ^= n & 1;
+        left -= n;
+    }
     // graph replays cover whole multiples of the captured steps from parity 0
     if (left >= 2 && c->use_graphs) {
         if (c->cur == 1) {
@@ -1639,6 +1822,7 @@ std::string plan_signature(const lbm_ctx* c) {
         sig += std::to_string(L.tx) + ":" + std::to_string(L.count) + ":" + std::to_string(L.variant) + ";";
     for (const WorkItem& w : c->work) sig += std::to_string(w.nrows) + ",";
     if (c->multi) sig += "multi";
+    if (c->tile_items) sig += "tile";
     return sig;
 }
 }  // namespace
@@ -1850,9 +2034,12 @@ lbm_status lbm_inject_batched_wait_timeout(lbm_ctx* c, int rounds) {
     if (!batched_plan(c) && !multi_plan(c))
         return fail(c, LBM_ESTATE, "the context runs neither the batched nor the persistent launch");
     // two steps; every item of the second waits for one finished item (batched)
-    // or step (persistent) more than there are, so each of those waits runs out
-    // after `rounds` rounds
-    LBM_CK(c, batched_plan(c) ? enqueue_batched(c, c->cur, 2, 1, rounds) : enqueue_multi(c, c->cur, 2, 1, rounds));
+    // or step (persistent, and the tiles that stand in for the batched launch in
+    // small contexts) more than there are, so each of those waits runs out after
+    // `rounds` rounds
+    LBM_CK(c, tile_plan(c)      ? enqueue_tile(c, c->cur, 2, 1, rounds)
+              : batched_plan(c) ? enqueue_batched(c, c->cur, 2, 1, rounds)
+                                : enqueue_multi(c, c->cur, 2, 1, rounds));
     return LBM_OK;
 }
 

@@ -773,6 +773,68 @@ __device__ __forceinline__ void mon_step_store(const MonAcc<R>& acc, const StepA
 }
 
 // ---------------------------------------------------------------------------
+// Collision and push-streaming of cell X of the row at cell offset rY (rDn, rUp:
+// the rows below and above; bot, top: a wall there instead), from the 3x3
+// neighbourhoods of phi, mu and p, the cell's h (conservative forms: h[0] is the
+// low part of phi) and g, and phi u of the previous step. colm, colp: the columns
+// X - 1 and X + 1, wrapped.
+template <class F, bool MON, typename R, typename AT>
+__device__ __forceinline__ void collide_push(const Consts<R>& C, const PopIO<F>& io, AT* phiu, AT* p_out, int rY,
+                                             int rDn, int rUp, bool bot, bool top, int X, int colm, int colp,
+                                             const Nbr<R>& nphi, const Nbr<R>& nmu, const Nbr<R>& np,
+                                             const R (&h)[9], const R (&g)[9], R pux, R puy, MonAcc<R>& mon) {
+    const int c = rY + X;
+    const R phi = nphi.z[1][1], mu = nmu.z[1][1];
+    R gphix, gphiy, gmux, gmuy, gpx, gpy;
+    nphi.grad(gphix, gphiy);
+    nmu.grad(gmux, gmuy);
+    np.grad(gpx, gpy);
+    const R lapmu = nmu.lap();
+    const Macro<R> m = macroscopic(C, g, phi, mu, gphix, gphiy, gmux, gmuy, lapmu, gpx, gpy);
+    const R phiux = phi * m.ux, phiuy = phi * m.uy;
+    if constexpr (MON) mon.add(phi, F::cons ? h[0] : R(0), m.rho, m.ux, m.uy);
+    R gpost[9], hpost[9];
+    collide_cell(C, m, phi, mu, phiux - pux, phiuy - puy, g, h, gpost, hpost);
+
+    float2 h0c = make_float2(0.f, 0.f);
+    if constexpr (F::cons) {
+        // h_0 absorbs the storage rounding of h_1..h_8: the stored populations
+        // of this cell still sum to phi (collision conserves phi: sum h^eq = phi,
+        // sum R_i = 0), so rounding cannot change sum(phi).
+        R rest = R(0);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            hpost[i] = io.round_h(hpost[i]);
+            rest += hpost[i];
+        }
+        h0c = io.conservative_h0(phi, h[0] /* low part of phi */, rest);
+    }
+    // Push-streaming: population i moves to x + c_i; into a wall it comes back
+    // reversed at x (halfway bounce-back, Sec. 4.3). Wall rows are uniform per row.
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int cyi = cy_of(i), cxi = cx_of(i);
+        const int col = cxi < 0 ? colm : (cxi > 0 ? colp : X);
+        int dst = (cyi == 0 ? rY : (cyi > 0 ? rUp : rDn)) + col;
+        int k = i;
+        if ((cyi > 0 && top) || (cyi < 0 && bot)) {
+            dst = c;
+            k = opp_of(i);
+        }
+        if constexpr (F::cons) {
+            if (i == 0) io.store_h0(dst, h0c);
+            else io.store_h(k, dst, hpost[i]);
+        } else {
+            io.store_h(k, dst, hpost[i]);
+        }
+        io.store_g(k, dst, gpost[i]);
+    }
+    phiu[c] = AT(phiux);
+    phiu[io.S + c] = AT(phiuy);
+    p_out[c] = AT(m.p);
+}
+
+// ---------------------------------------------------------------------------
 // The fused step kernel. Rings in shared memory (slots by row number, powers of
 // two so a slot is one AND):
 //   phi   [8][TX+4]      rows Y-2 .. Y+2 (and the lead row being written)
@@ -985,7 +1047,6 @@ __global__ void __launch_bounds__(TX, StepOcc<FORM, TX>::value) step_kernel(cons
     auto collide_row = [&](int Y, const R (&g)[9], R pux, R puy) {
         if (!act) return;
         const int rY = rowoff(Y);
-        const int c = rY + X;
         Nbr<R> nphi, nmu, np;
 #pragma unroll
         for (int dy = 0; dy < 3; ++dy) {
@@ -999,12 +1060,6 @@ __global__ void __launch_bounds__(TX, StepOcc<FORM, TX>::value) step_kernel(cons
                 np.z[dy][dx] = qr[dx];
             }
         }
-        const R phi = nphi.z[1][1], mu = nmu.z[1][1];
-        R gphix, gphiy, gmux, gmuy, gpx, gpy;
-        nphi.grad(gphix, gphiy);
-        nmu.grad(gmux, gmuy);
-        np.grad(gpx, gpy);
-        const R lapmu = nmu.lap();
         R h[9];
         if constexpr (F::cons) {
             h[0] = hpair(Y)[tid + 2].y;        // low part of phi
@@ -1014,52 +1069,9 @@ __global__ void __launch_bounds__(TX, StepOcc<FORM, TX>::value) step_kernel(cons
 #pragma unroll
             for (int i = 0; i < 9; ++i) h[i] = hplane(Y, i)[tid + 2];
         }
-
-        const Macro<R> m = macroscopic(C, g, phi, mu, gphix, gphiy, gmux, gmuy, lapmu, gpx, gpy);
-        const R phiux = phi * m.ux, phiuy = phi * m.uy;
-        if constexpr (MON) mon.add(phi, F::cons ? h[0] : R(0), m.rho, m.ux, m.uy);
-        R gpost[9], hpost[9];
-        collide_cell(C, m, phi, mu, phiux - pux, phiuy - puy, g, h, gpost, hpost);
-
-        float2 h0c = make_float2(0.f, 0.f);
-        if constexpr (F::cons) {
-            // h_0 absorbs the storage rounding of h_1..h_8: the stored populations
-            // of this cell still sum to phi (collision conserves phi: sum h^eq = phi,
-            // sum R_i = 0), so rounding cannot change sum(phi).
-            R rest = R(0);
-#pragma unroll
-            for (int i = 1; i < 9; ++i) {
-                hpost[i] = io.round_h(hpost[i]);
-                rest += hpost[i];
-            }
-            h0c = io.conservative_h0(phi, h[0] /* low part of phi */, rest);
-        }
-        // Push-streaming: population i moves to x + c_i; into a wall it comes back
-        // reversed at x (halfway bounce-back, Sec. 4.3). Wall rows are uniform per row.
         const bool bot = walls && Y == 0, top = walls && Y == ny - 1;
-        const int rDn = bot ? 0 : rowoff(Y - 1);
-        const int rUp = top ? 0 : rowoff(Y + 1);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int cyi = cy_of(i), cxi = cx_of(i);
-            const int col = cxi < 0 ? colm : (cxi > 0 ? colp : X);
-            int dst = (cyi == 0 ? rY : (cyi > 0 ? rUp : rDn)) + col;
-            int k = i;
-            if ((cyi > 0 && top) || (cyi < 0 && bot)) {
-                dst = c;
-                k = opp_of(i);
-            }
-            if constexpr (F::cons) {
-                if (i == 0) io.store_h0(dst, h0c);
-                else io.store_h(k, dst, hpost[i]);
-            } else {
-                io.store_h(k, dst, hpost[i]);
-            }
-            io.store_g(k, dst, gpost[i]);
-        }
-        phiu[c] = AT(phiux);
-        phiu[S + c] = AT(phiuy);
-        p_out[c] = AT(m.p);
+        collide_push<F, MON>(C, io, phiu, p_out, rY, bot ? 0 : rowoff(Y - 1), top ? 0 : rowoff(Y + 1), bot, top, X,
+                             colm, colp, nphi, nmu, np, h, g, pux, puy, mon);
     };
 
     const int Y0 = wk.ystart;

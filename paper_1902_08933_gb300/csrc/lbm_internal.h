@@ -44,6 +44,9 @@ struct WorkItem {
 constexpr int kDescWide = -2;
 // the persistent multi-step plan (step_kernel_x2_multi): neighbour items an item
 constexpr int kMaxNbr = 8;
+// the tile plan (step_kernel_tile): items within 3 cells of an item, tiles of at
+// least 2 x 2 cells: at most two on either side
+constexpr int kMaxTileNbr = 24;
 struct BlockDesc {
     int item[2];
 };
@@ -93,6 +96,7 @@ struct StepArgs {
     int nsteps;
     int wait_limit;
     int wait_extra;
+    int tile_ulog;         // tile plan: log2 of the units (cells or pairs) of a tile's row
 };
 
 // Device layout of lbm_monitor (include/lbm.h; the host checks size and offsets).
@@ -148,6 +152,11 @@ template <int FORM> int batched_occupancy_t();             // resident blocks pe
 template <int FORM> cudaError_t launch_multi_t(int tile_x, const StepArgs& a, int nwork, cudaStream_t s,
                                                bool monitor);
 template <int FORM> int multi_occupancy_t(int tile_x);
+// several steps of a tile plan in one cooperative launch (pair: two cells a
+// thread; occ: the kernel compiled for that many resident blocks a SM), and its
+// residency (0: the form has no such kernel)
+template <int FORM> cudaError_t launch_tile_t(bool pair, int occ, const StepArgs& a, int grid, cudaStream_t s);
+template <int FORM> int tile_occupancy_t(bool pair, int occ);
 template <int FORM> int step_occupancy_t(int tile_x, int variant);   // resident blocks per SM
 template <int FORM> bool has_tma_t();                      // the form has a TMA-fed kernel
 template <int FORM> bool has_async_t();                    // the form has the cp.async kernel

@@ -6,6 +6,7 @@
 #include "lbm_device.cuh"
 #include "lbm_step_tma.cuh"
 #include "lbm_step_x2.cuh"
+#include "lbm_tile.cuh"
 
 namespace lbm {
 
@@ -222,6 +223,44 @@ int multi_occupancy_t(int tile_x) {
     return n;
 }
 
+// The tile plan's kernel of a form: two cells a thread (pair) at 3 or 4 resident
+// blocks a SM; one cell a thread at 5 (FP32) or 2 (FP64). Null if there is none.
+template <int FORM>
+static const void* tile_kernel(bool pair, int occ) {
+    if constexpr (kHasTma<FORM>) {
+        if (pair && occ == 3) return (const void*)step_kernel_tile<FORM, true, 3>;
+        if (pair && occ == 4) return (const void*)step_kernel_tile<FORM, true, 4>;
+    }
+    constexpr int one = kHasTma<FORM> ? 5 : 2;
+    return !pair && occ == one ? (const void*)step_kernel_tile<FORM, false, one> : nullptr;
+}
+
+// grid blocks (at most those resident, tile_occupancy_t) share a.ndesc items
+template <int FORM>
+cudaError_t launch_tile_t(bool pair, int occ, const StepArgs& a, int grid, cudaStream_t s) {
+    const void* k = tile_kernel<FORM>(pair, occ);
+    if (!k || grid <= 0 || a.done == nullptr || a.nbr == nullptr) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kTileThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = a.nsteps > 1 ? 1 : 0;   // one step: no block waits
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[1] = {const_cast<StepArgs*>(&a)};
+    return cudaLaunchKernelExC(&cfg, k, args);
+}
+
+template <int FORM>
+int tile_occupancy_t(bool pair, int occ) {
+    const void* k = tile_kernel<FORM>(pair, occ);
+    int n = 0;
+    if (!k || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kTileThreads, 0) != cudaSuccess) return 0;
+    return n;
+}
+
 template <int FORM>
 size_t step_smem_t(int tile_x) {
     switch (tile_x) {
@@ -322,6 +361,8 @@ cudaError_t launch_populations_t(const AuxArgs& a, int ncells, double* out_h, do
     template int batched_occupancy_t<F>();                                                    \
     template cudaError_t launch_multi_t<F>(int, const StepArgs&, int, cudaStream_t, bool);    \
     template int multi_occupancy_t<F>(int);                                                   \
+    template cudaError_t launch_tile_t<F>(bool, int, const StepArgs&, int, cudaStream_t);     \
+    template int tile_occupancy_t<F>(bool, int);                                              \
     template int step_occupancy_t<F>(int, int);                                               \
     template bool has_tma_t<F>();                                                             \
     template bool has_async_t<F>();                                                           \

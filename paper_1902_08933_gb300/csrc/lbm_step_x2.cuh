@@ -78,6 +78,127 @@ struct X2Occ {
     static constexpr int value = by_smem < 1 ? 1 : (by_smem < by_regs ? by_smem : by_regs);
 };
 
+// 3x3 neighbourhoods of the pair at shared-memory index j (cells j, j+1) from three rows
+__device__ __forceinline__ void nbr_pair(const float* r0, const float* r1, const float* r2, int j, Nbr<F2>& n) {
+    const float* rows[3] = {r0, r1, r2};
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy) {
+        const float2 a2 = *reinterpret_cast<const float2*>(rows[dy] + j - 2);
+        const float2 b2 = *reinterpret_cast<const float2*>(rows[dy] + j);
+        const float2 c2 = *reinterpret_cast<const float2*>(rows[dy] + j + 2);
+        n.z[dy][0] = F2(a2.y, b2.x);
+        n.z[dy][1] = F2(b2);
+        n.z[dy][2] = F2(b2.y, c2.x);
+    }
+}
+
+// The arrays a step writes.
+template <int FORM>
+struct X2Out {
+    typename Form<FORM>::HT* h;
+    float2* h0;
+    typename Form<FORM>::GT* g;
+    float *phiu, *p;
+    long long S;
+};
+
+// Collision and push-streaming of the pair (X, X + 1) of row Y. rowoff(y): the
+// cell offset of row y (wrapped where periodic); load_nbr(nphi, nmu, np): the 3x3
+// neighbourhoods of phi, mu and p; load_h(h, lo): the stored h (conservative
+// forms: h_1..h_8, and lo, the low parts of phi); g and phi u of the previous
+// step; colm, colp: the columns X - 1 and X + 2, wrapped. (The loads are passed as
+// functions so that each is made where its values are first needed: made ahead of
+// the stencils they cost the march kernel 2 to 4 % of its time.)
+template <int FORM, int MON, typename RowOff, typename LoadNbr, typename LoadH>
+__device__ __forceinline__ void x2_collide_push(const Consts<float>& C, const X2Out<FORM>& out, int Y, int X,
+                                                int colm, int colp, RowOff&& rowoff, LoadNbr&& load_nbr,
+                                                LoadH&& load_h, const F2 (&g)[9], F2 pu_x, F2 pu_y,
+                                                MonAcc<F2>& mon) {
+    using F = Form<FORM>;
+    const long long S = out.S;
+    const int ny = C.ny, walls = C.walls;
+    const int rY = rowoff(Y);
+    const int c = rY + X;
+    // output planes: h_k (k >= 1 for conservative forms), g_k
+    auto hplane_out = [&](int k) { return out.h + (long long)(F::cons ? k - 1 : k) * S; };
+    auto gplane_out = [&](int k) { return out.g + (long long)k * S; };
+    Nbr<F2> nphi, nmu, np;
+    load_nbr(nphi, nmu, np);
+    const F2 phi = nphi.z[1][1], mu = nmu.z[1][1];
+    F2 gphix, gphiy, gmux, gmuy, gpx, gpy;
+    nphi.grad(gphix, gphiy);
+    nmu.grad(gmux, gmuy);
+    np.grad(gpx, gpy);
+    const F2 lapmu = nmu.lap();
+    F2 h[9];
+    F2 lo = F2(0.f);
+    load_h(h, lo);
+    const Macro<F2> m = macroscopic<F::g16>(C, g, phi, mu, gphix, gphiy, gmux, gmuy, lapmu, gpx, gpy);
+    const F2 phiux = phi * m.ux, phiuy = phi * m.uy;
+    if constexpr (MON) {
+        mon.add(phi, lo, m.rho, m.ux, m.uy);
+    }
+    // Push-streaming as each result is formed (halfway bounce-back into walls;
+    // wall rows uniform per row). Conservative forms: h_0 goes last, as phi
+    // minus the stored h_1..h_8 (per cell, as in step_kernel).
+    const bool bot = walls && Y == 0, top = walls && Y == ny - 1;
+    const int rDn = bot ? 0 : rowoff(Y - 1);
+    const int rUp = top ? 0 : rowoff(Y + 1);
+    // sums of the stored h_1..h_8 of the two cells (FP16 h: in units of hs)
+    float ra = 0.f, rb = 0.f;
+    collide_emit<F::g16, F::h16>(C, m, phi, mu, phiux - pu_x, phiuy - pu_y, g, h, [&](int i, F2 gi, F2 hi) {
+        const auto gq = to_store(gi, out.g);
+        if constexpr (F::cons) {
+            if (i == 0) {          // rest direction: g_0 now, h_0 after all h_1..h_8
+                st_both(gplane_out(0) + c, gq);
+                return;
+            }
+        }
+        const auto hq = to_store(hi, out.h);
+        if constexpr (F::cons) {
+            ra += first_f(hq);
+            rb += second_f(hq);
+        }
+        const int cyi = cy_of(i), cxi = cx_of(i);
+        if ((cyi > 0 && top) || (cyi < 0 && bot)) {   // back into the own pair, reversed
+            const int k = opp_of(i);
+            st_both(hplane_out(k) + c, hq);
+            st_both(gplane_out(k) + c, gq);
+            return;
+        }
+        const int r = cyi == 0 ? rY : (cyi > 0 ? rUp : rDn);
+        if (cxi == 0) {
+            if (!F::cons || i != 0) st_both(hplane_out(i) + r + X, hq);
+            st_both(gplane_out(i) + r + X, gq);
+        } else {
+            const int da = r + (cxi > 0 ? X + 1 : colm);   // destination of cell X
+            const int db = r + (cxi > 0 ? colp : X);       // destination of cell X + 1
+            st_first(hplane_out(i) + da, hq);
+            st_second(hplane_out(i) + db, hq);
+            st_first(gplane_out(i) + da, gq);
+            st_second(gplane_out(i) + db, gq);
+        }
+    });
+    if constexpr (F::h16) {   // exact: the inverse scale is a power of two
+        ra *= C.ihs;
+        rb *= C.ihs;
+    }
+    if constexpr (F::cons) {
+        float s_, e_, hi, l2;
+        float4 h0c;
+        two_sum(phi.v.x, -ra, s_, e_);
+        fast_two_sum(s_, e_ + lo.v.x, hi, l2);
+        h0c.x = hi; h0c.y = l2;
+        two_sum(phi.v.y, -rb, s_, e_);
+        fast_two_sum(s_, e_ + lo.v.y, hi, l2);
+        h0c.z = hi; h0c.w = l2;
+        *reinterpret_cast<float4*>(out.h0 + c) = h0c;
+    }
+    st_pair(out.phiu + c, phiux);
+    st_pair(out.phiu + S + c, phiuy);
+    st_pair(out.p + c, m.p);
+}
+
 // One work item (a strip of 2 TX columns of one instance, a run of rows) marched
 // by a group of TX threads (32, 64 or 128): a whole thread block (step_kernel_x2:
 // barrier 0, the one __syncthreads uses; TX its compile-time block size, so the
@@ -150,10 +271,6 @@ __device__ __forceinline__ void x2_item(const StepArgs& a, int item, unsigned ch
     auto hpairs = [&](int y) { return reinterpret_cast<float2*>(hslot(y)); };   // conservative h_0
     // population i of the cell pair at c as stored (FP16: still scaled by gs)
     auto ld_g = [&](int i, int c) -> F2 { return ld_pair(gin + (long long)i * S + c); };
-    // output planes: h_k (k >= 1 for conservative forms), g_k
-    auto hplane_out = [&](int k) { return hout + (long long)(F::cons ? k - 1 : k) * S; };
-    auto gplane_out = [&](int k) { return gout + (long long)k * S; };
-
     // Column pairs of the lead / p rows: pair q covers x0-2+2q, x0-1+2q (ring index 2+2q).
     const int nq = (w + 4) >> 1;
     const bool q0 = tid < nq, q1 = tid + TX < nq;
@@ -276,19 +393,6 @@ __device__ __forceinline__ void x2_item(const StepArgs& a, int item, unsigned ch
         if (q0) st_pair(dst + 2 + 2 * tid, ld_pair(src + qc0));
         if (q1) st_pair(dst + 2 + 2 * (tid + TX), ld_pair(src + qc1));
     };
-    // 3x3 neighbourhoods of the pair at ring index j (cells j, j+1) from three rows
-    auto nbr_pair = [&](const float* r0, const float* r1, const float* r2, int j, Nbr<F2>& n) {
-        const float* rows[3] = {r0, r1, r2};
-#pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-            const float2 a2 = *reinterpret_cast<const float2*>(rows[dy] + j - 2);
-            const float2 b2 = *reinterpret_cast<const float2*>(rows[dy] + j);
-            const float2 c2 = *reinterpret_cast<const float2*>(rows[dy] + j + 2);
-            n.z[dy][0] = F2(a2.y, b2.x);
-            n.z[dy][1] = F2(b2);
-            n.z[dy][2] = F2(b2.y, c2.x);
-        }
-    };
     // 3x3 neighbourhood of the low parts of phi around the pair at ring index j
     // of row M, from the h_0 pair slots of rows M - 1, M, M + 1 (all three are in
     // the slot window when mu of M is formed; a ghost row beyond a wall is its
@@ -334,92 +438,22 @@ __device__ __forceinline__ void x2_item(const StepArgs& a, int item, unsigned ch
     // C. collision and push-streaming of the pair in row Y.
     auto collide_row = [&](int Y, const F2 (&g)[9], F2 pu_x, F2 pu_y) {
         if (!act) return;
-        const int rY = rowoff(Y);
-        const int c = rY + X;
-        Nbr<F2> nphi, nmu, np;
-        nbr_pair(prow(Y - 1), prow(Y), prow(Y + 1), jX, nphi);
-        nbr_pair(mrow(Y - 1), mrow(Y), mrow(Y + 1), jX, nmu);
-        nbr_pair(qrow(Y - 1), qrow(Y), qrow(Y + 1), jX, np);
-        const F2 phi = nphi.z[1][1], mu = nmu.z[1][1];
-        F2 gphix, gphiy, gmux, gmuy, gpx, gpy;
-        nphi.grad(gphix, gphiy);
-        nmu.grad(gmux, gmuy);
-        np.grad(gpx, gpy);
-        const F2 lapmu = nmu.lap();
-        F2 h[9];
-        F2 lo = F2(0.f);
-        if constexpr (F::cons) {
-            const float4 l4 = *reinterpret_cast<const float4*>(&hpairs(Y)[jX]);
-            lo = F2(l4.y, l4.w);
-            h[0] = lo;   // (not stored: the conservative h_0 is formed after the collision)
-        }
+        auto load_nbr = [&](Nbr<F2>& nphi, Nbr<F2>& nmu, Nbr<F2>& np) {
+            nbr_pair(prow(Y - 1), prow(Y), prow(Y + 1), jX, nphi);
+            nbr_pair(mrow(Y - 1), mrow(Y), mrow(Y + 1), jX, nmu);
+            nbr_pair(qrow(Y - 1), qrow(Y), qrow(Y + 1), jX, np);
+        };
+        auto load_h = [&](F2 (&h)[9], F2& lo) {
+            if constexpr (F::cons) {
+                const float4 l4 = *reinterpret_cast<const float4*>(&hpairs(Y)[jX]);
+                lo = F2(l4.y, l4.w);
+                h[0] = lo;   // (not stored: the conservative h_0 is formed after the collision)
+            }
 #pragma unroll
-        for (int i = F::cons ? 1 : 0; i < 9; ++i) h[i] = ld_pair(hplane(Y, i) + jX);   // as stored
-
-        const Macro<F2> m = macroscopic<F::g16>(C, g, phi, mu, gphix, gphiy, gmux, gmuy, lapmu, gpx, gpy);
-        const F2 phiux = phi * m.ux, phiuy = phi * m.uy;
-        if constexpr (MON) {
-            mon.add(phi, lo, m.rho, m.ux, m.uy);
-        }
-        // Push-streaming as each result is formed (halfway bounce-back into walls;
-        // wall rows uniform per row). Conservative forms: h_0 goes last, as phi
-        // minus the stored h_1..h_8 (per cell, as in step_kernel).
-        const bool bot = walls && Y == 0, top = walls && Y == ny - 1;
-        const int rDn = bot ? 0 : rowoff(Y - 1);
-        const int rUp = top ? 0 : rowoff(Y + 1);
-        // sums of the stored h_1..h_8 of the two cells (FP16 h: in units of hs)
-        float ra = 0.f, rb = 0.f;
-        collide_emit<F::g16, F::h16>(C, m, phi, mu, phiux - pu_x, phiuy - pu_y, g, h, [&](int i, F2 gi, F2 hi) {
-            const auto gq = to_store(gi, gout);
-            if constexpr (F::cons) {
-                if (i == 0) {          // rest direction: g_0 now, h_0 after all h_1..h_8
-                    st_both(gplane_out(0) + c, gq);
-                    return;
-                }
-            }
-            const auto hq = to_store(hi, hout);
-            if constexpr (F::cons) {
-                ra += first_f(hq);
-                rb += second_f(hq);
-            }
-            const int cyi = cy_of(i), cxi = cx_of(i);
-            if ((cyi > 0 && top) || (cyi < 0 && bot)) {   // back into the own pair, reversed
-                const int k = opp_of(i);
-                st_both(hplane_out(k) + c, hq);
-                st_both(gplane_out(k) + c, gq);
-                return;
-            }
-            const int r = cyi == 0 ? rY : (cyi > 0 ? rUp : rDn);
-            if (cxi == 0) {
-                if (!F::cons || i != 0) st_both(hplane_out(i) + r + X, hq);
-                st_both(gplane_out(i) + r + X, gq);
-            } else {
-                const int da = r + (cxi > 0 ? X + 1 : colm);   // destination of cell X
-                const int db = r + (cxi > 0 ? colp : X);       // destination of cell X + 1
-                st_first(hplane_out(i) + da, hq);
-                st_second(hplane_out(i) + db, hq);
-                st_first(gplane_out(i) + da, gq);
-                st_second(gplane_out(i) + db, gq);
-            }
-        });
-        if constexpr (F::h16) {   // exact: ihs is a power of two
-            ra *= ihs;
-            rb *= ihs;
-        }
-        if constexpr (F::cons) {
-            float s_, e_, hi, l2;
-            float4 h0c;
-            two_sum(phi.v.x, -ra, s_, e_);
-            fast_two_sum(s_, e_ + lo.v.x, hi, l2);
-            h0c.x = hi; h0c.y = l2;
-            two_sum(phi.v.y, -rb, s_, e_);
-            fast_two_sum(s_, e_ + lo.v.y, hi, l2);
-            h0c.z = hi; h0c.w = l2;
-            *reinterpret_cast<float4*>(h0out + c) = h0c;
-        }
-        st_pair(phiu + c, phiux);
-        st_pair(phiu + S + c, phiuy);
-        st_pair(p_out + c, m.p);
+            for (int i = F::cons ? 1 : 0; i < 9; ++i) h[i] = ld_pair(hplane(Y, i) + jX);   // as stored
+        };
+        const X2Out<FORM> out{hout, h0out, gout, phiu, p_out, S};
+        x2_collide_push<FORM, MON>(C, out, Y, X, colm, colp, rowoff, load_nbr, load_h, g, pu_x, pu_y, mon);
     };
 
     const int Y0 = wk.ystart;
