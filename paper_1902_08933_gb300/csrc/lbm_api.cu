@@ -112,6 +112,10 @@ DevInst derive(const lbm_params& p, long long base, int form) {
     d.eta = p.mobility / ((1.0 / 3.0) * (p.tau_h - 0.5));   // Eq. 17
     const double gamma = (p.rho_A - p.rho_B) / (phiA * p.rho_B - phiB * p.rho_A);
     d.gammaM = gamma * p.mobility;
+    d.beta4 = 4.0 * d.beta;
+    d.kappa6 = d.kappa / 6.0;
+    d.gammaM6 = d.gammaM / 6.0;
+    d.drho12 = d.drho / 12.0;
     d.inv_tau_h = 1.0 / p.tau_h;
     d.force_x = p.force_x;
     d.force_y = p.force_y;
@@ -631,17 +635,17 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
 // plan of row marches made beside it serves the monitored ones.
 //
 // Shape: the smallest of 8 x 4, 8 x 8 and 16 x 8 units whose items leave no SM
-// with two (the latency of a step falls with the tile: FP64 64 x 64 15.1 us with
-// 16 x 8, 12.3 with 8 x 4; LBM_F32_C 4.5 and 3.8); beyond that 16 x 8 or 8 x 16,
+// with two (the latency of a step falls with the tile: FP64 64 x 64 12.7 us with
+// 16 x 8, 10.3 with 8 x 4; LBM_F32_C 4.5 and 3.8); beyond that 16 x 8 or 8 x 16,
 // whichever needs fewer rounds of resident blocks.
 // Against the row marches (us a step, tile and march): a march takes about 22 us
-// (FP32) or 100 (FP64) whatever the size until its 8-row runs fill the GPU. FP32
+// (FP32) or 82 (FP64) whatever the size until its 8-row runs fill the GPU. FP32
 // pairs: 512 x 512 (2 rounds) 12.9 and 22.9, 130 x 2000 (2) 16.2 and 25.3, 512 x
 // 1024 (4) 26 and 27.5, 1024 x 1024 (7) 58 and 41: up to 3 rounds. One cell a
 // thread in FP32: 513 x 513 (3) 16.5 and 25.0, 517 x 1033 (6) 33 and 31: up to 4.
 // FP64 is bound by its arithmetic either way, so the tile wins by balance: 512 x
-// 512 158 and 188, 517 x 1033 (5 strips of 128 for 4.04) 318 and 410, 1024 x 1024
-// 609 and 607: taken while 1.2 x rounds x blocks stays below the march's waves x
+// 512 121 and 146, 517 x 1033 (5 strips of 128 for 4.04) 248 and 308, 1024 x 1024
+// 471 and 456: taken while 1.2 x rounds x blocks stays below the march's waves x
 // (rows + 3) x blocks, both in units of 128 cells.
 lbm_status plan_tile(lbm_ctx* c, int sms) {
     c->tile_items = 0;

@@ -28,6 +28,7 @@ struct DevInst {
     double force_x, force_y, gravity;
     double h_scale, g_scale;         // storage scales of reduced-precision forms (powers of 2)
     double tgm0, inv_tau_g0;         // tau_g - 1/2 and 1/tau_g for uniform_nu
+    double beta4, kappa6, gammaM6, drho12;   // 4 beta, kappa / 6, gammaM / 6, drho / 12
 };
 
 // One thread block's work: a strip of columns [x0, x0 + TX) (clipped to nx) of

@@ -274,7 +274,8 @@ __device__ __forceinline__ void tile_item_1(const StepArgs& a, const Consts<type
         const int cr = walls ? rowg(y0 + ry) - y0 : ry;   // a ghost row's mu is its mirror row's
         Nbr<R> n;
         nbr(sm.phi, (cr + 2) * RW + rx + 4, n);
-        sm.mu[(ry + 2) * RW + rx + 4] = chem_pot(C, n.z[1][1], n.lap());
+        if constexpr (sizeof(R) == 8) sm.mu[(ry + 2) * RW + rx + 4] = chem_pot_f64(C, n);
+        else sm.mu[(ry + 2) * RW + rx + 4] = chem_pot(C, n.z[1][1], n.lap());
     };
     if (act) mu_at(ty, tx);
     for (int k = h0; k < H.count(1); k += kTileThreads) {
@@ -301,7 +302,7 @@ __device__ __forceinline__ void tile_item_1(const StepArgs& a, const Consts<type
 // a tile's loads in flight) while every item then has a block of its own, else 4
 // (128 registers, no spills). Measured, LBM_F32_C, us a step: 64 x 64 3.8 with 3
 // and 4.2 with 4; 512 x 512 (1024 items) 15.7 with 3, 12.9 with 4, 18.5 with 5.
-// FP64 runs 2 (255 registers): 512 x 512 158 us against 172 with 3.
+// FP64 runs 2 (255 registers): 512 x 512 121 us against 130 with 3, 139 with 4.
 template <int FORM, bool PAIR, int OCC>
 __global__ void __launch_bounds__(kTileThreads, OCC) step_kernel_tile(const StepArgs a) {
     using R = typename Form<FORM>::R;
