@@ -507,17 +507,19 @@ void lbm_destroy(lbm_ctx* ctx);
  * bounce-back walls). Equilibrium of Remark 3 (g_0 stored shifted by rho_0),
  * force term w_i{S + c.F/c_s^2 + (cc - c_s^2 I):(uF + Fu + Q S I)/(2 c_s^4)}
  * with Q = (2/d) c_s^2 - xi/(tau_g - 1/2), u by Eq. 27a (rho = 1), p by Eq. 28,
- * BGK of Eq. 24 with tau_g = nu / c_s^2 + 1/2. One kernel a step.
+ * BGK of Eq. 24 with tau_g = nu / c_s^2 + 1/2.
  * model LBM_SP_NEARLY_INCOMPRESSIBLE is Remark 1 instead (rho~ = rho,
  * p = rho c_s^2): rho = sum g + S/2 (Eq. 27aa), u = (sum c g + F/2)/rho,
  * g^eq = rho (w_i + s_i(u)) (Eq. 29bb), force term with uF + Fu - uuS + Q div(u) I,
  * Q = (2/d) rho c_s^2 - xi/(tau_g - 1/2), div u by Eq. 30a (mirror at walls);
- * the total mass grows by sum S a step. Two kernels a step.
+ * the total mass grows by sum S a step.
  * model LBM_SP_HE_INCOMPRESSIBLE is Remark 2: g in units of pressure,
  * g^eq = w_i p + p_0 s_i(u) (Eq. 29bd), p = sum g + p_0 S_1/2, p_0 u = sum c g +
  * p_0 F_1/2, G_i with p_0 S_1, p_0 F_1 and ((2/d) p_0 c_s^2 - xi/(tau_g - 1/2))
  * div u (as printed); the source field is S_1, (force_x, force_y) is F_1, p0 > 0.
- * Two kernels a step, like Remark 1. */
+ * One kernel a step; domains whose tiles fit on the GPU at once run up to 256
+ * steps in one cooperative launch with bounded waits between tiles: one that ran
+ * out makes the read-backs return LBM_ETIMEOUT until lbm_sp_init. */
 enum { LBM_SP_INCOMPRESSIBLE_SOURCE = 0, LBM_SP_NEARLY_INCOMPRESSIBLE = 1, LBM_SP_HE_INCOMPRESSIBLE = 2 };
 /* scheme LBM_SP_SCHEME_REMARK4 (with model LBM_SP_INCOMPRESSIBLE_SOURCE only)
  * evolves the Remark 3 model with the explicit discretization of D_i G_i of
@@ -528,8 +530,7 @@ enum { LBM_SP_INCOMPRESSIBLE_SOURCE = 0, LBM_SP_NEARLY_INCOMPRESSIBLE = 1, LBM_S
  * u = sum c f (explicit), p = c_s^2/(1 - w_0) [sum_{i != 0} f_i + s_0(u) +
  * tau_g G_0]. G_i(x + c_i, t) across a wall is taken at the mirrored cell;
  * bounce-back acts on f - G/2; G at t = -1 is G at t = 0. G at t - 1 is
- * recomputed from u and F(u) at t - 1 (kept, four planes) and S. Two kernels
- * a step.
+ * recomputed from u at t - 1 (kept, two planes) and S.
  * The scheme of Eq. 24 (LBM_SP_SCHEME_EQ24) needs drag_lin = drag_quad = 0. */
 enum { LBM_SP_SCHEME_EQ24 = 0, LBM_SP_SCHEME_REMARK4 = 1 };
 typedef struct lbm_sp_params {

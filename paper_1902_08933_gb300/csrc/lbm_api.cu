@@ -13,6 +13,7 @@
 #include "lbm.h"
 #include "lbm_internal.h"
 #include "lbm_mbar.cuh"
+#include "lbm_tileplan.h"
 
 using lbm::AuxArgs;
 using lbm::DevInst;
@@ -668,13 +669,8 @@ lbm_status plan_tile(lbm_ctx* c, int sms) {
         });
         return (long long)sms * n;
     };
-    int U = 16, R = 8;
-    for (const auto& s : {std::pair<int, int>{8, 4}, {8, 8}, {16, 8}})
-        if (count(s.first, s.second) <= sms) {
-            U = s.first;
-            R = s.second;
-            break;
-        }
+    int U, R;
+    lbm::tile_shape(count, sms, &U, &R);
     int occ = f64 ? 2 : pair ? 3 : 5;
     long long slots = slots_at(occ);
     if (pair && count(U, R) > slots) slots = slots_at(occ = 4);
@@ -698,48 +694,13 @@ lbm_status plan_tile(lbm_ctx* c, int sms) {
     }
     int ulog = 0;
     while ((1 << ulog) < U) ++ulog;
-    // each instance's columns (in units) and rows cut into equal parts, part i
-    // being [cut(i), cut(i + 1)): at least 2 wide and high, so that the items
-    // within the 3 cells a step reaches are at most two away
-    std::vector<WorkItem> items;
-    std::vector<int> nbr;
+    lbm::TileList list;
     for (int k = 0; k < c->n; ++k) {
         const lbm_params& p = c->params[k];
-        const int nu = p.nx / cpt, kx = (nu + U - 1) / U, ky = (p.ny + R - 1) / R;
-        auto xcut = [&](int i) { return (int)((long long)nu * i / kx) * cpt; };
-        auto ycut = [&](int i) { return (int)((long long)p.ny * i / ky); };
-        const int first = (int)items.size();
-        // parts within 3 cells of part i along one axis (itself among them)
-        auto near_parts = [](int m, int n, bool periodic, auto&& cut) {
-            std::vector<std::vector<int>> v(m);
-            for (int i = 0; i < m; ++i)
-                for (int j = i - 2; j <= i + 2; ++j) {
-                    if (!periodic && (j < 0 || j >= m)) continue;
-                    const int q = ((j % m) + m) % m, sh = (j - q) / m * n;   // part q, moved by whole periods
-                    if (cut(q) + sh >= cut(i + 1) + 3 || cut(i) - 3 >= cut(q + 1) + sh) continue;
-                    if (std::find(v[i].begin(), v[i].end(), q) == v[i].end()) v[i].push_back(q);
-                }
-            return v;
-        };
-        const auto nearx = near_parts(kx, p.nx, true, xcut);
-        const auto neary = near_parts(ky, p.ny, p.bc_y != LBM_BC_BOUNCEBACK, ycut);
-        for (int j = 0; j < ky; ++j)
-            for (int i = 0; i < kx; ++i) {
-                WorkItem w;
-                w.inst = k;
-                w.x0 = xcut(i);
-                w.dir = xcut(i + 1) - w.x0;   // columns
-                w.ystart = ycut(j);
-                w.nrows = ycut(j + 1) - w.ystart;
-                w.pad = 0;
-                items.push_back(w);
-                const size_t at = nbr.size();
-                for (int jj : neary[j])
-                    for (int ii : nearx[i])
-                        if (ii != i || jj != j) nbr.push_back(first + jj * kx + ii);
-                nbr.resize(at + lbm::kMaxTileNbr, -1);   // at most 5 x 5 - 1
-            }
+        lbm::add_tiles(list, k, p.nx, p.ny, cpt, p.bc_y != LBM_BC_BOUNCEBACK, U, R);
     }
+    const std::vector<WorkItem>& items = list.items;
+    const std::vector<int>& nbr = list.nbr;
     const size_t wb = (items.size() * sizeof(WorkItem) + 255) & ~size_t(255);
     const size_t nb = (nbr.size() * sizeof(int) + 255) & ~size_t(255);
     const size_t db = (items.size() + 1) * sizeof(int);

@@ -740,6 +740,49 @@ __device__ __forceinline__ int atom_add_acq_rel_gpu(int* p, int v) {
     return old;
 }
 
+__device__ __forceinline__ int ld_acquire_gpu(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Before step s > 0 of an item of a tile plan: waits (bounded: wait_limit rounds)
+// until its neighbour items (nbr, kMaxTileNbr of them, -1 padded) have finished
+// step `need` - 1, counted in done. A wait that runs out records a timeout in
+// *status and raises *abort_flag, which ends the others' waits; returns false to
+// every thread of the block then. s_bad: a shared word.
+__device__ __forceinline__ bool tile_wait(const int* done, const int* nbr, int need, int wait_limit, int* status,
+                                          int* abort_flag, int* s_bad, int tid) {
+    if (tid < 32) {
+        int ok = 1;
+        const int n = tid < kMaxTileNbr ? nbr[tid] : -1;
+        if (n >= 0) {
+            ok = 0;
+            for (int it = 0; it < wait_limit; ++it) {
+                if (ld_acquire_gpu(done + n) >= need) {
+                    ok = 1;
+                    break;
+                }
+                if (it >= 256) {   // neighbours are within a step of each other: rarely
+                    if (*reinterpret_cast<volatile int*>(abort_flag)) break;
+                    __nanosleep(64);
+                }
+            }
+            __threadfence();
+        }
+        const unsigned bad = __ballot_sync(0xffffffffu, !ok);
+        if (tid == 0) {
+            if (bad) {
+                atomicExch(status, kStatusTimeout);
+                atomicExch(abort_flag, 1);
+            }
+            *s_bad = bad != 0;
+        }
+    }
+    __syncthreads();
+    return *s_bad == 0;
+}
+
 template <typename R>
 __device__ __forceinline__ void mon_block_store(const MonAcc<R>& acc, const StepArgs& a, int inst, int item,
                                                 int pos, int tid, int nthr, int bar, int grp) {

@@ -4,10 +4,9 @@
 //
 // Remark 3 (model LBM_SP_INCOMPRESSIBLE_SOURCE): rho~ = rho_0 and a constant
 // density (rho = 1), the incompressible Navier-Stokes equations with a mass
-// source (div u = S) and a uniform body force. One kernel a step: the cell's
-// populations and source give u (Eq. 27a) and p (Eq. 28 with G_0), the
-// equilibrium (Eq. 25 with rho~ = rho_0, rho = 1; g_0 stored shifted by rho_0)
-// and the force term
+// source (div u = S) and a uniform body force: the cell's populations and source
+// give u (Eq. 27a) and p (Eq. 28 with G_0), the equilibrium (Eq. 25 with rho~ =
+// rho_0, rho = 1; g_0 stored shifted by rho_0) and the force term
 //   G_i = w_i { S + c_i.F / c_s^2 + (c_i c_i - c_s^2 I):(u F + F u + Q S I) / (2 c_s^4) },
 //   Q = (2/d) c_s^2 - xi / (tau_g - 1/2),
 // then BGK (Eq. 24) and push-streaming (x periodic; y periodic or halfway
@@ -16,61 +15,35 @@
 // Remark 1 (LBM_SP_NEARLY_INCOMPRESSIBLE; rho~ = rho, p = rho c_s^2): rho =
 // sum g + S/2 (Eq. 27aa), u = (sum c g + F/2) / rho, g^eq = rho (w_i + s_i(u))
 // (Eq. 29bb), G_i with (u F + F u - u u S + Q div(u) I) and Q = (2/d) rho c_s^2 -
-// xi / (tau_g - 1/2); div u by Eq. 30a from a plane of u (mirror at walls), so
-// a step is two kernels (rho and u, then the collision). The populations are
+// xi / (tau_g - 1/2); div u by Eq. 30a (mirror at walls). The populations are
 // stored as g_i - w_i (their rest state at rho = 1), so that FP32 storage keeps
 // the small deviations that carry the flow: rho = 1 + sum(g - w) + S/2.
 //
-// Remark 2 (LBM_SP_HE_INCOMPRESSIBLE): the same two kernels with g in units of
-// pressure (g^eq = w_i p + p_0 s_i(u), Eq. 29bd; p_0 S_1 and p_0 F_1), stored as
-// g_i - w_i p_0.
+// Remark 2 (LBM_SP_HE_INCOMPRESSIBLE): the same with g in units of pressure (g^eq
+// = w_i p + p_0 s_i(u), Eq. 29bd; p_0 S_1 and p_0 F_1), stored as g_i - w_i p_0.
 //
 // Remark 4 (scheme LBM_SP_SCHEME_REMARK4): the Remark 3 model with a
 // velocity-dependent force F(u) = F_0 - (lambda + beta |u|) u, evolved with the
-// explicit D_i G_i (unshifted f, u = sum c f). A first kernel writes u and
-// F(u); the second rebuilds G_i at the destination x + c_i from its u, F(u) and
-// S, and G_i(x, t - 1) from u and F at t - 1 (four planes kept instead of the
-// nine planes of G).
+// explicit D_i G_i (unshifted f, u = sum c f). G_i at the destination x + c_i is
+// the destination's own, which its thread forms from its f; G_i(x, t - 1) is
+// formed again from u at t - 1 (two planes kept instead of the nine planes of G).
 //
-// FP32 with nx even runs kernels with two horizontally adjacent cells a thread
-// in packed FP32 instructions. The collisions of Remarks 1 and 2 and of the
-// two-cell Remark 4 kernel take opposite directions in pairs (the parts of s_i
-// and G_i even in c shared, the odd parts sign-flipped).
+// Every step is one kernel: Remark 3 one unit a thread, the others a row march or,
+// in small domains, tiles for several steps. A unit is a cell, or in FP32 with nx
+// even two horizontally adjacent cells in packed FP32 instructions. The cell
+// arithmetic (sp_moments_of, sp_collide) is written once for all of them.
 #include <cmath>
 #include <cstring>
 #include <string>
 
 #include "lbm.h"
+#include "lbm_mbar.cuh"
+#include "lbm_tileplan.h"
 #include "lbm_device.cuh"   // lbm::F2, two cells' FP32 values in packed instructions
 
 namespace {
 
 using lbm::F2;
-__device__ __forceinline__ F2& operator+=(F2& a, F2 b) { return a = a + b; }
-__device__ __forceinline__ F2& operator*=(F2& a, F2 b) { return a = a * b; }
-// 1/x and sqrt(x), correctly rounded per lane, so one-cell and two-cell kernels agree
-template <typename R> __device__ __forceinline__ R sp_inv(R x) { return R(1) / x; }
-__device__ __forceinline__ F2 sp_inv(F2 x) { return F2(1.f / x.v.x, 1.f / x.v.y); }
-template <typename R> __device__ __forceinline__ R sp_sqrt(R x) { return sqrt(x); }
-__device__ __forceinline__ F2 sp_sqrt(F2 x) { return F2(sqrtf(x.v.x), sqrtf(x.v.y)); }
-
-// Loads and stores of cell pairs (x, x + 1), x even: one 8-byte access.
-__device__ __forceinline__ F2 ld2(const float* p) { return F2(*reinterpret_cast<const float2*>(p)); }
-__device__ __forceinline__ void st2(float* p, F2 v) { *reinterpret_cast<float2*>(p) = v.v; }
-// A row of a plane around the pair: columns x - 2 .. x + 3 as three pairs
-// (wrapping in x; nx even). at(dx) is the pair of columns (x + dx, x + 1 + dx).
-struct Row2 {
-    float2 l, m, r;
-    __device__ __forceinline__ Row2(const float* row, int x, int nx) {
-        l = *reinterpret_cast<const float2*>(row + (x == 0 ? nx - 2 : x - 2));
-        m = *reinterpret_cast<const float2*>(row + x);
-        r = *reinterpret_cast<const float2*>(row + (x + 2 == nx ? 0 : x + 2));
-    }
-    __device__ __forceinline__ F2 at(int dx) const {
-        return dx < 0 ? F2(l.y, m.x) : (dx > 0 ? F2(m.y, r.x) : F2(m));
-    }
-};
-
 constexpr int kQ = 9;
 __host__ __device__ constexpr int sx(int i) { return i == 1 || i == 5 || i == 8 ? 1 : (i == 3 || i == 6 || i == 7 ? -1 : 0); }
 __host__ __device__ constexpr int sy(int i) { return i == 2 || i == 5 || i == 6 ? 1 : (i == 4 || i == 7 || i == 8 ? -1 : 0); }
@@ -79,23 +52,6 @@ __host__ __device__ constexpr int sopp(int i) { return i == 0 ? 0 : (i <= 4 ? (i
 static_assert(sopp(1) == 3 && sopp(2) == 4 && sopp(5) == 7 && sopp(6) == 8 && sopp(8) == 6, "D2Q9 opposites");
 // one direction of each opposite pair (1, 2, 5, 6; their opposites 3, 4, 7, 8)
 __host__ __device__ constexpr int pair2(int q) { return q == 0 ? 1 : q == 1 ? 2 : q == 2 ? 5 : 6; }
-
-// Push-streaming of direction i of a pair (x, x + 1), x even (32-bit offsets:
-// the context checks 9 nx ny < 2^31): with bounce, back
-// into the pair as the opposite direction (halfway wall); else to row yrow,
-// columns x + c_x and x + 1 + c_x (wrapped). c_x = 0 keeps the pair together.
-__device__ __forceinline__ void sp_store2(float* __restrict__ gout, int N, int c, int x, int yrow, int nx,
-                                          bool bounce, int i, F2 v) {
-    if (bounce) {
-        st2(gout + sopp(i) * N + c, v);
-    } else if (sx(i) == 0) {
-        st2(gout + i * N + yrow * nx + x, v);
-    } else {
-        const int row = i * N + yrow * nx;
-        gout[row + (sx(i) < 0 ? (x == 0 ? nx - 1 : x - 1) : x + 1)] = v.v.x;
-        gout[row + (sx(i) < 0 ? x : (x + 2 == nx ? 0 : x + 2))] = v.v.y;
-    }
-}
 
 struct SpConst {
     int nx, ny, walls;
@@ -144,70 +100,6 @@ __device__ __forceinline__ SpCell<R> sp_moments(const SpConst& K, const R g[kQ],
     return m;
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256) sp_step_kernel(const R* __restrict__ gin, R* __restrict__ gout,
-                                                      const R* __restrict__ src, long long N, SpConst K) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    const int x = (int)(c % K.nx), y = (int)(c / K.nx);
-    R g[kQ], G[kQ];
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) g[i] = gin[i * N + c];
-    const R S = src[c];
-    const SpCell<R> m = sp_moments(K, g, S, G);
-    const R uu = m.ux * m.ux + m.uy * m.uy;
-    const R ig = R(K.inv_tau), sg = R(K.src);
-    const bool bot = K.walls && y == 0, top = K.walls && y == K.ny - 1;
-    const int xs[3] = {x == 0 ? K.nx - 1 : x - 1, x, x == K.nx - 1 ? 0 : x + 1};
-    const int ys[3] = {K.walls ? y - 1 : (y == 0 ? K.ny - 1 : y - 1), y,
-                       K.walls ? y + 1 : (y == K.ny - 1 ? 0 : y + 1)};
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-        const R cu = R(sx(i)) * m.ux + R(sy(i)) * m.uy;
-        const R si = R(sw(i)) * (R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu);
-        const R geq = i == 0 ? R(3) * m.p * (R(sw(0)) - R(1)) + si : R(3) * m.p * R(sw(i)) + si;
-        const R post = g[i] - (g[i] - geq) * ig + sg * G[i];
-        long long dst;
-        int k = i;
-        if ((sy(i) > 0 && top) || (sy(i) < 0 && bot)) {
-            dst = c;
-            k = sopp(i);
-        } else {
-            dst = (long long)ys[sy(i) + 1] * K.nx + xs[sx(i) + 1];
-        }
-        gout[k * N + dst] = post;
-    }
-}
-
-// FP32 step of Remark 3 with two horizontally adjacent cells (x, x + 1), x
-// even, per thread, computed together in packed FP32 instructions (F2): the
-// loads, the S read and the stores of directions with c_x = 0 are 8-byte
-// pairs; directions with c_x != 0 split into two 4-byte stores. nx even.
-__global__ void __launch_bounds__(256, 4) sp_step_x2_kernel(const float* __restrict__ gin, float* __restrict__ gout,
-                                                         const float* __restrict__ src, int N, SpConst K) {
-    const int c = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (c >= N) return;
-    const int x = (int)(c % K.nx), y = (int)(c / K.nx);
-    F2 g[kQ], G[kQ];
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) g[i] = F2(*reinterpret_cast<const float2*>(gin + i * N + c));
-    const F2 S(*reinterpret_cast<const float2*>(src + c));
-    const SpCell<F2> m = sp_moments(K, g, S, G);
-    const F2 uu = m.ux * m.ux + m.uy * m.uy;
-    const F2 ig = F2(float(K.inv_tau)), sg = F2(float(K.src));
-    const bool bot = K.walls && y == 0, top = K.walls && y == K.ny - 1;
-    const int ys[3] = {K.walls ? y - 1 : (y == 0 ? K.ny - 1 : y - 1), y,
-                       K.walls ? y + 1 : (y == K.ny - 1 ? 0 : y + 1)};
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-        const F2 cu = float(sx(i)) * m.ux + float(sy(i)) * m.uy;
-        const F2 si = float(sw(i)) * (F2(3.f) * cu + F2(4.5f) * cu * cu - F2(1.5f) * uu);
-        const F2 geq = i == 0 ? F2(3.f) * m.p * F2(float(sw(0) - 1.0)) + si : F2(3.f) * m.p * F2(float(sw(i))) + si;
-        const F2 post = g[i] - (g[i] - geq) * ig + sg * G[i];
-        sp_store2(gout, N, c, x, ys[sy(i) + 1], K.nx, (sy(i) > 0 && top) || (sy(i) < 0 && bot), i, post);
-    }
-}
-
 // ---- Remarks 1 and 2 (M = 1, 2) ----
 // g holds g_i - w_i a0 (a0 = 1 for Remark 1, p_0 for Remark 2: the rest state).
 // d = rho - 1 (Remark 1) or p - p_0 (Remark 2); a = rho or p_0, the factor of
@@ -226,7 +118,7 @@ __device__ __forceinline__ void sp1_moments(const SpConst& K, const R g[kQ], R S
     if constexpr (M == 1) {
         d = m0 + R(0.5) * S;                       // Eq. 27aa
         a = R(1) + d;
-        const R ir = sp_inv(a);
+        const R ir = R(1) / a;
         ux = (jx + R(0.5) * R(K.fx)) * ir;         // Eq. 27a
         uy = (jy + R(0.5) * R(K.fy)) * ir;
     } else {
@@ -234,174 +126,6 @@ __device__ __forceinline__ void sp1_moments(const SpConst& K, const R g[kQ], R S
         a = R(K.p0);
         ux = (jx + R(K.hp0fx)) * R(K.ip0);         // p_0 u = sum c g + p_0 F_1 / 2
         uy = (jy + R(K.hp0fy)) * R(K.ip0);
-    }
-}
-
-// post-collision value of direction i (Eq. 24 with the force term of the remark)
-template <int M, typename R>
-__device__ __forceinline__ R sp1_post(const SpConst& K, int i, R gi, R d, R a, R ux, R uy, R S, R Qd) {
-    const R sc = M == 1 ? R(1) : R(K.p0);          // S and F in the units of g
-    const R fx = R(K.fx) * sc, fy = R(K.fy) * sc, Sg = S * sc;
-    const R cu = R(sx(i)) * ux + R(sy(i)) * uy, cF = R(sx(i)) * fx + R(sy(i)) * fy;
-    const R uF = ux * fx + uy * fy, uu = ux * ux + uy * uy;
-    const R c2 = R(sx(i) * sx(i) + sy(i) * sy(i));
-    const R si = R(sw(i)) * (R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu);
-    const R geq = d * R(sw(i)) + a * si;
-    // (cc - c_s^2 I):(uF + Fu [- uu S] + Q div u I) / (2 c_s^4)
-    //   = 9 (c.u)(c.F) - 3 u.F [- 4.5 ((c.u)^2 - u.u / 3) S] + 4.5 (|c|^2 - 2/3) Q div u
-    R Gi = Sg + R(3) * cF + R(9) * cu * cF - R(3) * uF + R(4.5) * (c2 - R(2.0 / 3.0)) * Qd;
-    if constexpr (M == 1) Gi = Gi - R(4.5) * (cu * cu - uu * R(1.0 / 3.0)) * Sg;   // the u u S of Remark 1
-    return gi - (gi - geq) * R(K.inv_tau) + R(K.src) * (R(sw(i)) * Gi);
-}
-
-// The same for a direction i and its opposite j = opp(i): c_j = -c_i, so s_i and
-// G_i split into a part even in c (shared) and an odd part (sign flipped).
-template <int M, typename R>
-__device__ __forceinline__ void sp1_post_pair(const SpConst& K, int i, R gi, R gj, R d, R a, R ux, R uy, R S,
-                                              R Qd, R& pi, R& pj) {
-    const R sc = M == 1 ? R(1) : R(K.p0);
-    const R fx = R(K.fx) * sc, fy = R(K.fy) * sc, Sg = S * sc;
-    const R cu = R(sx(i)) * ux + R(sy(i)) * uy, cF = R(sx(i)) * fx + R(sy(i)) * fy;
-    const R uF = ux * fx + uy * fy, uu = ux * ux + uy * uy;
-    const R c2 = R(sx(i) * sx(i) + sy(i) * sy(i));
-    const R wi = R(sw(i));
-    const R geq_e = d * wi + a * (wi * (R(4.5) * cu * cu - R(1.5) * uu)), geq_o = a * (wi * (R(3) * cu));
-    R G_e = Sg + R(9) * cu * cF - R(3) * uF + R(4.5) * (c2 - R(2.0 / 3.0)) * Qd;
-    if constexpr (M == 1) G_e = G_e - R(4.5) * (cu * cu - uu * R(1.0 / 3.0)) * Sg;   // the u u S of Remark 1
-    G_e = wi * G_e;
-    const R G_o = wi * (R(3) * cF);
-    const R ig = R(K.inv_tau), sg = R(K.src);
-    pi = gi - (gi - (geq_e + geq_o)) * ig + sg * (G_e + G_o);
-    pj = gj - (gj - (geq_e - geq_o)) * ig + sg * (G_e - G_o);
-}
-
-
-template <int M, typename R>
-__global__ void __launch_bounds__(256) sp1_moments_kernel(const R* __restrict__ gin, const R* __restrict__ src,
-                                                          long long N, SpConst K, R* __restrict__ ufield) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    R g[kQ], d, a, ux, uy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) g[i] = gin[i * N + c];
-    sp1_moments<M>(K, g, src[c], d, a, ux, uy);
-    ufield[c] = ux;
-    ufield[N + c] = uy;
-}
-
-template <int M, typename R>
-__global__ void __launch_bounds__(256) sp1_step_kernel(const R* __restrict__ gin, R* __restrict__ gout,
-                                                       const R* __restrict__ src, const R* __restrict__ ufield,
-                                                       long long N, SpConst K) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    const int x = (int)(c % K.nx), y = (int)(c / K.nx);
-    R g[kQ], d, a, ux, uy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) g[i] = gin[i * N + c];
-    const R S = src[c];
-    sp1_moments<M>(K, g, S, d, a, ux, uy);
-    const int xs[3] = {x == 0 ? K.nx - 1 : x - 1, x, x == K.nx - 1 ? 0 : x + 1};
-    // stencil rows: mirror at walls (reading Q7), wrap when periodic
-    const int yst[3] = {y == 0 ? (K.walls ? 0 : K.ny - 1) : y - 1, y,
-                        y == K.ny - 1 ? (K.walls ? K.ny - 1 : 0) : y + 1};
-    R divu = R(0);   // Eq. 30a applied to u
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) {
-        const long long n = (long long)yst[sy(i) + 1] * K.nx + xs[sx(i) + 1];
-        R cu = R(0);
-        if (sx(i)) cu += sx(i) > 0 ? ufield[n] : -ufield[n];
-        if (sy(i)) cu += sy(i) > 0 ? ufield[N + n] : -ufield[N + n];
-        divu += R(sw(i)) * cu;
-    }
-    divu *= R(3);
-    // Q = (2/d) a c_s^2 - xi / (tau_g - 1/2); K.Qd0 = -xi / (tau_g - 1/2)
-    const R Qd = (a * R(1.0 / 3.0) + R(K.Qd0)) * divu;
-    const bool bot = K.walls && y == 0, top = K.walls && y == K.ny - 1;
-    const int ys[3] = {K.walls ? y - 1 : (y == 0 ? K.ny - 1 : y - 1), y,
-                       K.walls ? y + 1 : (y == K.ny - 1 ? 0 : y + 1)};
-    auto emit = [&](int i, R post) {
-        long long dst;
-        int k = i;
-        if ((sy(i) > 0 && top) || (sy(i) < 0 && bot)) {
-            dst = c;
-            k = sopp(i);
-        } else {
-            dst = (long long)ys[sy(i) + 1] * K.nx + xs[sx(i) + 1];
-        }
-        gout[k * N + dst] = post;
-    };
-    emit(0, sp1_post<M>(K, 0, g[0], d, a, ux, uy, S, Qd));
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = pair2(q), j = sopp(i);
-        R pi, pj;
-        sp1_post_pair<M>(K, i, g[i], g[j], d, a, ux, uy, S, Qd, pi, pj);
-        emit(i, pi);
-        emit(j, pj);
-    }
-}
-
-// FP32, two cells a thread (nx even)
-template <int M>
-__global__ void __launch_bounds__(256) sp1_moments_x2_kernel(const float* __restrict__ gin,
-                                                             const float* __restrict__ src, int N, SpConst K,
-                                                             float* __restrict__ ufield) {
-    const int c = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (c >= N) return;
-    F2 g[kQ], d, a, ux, uy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) g[i] = ld2(gin + i * N + c);
-    sp1_moments<M>(K, g, ld2(src + c), d, a, ux, uy);
-    st2(ufield + c, ux);
-    st2(ufield + N + c, uy);
-}
-
-template <int M>
-__global__ void __launch_bounds__(256, 3) sp1_step_x2_kernel(const float* __restrict__ gin, float* __restrict__ gout,
-                                                          const float* __restrict__ src,
-                                                          const float* __restrict__ ufield, int N, SpConst K) {
-    const int c = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (c >= N) return;
-    const int x = (int)(c % K.nx), y = (int)(c / K.nx);
-    F2 g[kQ], d, a, ux, uy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) g[i] = ld2(gin + i * N + c);
-    const F2 S = ld2(src + c);
-    sp1_moments<M>(K, g, S, d, a, ux, uy);
-    // stencil rows: mirror at walls (reading Q7), wrap when periodic
-    const int yst[3] = {y == 0 ? (K.walls ? 0 : K.ny - 1) : y - 1, y,
-                        y == K.ny - 1 ? (K.walls ? K.ny - 1 : 0) : y + 1};
-    F2 divu(0.f);   // Eq. 30a applied to u
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const int row = yst[r] * K.nx;
-        const Row2 UX(ufield + row, x, K.nx), UY(ufield + N + row, x, K.nx);
-#pragma unroll
-        for (int i = 1; i < kQ; ++i) {
-            if (sy(i) + 1 != r) continue;
-            F2 cu(0.f);
-            if (sx(i)) cu += sx(i) > 0 ? UX.at(sx(i)) : -UX.at(sx(i));
-            if (sy(i)) cu += sy(i) > 0 ? UY.at(sx(i)) : -UY.at(sx(i));
-            divu += F2(float(sw(i))) * cu;
-        }
-    }
-    divu *= F2(3.f);
-    const F2 Qd = (a * F2(float(1.0 / 3.0)) + F2(float(K.Qd0))) * divu;
-    const bool bot = K.walls && y == 0, top = K.walls && y == K.ny - 1;
-    const int ys[3] = {K.walls ? y - 1 : (y == 0 ? K.ny - 1 : y - 1), y,
-                       K.walls ? y + 1 : (y == K.ny - 1 ? 0 : y + 1)};
-    auto emit = [&](int i, F2 post) {
-        sp_store2(gout, N, c, x, ys[sy(i) + 1], K.nx, (sy(i) > 0 && top) || (sy(i) < 0 && bot), i, post);
-    };
-    emit(0, sp1_post<M>(K, 0, g[0], d, a, ux, uy, S, Qd));
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = pair2(q), j = sopp(i);
-        F2 pi, pj;
-        sp1_post_pair<M>(K, i, g[i], g[j], d, a, ux, uy, S, Qd, pi, pj);
-        emit(i, pi);
-        emit(j, pj);
     }
 }
 
@@ -438,7 +162,7 @@ __device__ __forceinline__ void sp4_u(const R f[kQ], R& ux, R& uy) {
 
 template <typename R>
 __device__ __forceinline__ void sp4_force(const SpConst& K, R ux, R uy, R& Fx, R& Fy) {
-    const R k = R(K.dl) + R(K.dq) * sp_sqrt(ux * ux + uy * uy);
+    const R k = R(K.dl) + R(K.dq) * sqrt(ux * ux + uy * uy);
     Fx = R(K.fx) - k * ux;
     Fy = R(K.fy) - k * uy;
 }
@@ -450,175 +174,6 @@ __device__ __forceinline__ R sp4_G(const SpConst& K, int i, R S, R ux, R uy, R F
     const R c2 = R(sx(i) * sx(i) + sy(i) * sy(i));
     return R(sw(i)) * (S + R(3) * cF + R(9) * cu * cF - R(3) * (ux * Fx + uy * Fy) +
                        R(4.5) * (c2 - R(2.0 / 3.0)) * R(K.Qc) * S);
-}
-
-// sp4_G split into the part even in c and the odd part c.F / c_s^2 (times w_i)
-template <typename R>
-__device__ __forceinline__ void sp4_G_parts(const SpConst& K, int i, R S, R ux, R uy, R Fx, R Fy, R& e, R& o) {
-    const R cu = R(sx(i)) * ux + R(sy(i)) * uy, cF = R(sx(i)) * Fx + R(sy(i)) * Fy;
-    const R c2 = R(sx(i) * sx(i) + sy(i) * sy(i));
-    e = R(sw(i)) * (S + R(9) * cu * cF - R(3) * (ux * Fx + uy * Fy) + R(4.5) * (c2 - R(2.0 / 3.0)) * R(K.Qc) * S);
-    o = R(sw(i)) * (R(3) * cF);
-}
-
-// u = sum c f and F(u) of every cell, four planes (the update at x needs G at
-// x + c_i, so these first; F is kept so that no neighbour evaluates the drag)
-template <typename R>
-__global__ void __launch_bounds__(256) sp4_moments_kernel(const R* __restrict__ fin, long long N,
-                                                          SpConst K, R* __restrict__ unow) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    R f[kQ], ux, uy, Fx, Fy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) f[i] = fin[i * N + c];
-    sp4_u(f, ux, uy);
-    sp4_force(K, ux, uy, Fx, Fy);
-    unow[c] = ux;
-    unow[N + c] = uy;
-    unow[2 * N + c] = Fx;
-    unow[3 * N + c] = Fy;
-}
-
-template <typename R>
-__global__ void __launch_bounds__(256) sp4_step_kernel(const R* __restrict__ fin, R* __restrict__ fout,
-                                                       const R* __restrict__ src, const R* __restrict__ unow,
-                                                       const R* __restrict__ uprev, long long N, SpConst K) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    const int x = (int)(c % K.nx), y = (int)(c / K.nx);
-    R f[kQ], ux, uy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) f[i] = fin[i * N + c];
-    const R S = src[c];
-    sp4_u(f, ux, uy);
-    const R Fx = unow[2 * N + c], Fy = unow[3 * N + c];
-    R rest = R(0);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) rest += f[i];
-    const R uu = ux * ux + uy * uy;
-    const R G0 = sp4_G(K, 0, S, ux, uy, Fx, Fy);
-    // Eq. 28 for the unshifted f: c_s^2 / (1 - w_0) = 3/5, s_0(u) = -(2/3) u.u, tau_g G_0
-    const R p = R(0.6) * (rest - R(2.0 / 3.0) * uu + R(K.tau) * G0);
-    const R upx = uprev[c], upy = uprev[N + c], Fpx = uprev[2 * N + c], Fpy = uprev[3 * N + c];
-    const R ig = R(K.inv_tau);
-    const bool bot = K.walls && y == 0, top = K.walls && y == K.ny - 1;
-    const int xs[3] = {x == 0 ? K.nx - 1 : x - 1, x, x == K.nx - 1 ? 0 : x + 1};
-    const int ys[3] = {K.walls ? y - 1 : (y == 0 ? K.ny - 1 : y - 1), y,
-                       K.walls ? y + 1 : (y == K.ny - 1 ? 0 : y + 1)};
-    // G_i(x + c_i, t): the destination cell, mirrored about a wall
-    auto Gnb = [&](int i) {
-        const bool wall = (sy(i) > 0 && top) || (sy(i) < 0 && bot);
-        const long long n = (long long)(wall ? y : ys[sy(i) + 1]) * K.nx + xs[sx(i) + 1];
-        return sp4_G(K, i, src[n], unow[n], unow[N + n], unow[2 * N + n], unow[3 * N + n]);
-    };
-    // to x + c_i, or (wall) back into this cell as opp(i) after the bounce-back of g = f - G/2
-    auto emit = [&](int i, R post, R Gn, R Gopp) {
-        if ((sy(i) > 0 && top) || (sy(i) < 0 && bot))
-            fout[sopp(i) * N + c] = post - R(0.5) * Gn + R(0.5) * Gopp;
-        else
-            fout[i * N + (long long)ys[sy(i) + 1] * K.nx + xs[sx(i) + 1]] = post;
-    };
-    {   // rest direction: its destination is this cell
-        const R geq = R(3) * p * (R(sw(0)) - R(1)) + R(sw(0)) * (-R(1.5) * uu);
-        const R Gp = sp4_G(K, 0, S, upx, upy, Fpx, Fpy);
-        emit(0, f[0] - (f[0] - geq) * ig + G0 + R(0.5) * (G0 - Gp), G0, G0);
-    }
-    // opposite pairs: G at t and t - 1 and s_i split into parts even and odd in c
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = pair2(q), j = sopp(i);
-        const R wi = R(sw(i));
-        const R cu = R(sx(i)) * ux + R(sy(i)) * uy;
-        const R ge = R(3) * p * wi + wi * (R(4.5) * cu * cu - R(1.5) * uu), go = wi * (R(3) * cu);
-        R Ge, Go, Gpe, Gpo;
-        sp4_G_parts(K, i, S, ux, uy, Fx, Fy, Ge, Go);
-        sp4_G_parts(K, i, S, upx, upy, Fpx, Fpy, Gpe, Gpo);
-        const R Gi = Ge + Go, Gj = Ge - Go, Gni = Gnb(i), Gnj = Gnb(j);
-        emit(i, f[i] - (f[i] - (ge + go)) * ig + Gi + R(0.5) * (Gni - (Gpe + Gpo)), Gni, Gj);
-        emit(j, f[j] - (f[j] - (ge - go)) * ig + Gj + R(0.5) * (Gnj - (Gpe - Gpo)), Gnj, Gi);
-    }
-}
-
-// Remark 4 scheme, FP32, two cells a thread (nx even)
-__global__ void __launch_bounds__(256) sp4_moments_x2_kernel(const float* __restrict__ fin, int N,
-                                                             SpConst K, float* __restrict__ unow) {
-    const int c = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (c >= N) return;
-    F2 f[kQ], ux, uy, Fx, Fy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) f[i] = ld2(fin + i * N + c);
-    sp4_u(f, ux, uy);
-    sp4_force(K, ux, uy, Fx, Fy);
-    st2(unow + c, ux);
-    st2(unow + N + c, uy);
-    st2(unow + 2 * N + c, Fx);
-    st2(unow + 3 * N + c, Fy);
-}
-
-__global__ void __launch_bounds__(256) sp4_step_x2_kernel(const float* __restrict__ fin, float* __restrict__ fout,
-                                                          const float* __restrict__ src,
-                                                          const float* __restrict__ unow,
-                                                          const float* __restrict__ uprev, int N, SpConst K) {
-    const int c = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (c >= N) return;
-    const int x = (int)(c % K.nx), y = (int)(c / K.nx);
-    F2 f[kQ], ux, uy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) f[i] = ld2(fin + i * N + c);
-    const F2 S = ld2(src + c);
-    sp4_u(f, ux, uy);
-    const F2 Fx = ld2(unow + 2 * N + c), Fy = ld2(unow + 3 * N + c);
-    F2 rest(0.f);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) rest += f[i];
-    const F2 uu = ux * ux + uy * uy;
-    const F2 G0 = sp4_G(K, 0, S, ux, uy, Fx, Fy);
-    const F2 p = F2(0.6f) * (rest - F2(float(2.0 / 3.0)) * uu + F2(float(K.tau)) * G0);
-    const F2 upx = ld2(uprev + c), upy = ld2(uprev + N + c), Fpx = ld2(uprev + 2 * N + c),
-             Fpy = ld2(uprev + 3 * N + c);
-    const F2 ig(float(K.inv_tau));
-    const bool bot = K.walls && y == 0, top = K.walls && y == K.ny - 1;
-    const int ys[3] = {K.walls ? y - 1 : (y == 0 ? K.ny - 1 : y - 1), y,
-                       K.walls ? y + 1 : (y == K.ny - 1 ? 0 : y + 1)};
-    // rows of the destinations x + c_i for G_i(x + c_i, t): mirrored about a wall
-    const int yst[3] = {y == 0 ? (K.walls ? 0 : K.ny - 1) : y - 1, y,
-                        y == K.ny - 1 ? (K.walls ? K.ny - 1 : 0) : y + 1};
-    const int xl[3] = {x == 0 ? K.nx - 1 : x - 1, x, x + 1};   // left lane's x + c_x
-    const int xr[3] = {x, x + 1, x + 2 == K.nx ? 0 : x + 2};   // right lane's
-    // G_i(x + c_i, t) from the destination's u, F and S
-    auto Gnb = [&](int i) {
-        const int row = yst[sy(i) + 1] * K.nx;
-        const int a = row + xl[sx(i) + 1], b = row + xr[sx(i) + 1];
-        auto nb = [&](const float* pl) { return sx(i) == 0 ? ld2(pl + a) : F2(pl[a], pl[b]); };
-        return sp4_G(K, i, nb(src), nb(unow), nb(unow + N), nb(unow + 2 * N), nb(unow + 3 * N));
-    };
-    {   // rest direction: never crosses a wall; its destination is this cell
-        const F2 Gp = sp4_G(K, 0, S, upx, upy, Fpx, Fpy);
-        const F2 geq = F2(3.f) * p * F2(float(sw(0) - 1.0)) + float(sw(0)) * (-F2(1.5f) * uu);
-        sp_store2(fout, N, c, x, y, K.nx, false, 0, f[0] - (f[0] - geq) * ig + G0 + F2(0.5f) * (G0 - Gp));
-    }
-    // opposite pairs (i, j = opp(i)): G of this cell at t and t - 1 and s_i split
-    // into parts even and odd in c
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = pair2(q), j = sopp(i);
-        const float wi = float(sw(i));
-        const F2 cu = float(sx(i)) * ux + float(sy(i)) * uy;
-        const F2 ge = F2(3.f * wi) * p + wi * (F2(4.5f) * cu * cu - F2(1.5f) * uu), go = wi * (F2(3.f) * cu);
-        F2 Ge, Go, Gpe, Gpo;
-        sp4_G_parts(K, i, S, ux, uy, Fx, Fy, Ge, Go);
-        sp4_G_parts(K, i, S, upx, upy, Fpx, Fpy, Gpe, Gpo);
-        const F2 Gi = Ge + Go, Gj = Ge - Go;
-        const F2 Gni = Gnb(i), Gnj = Gnb(j);
-        F2 pi = f[i] - (f[i] - (ge + go)) * ig + Gi + F2(0.5f) * (Gni - (Gpe + Gpo));
-        F2 pj = f[j] - (f[j] - (ge - go)) * ig + Gj + F2(0.5f) * (Gnj - (Gpe - Gpo));
-        // bounce-back of g = f - G/2: leaves as i with G_i(x + c_i), returns as opp(i)
-        const bool bi = (sy(i) > 0 && top) || (sy(i) < 0 && bot), bj = (sy(j) > 0 && top) || (sy(j) < 0 && bot);
-        if (bi) pi = pi - F2(0.5f) * Gni + F2(0.5f) * Gj;
-        if (bj) pj = pj - F2(0.5f) * Gnj + F2(0.5f) * Gi;
-        sp_store2(fout, N, c, x, ys[sy(i) + 1], K.nx, bi, i, pi);
-        sp_store2(fout, N, c, x, ys[sy(j) + 1], K.nx, bj, j, pj);
-    }
 }
 
 template <typename R>
@@ -673,15 +228,562 @@ __global__ void sp_convert_kernel(const double* __restrict__ in, R* __restrict__
 }
 
 template <typename R>
-__global__ void sp_fill_kernel(R* __restrict__ out, double v, long long n) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < n) out[c] = R(v);
-}
-
-template <typename R>
 __global__ void sp_widen_kernel(const R* __restrict__ in, double* __restrict__ out, long long n) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c < n) out[c] = double(in[c]);
+}
+
+// ---- The step ----
+// One cell of a unit: float or double with explicit roundings; F2 is a unit of two
+// cells (x, x + 1), x even, in packed FP32 instructions (nx even).
+template <typename T>
+struct One {
+    T v;
+    One() = default;
+    __device__ __forceinline__ One(T x) : v(x) {}
+};
+__device__ __forceinline__ One<float> operator+(One<float> a, One<float> b) { return __fadd_rn(a.v, b.v); }
+__device__ __forceinline__ One<float> operator-(One<float> a, One<float> b) { return __fsub_rn(a.v, b.v); }
+__device__ __forceinline__ One<float> operator*(One<float> a, One<float> b) { return __fmul_rn(a.v, b.v); }
+__device__ __forceinline__ One<float> fmadd(One<float> a, One<float> b, One<float> c) { return __fmaf_rn(a.v, b.v, c.v); }
+__device__ __forceinline__ One<double> operator+(One<double> a, One<double> b) { return __dadd_rn(a.v, b.v); }
+__device__ __forceinline__ One<double> operator-(One<double> a, One<double> b) { return __dsub_rn(a.v, b.v); }
+__device__ __forceinline__ One<double> operator*(One<double> a, One<double> b) { return __dmul_rn(a.v, b.v); }
+__device__ __forceinline__ One<double> fmadd(One<double> a, One<double> b, One<double> c) { return __fma_rn(a.v, b.v, c.v); }
+// 1/x and sqrt(x), correctly rounded per lane
+template <typename T> __device__ __forceinline__ One<T> sp_inv(One<T> x) { return One<T>(T(1) / x.v); }
+template <typename T> __device__ __forceinline__ One<T> sp_sqrt(One<T> x) { return One<T>(sqrt(x.v)); }
+__device__ __forceinline__ F2 sp_inv(F2 x) { return F2(1.f / x.v.x, 1.f / x.v.y); }
+__device__ __forceinline__ F2 sp_sqrt(F2 x) { return F2(sqrtf(x.v.x), sqrtf(x.v.y)); }
+
+// How a unit sits in memory: T values of one cell or a pair, one access.
+template <typename V> struct Unit;
+template <typename T> struct Unit<One<T>> {
+    using R = T;       // element of a plane
+    using E = T;       // a unit in shared memory
+    static constexpr int cells = 1;
+    __device__ __forceinline__ static One<T> ld(const T* p) { return One<T>(*p); }
+    __device__ __forceinline__ static void st(T* p, One<T> v) { *p = v.v; }
+    __device__ __forceinline__ static E pack(One<T> v) { return v.v; }
+    // the unit dx cells right of unit t of a row in shared memory
+    __device__ __forceinline__ static One<T> at(const E* row, int t, int dx) { return One<T>(row[t + dx]); }
+    // push direction c_x = dx of unit x of a row; nx: columns
+    __device__ __forceinline__ static void push(T* row, int x, int nx, int dx, One<T> v) {
+        const int X = x + dx;
+        row[X < 0 ? nx - 1 : (X == nx ? 0 : X)] = v.v;
+    }
+};
+template <> struct Unit<F2> {
+    using R = float;
+    using E = float2;
+    static constexpr int cells = 2;
+    __device__ __forceinline__ static F2 ld(const float* p) { return F2(*reinterpret_cast<const float2*>(p)); }
+    __device__ __forceinline__ static void st(float* p, F2 v) { *reinterpret_cast<float2*>(p) = v.v; }
+    __device__ __forceinline__ static E pack(F2 v) { return v.v; }
+    __device__ __forceinline__ static F2 at(const E* row, int t, int dx) {
+        if (dx < 0) return F2(row[t - 1].y, row[t].x);
+        if (dx > 0) return F2(row[t].y, row[t + 1].x);
+        return F2(row[t]);
+    }
+    __device__ __forceinline__ static void push(float* row, int x, int nx, int dx, F2 v) {
+        if (dx == 0) {   // keeps the pair together
+            st(row + x, v);
+        } else {
+            row[dx < 0 ? (x == 0 ? nx - 1 : x - 1) : x + 1] = v.v.x;
+            row[dx < 0 ? x : (x + 2 == nx ? 0 : x + 2)] = v.v.y;
+        }
+    }
+};
+
+// Constants of the step in the arithmetic type, derived on the host (SpConst) so
+// that the kernels convert and combine nothing. F is in the units of g (Remark 2:
+// p_0 F_1); ka, kd, k0: 1 + 4.5 (|c|^2 - 2/3) Q of the axes, the diagonals and the
+// rest direction (Remark 3), times w_i.
+template <typename T>
+struct SpK {
+    int nx, ny, walls;
+    T om, sg, om_h;            // 1/tau_g, 1 - 1/(2 tau_g), om / 2
+    T fx, fy, hfx, hfy;        // F, F / 2
+    T sgfx, sgfy, hsgfx, hsgfy;   // sg F, sg F / 2
+    T ka, kd, k0, ska, skd, sk0;  // Remark 3, Remark 4; s..: times sg
+    T tgm, tau;
+    T sc, hS, p0, ip0;         // Remarks 1, 2: units of S; S / 2 in them; p_0, 1 / p_0 (Remark 1: unused)
+    T q, q0;                   // gs Q = (a q + q0) 12 div u
+    T dl, dq;                  // drag
+};
+
+template <typename T>
+SpK<T> sp_consts(const SpConst& K, int model) {
+    SpK<T> k;
+    const double sc = model == 2 ? K.p0 : 1.0, fx = sc * K.fx, fy = sc * K.fy, om = K.inv_tau, sg = K.src;
+    const double ka = (1.0 + 1.5 * K.Qc) / 9.0, kd = (1.0 + 6.0 * K.Qc) / 36.0, k0 = (1.0 - 3.0 * K.Qc) * 4.0 / 9.0;
+    k.nx = K.nx; k.ny = K.ny; k.walls = K.walls;
+    k.om = T(om); k.sg = T(sg); k.om_h = T(0.5 * om);
+    k.fx = T(fx); k.fy = T(fy); k.hfx = T(0.5 * fx); k.hfy = T(0.5 * fy);
+    k.sgfx = T(sg * fx); k.sgfy = T(sg * fy); k.hsgfx = T(0.5 * sg * fx); k.hsgfy = T(0.5 * sg * fy);
+    k.ka = T(ka); k.kd = T(kd); k.k0 = T(k0); k.ska = T(sg * ka); k.skd = T(sg * kd); k.sk0 = T(sg * k0);
+    k.tgm = T(K.tgm); k.tau = T(K.tau);
+    k.sc = T(sc); k.hS = T(0.5 * sc); k.p0 = T(K.p0); k.ip0 = T(K.ip0);
+    k.q = T(sg / 36.0); k.q0 = T(sg * K.Qd0 / 12.0);
+    k.dl = T(K.dl); k.dq = T(K.dq);
+    return k;
+}
+
+// The four models by one number: Remarks 1, 2, 3 and the Remark 4 scheme.
+// What a cell's neighbours need of it (values of the shared-memory ring): u for
+// div u (Remarks 1, 2), G_1 .. G_8 for G_i at x + c_i (Remark 4), nothing (3).
+template <int KIND> constexpr int kRing = KIND == 4 ? 8 : (KIND == 3 ? 0 : 2);
+
+// A cell's own values besides its populations and S.
+template <typename V>
+struct SpMom { V ux, uy, a, b; };   // u; Remarks 1, 2: d and a of the equilibrium; Remark 4: a = G_0
+
+template <typename V>
+__device__ __forceinline__ void sp_j(const V (&g)[kQ], V& jx, V& jy) {
+    const V a = g[5] - g[7], b = g[6] - g[8];
+    jx = (g[1] - g[3]) + (a - b);
+    jy = (g[2] - g[4]) + (a + b);
+}
+template <typename V>
+__device__ __forceinline__ V sp_rest(const V (&g)[kQ]) {
+    return ((g[1] + g[2]) + (g[3] + g[4])) + ((g[5] + g[6]) + (g[7] + g[8]));
+}
+
+// (1 - om) g + x. In FP32 as x - om g, then + g: 1 - om rounded to FP32 would
+// give every step a bias of up to 2^-25 of the momentum. (FP64: one operation.)
+template <typename T>
+__device__ __forceinline__ One<T> sp_relax(T om, One<T> g, One<T> x) {
+    if constexpr (sizeof(T) == 8) return fmadd(One<T>(T(1) - om), g, x);
+    else return fmadd(One<T>(-om), g, x) + g;
+}
+__device__ __forceinline__ F2 sp_relax(float om, F2 g, F2 x) { return fmadd(F2(-om), g, x) + g; }
+// The odd parts 3 w_i c.T of a vector T over the axes (a) and, as components, the
+// diagonals (d = a / 4), from T / 2. The FP32 constants here and below (w_i, w_0 -
+// 1, 3/5 and 3 p from p) are the roundings of the remarks' own factors: products
+// of them rounded once instead, or sums that conserve the momentum exactly, are
+// closer to FP64 but drift from these by up to 1e-4 of a weak velocity component
+// in 200 steps.
+template <typename V>
+__device__ __forceinline__ void sp_odd(V half, V& a, V& d) {
+    using T = typename Unit<V>::R;
+    a = V(T(1) / T(9)) * (V(T(6)) * half);
+    d = V(T(0.25)) * a;
+}
+
+// Remark 4: F(u), and the parts of G_i even and odd in c of the pairs (1, 3),
+// (2, 4), (5, 7), (6, 8); G_0 returned.
+template <typename V, typename T>
+__device__ __forceinline__ void sp4_F(const SpK<T>& K, V ux, V uy, V& Fx, V& Fy) {
+    const V k = fmadd(V(K.dq), sp_sqrt(fmadd(ux, ux, uy * uy)), V(K.dl));
+    Fx = V(K.fx) - k * ux;
+    Fy = V(K.fy) - k * uy;
+}
+template <typename V, typename T>
+__device__ __forceinline__ V sp4_Gs(const SpK<T>& K, V S, V ux, V uy, V Fx, V Fy, V (&e)[4], V (&o)[4]) {
+    const V t = V(T(-3)) * fmadd(ux, Fx, uy * Fy);
+    const V ea = fmadd(S, V(K.ka), V(T(1) / T(9)) * t), ed = fmadd(S, V(K.kd), V(T(1) / T(36)) * t);
+    const V up = V(T(0.25)) * (ux + uy), um = V(T(0.25)) * (uy - ux), Fp = Fx + Fy, Fm = Fy - Fx;
+    e[0] = fmadd(ux, Fx, ea);
+    e[1] = fmadd(uy, Fy, ea);
+    e[2] = fmadd(up, Fp, ed);
+    e[3] = fmadd(um, Fm, ed);
+    V dx, dy;
+    sp_odd(V(T(0.5)) * Fx, o[0], dx);
+    sp_odd(V(T(0.5)) * Fy, o[1], dy);
+    o[2] = dx + dy;
+    o[3] = dy - dx;
+    return fmadd(S, V(K.k0), V(T(4) / T(9)) * t);
+}
+
+// u and what the neighbours need (put(r, value): ring value r).
+template <int KIND, typename V, typename T, typename Put>
+__device__ __forceinline__ void sp_moments_of(const SpK<T>& K, const V (&g)[kQ], V S, SpMom<V>& m, Put&& put) {
+    V jx, jy;
+    sp_j(g, jx, jy);
+    if constexpr (KIND == 1) {                       // rho - 1 (Eq. 27aa), rho; u (Eq. 27a)
+        m.a = fmadd(V(K.hS), S, g[0] + sp_rest(g));
+        m.b = V(T(1)) + m.a;
+        const V ir = sp_inv(m.b);
+        m.ux = (jx + V(K.hfx)) * ir;
+        m.uy = (jy + V(K.hfy)) * ir;
+    } else if constexpr (KIND == 2) {                // p - p_0, p_0
+        m.a = fmadd(V(K.hS), S, g[0] + sp_rest(g));
+        m.b = V(K.p0);
+        m.ux = (jx + V(K.hfx)) * V(K.ip0);
+        m.uy = (jy + V(K.hfy)) * V(K.ip0);
+    } else if constexpr (KIND == 3) {
+        m.ux = jx + V(K.hfx);
+        m.uy = jy + V(K.hfy);
+    } else {                                         // Remark 4: u = sum c f, G_i with F(u)
+        m.ux = jx;
+        m.uy = jy;
+        V Fx, Fy, e[4], o[4];
+        sp4_F(K, jx, jy, Fx, Fy);
+        m.a = sp4_Gs(K, S, jx, jy, Fx, Fy, e, o);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            put(pair2(k) - 1, e[k] + o[k]);
+            put(sopp(pair2(k)) - 1, e[k] - o[k]);
+        }
+    }
+    if constexpr (KIND == 1 || KIND == 2) {
+        put(0, m.ux);
+        put(1, m.uy);
+    }
+}
+
+// Collision (Eq. 24 with the remark's equilibrium and force term). Opposite
+// directions share the part even in c: with sg = 1 - 1/(2 tau_g) and om = 1/tau_g,
+//   g_i* = (1 - om) g_i + E_i +- O_i,  E_i = (c.u)(c.V) + E0,  O_i = 3 w_i c.T,
+// V = w_i (4.5 (om a [- sg S]) u + 9 sg F), T = om a u + sg F; the axes' weights
+// are four times the diagonals'. nb(r, dx, dy): ring value r of a
+// neighbour (mirrored about a wall); up: u at t - 1 (Remark 4); emit(i, value,
+// wall value): the population leaving in direction i, and what returns if a wall
+// reflects it (the same but for Remark 4).
+template <int KIND, typename V, typename T, typename Nb, typename Emit>
+__device__ __forceinline__ void sp_collide(const SpK<T>& K, const V (&g)[kQ], V S, const SpMom<V>& m, V upx, V upy,
+                                           Nb&& nb, Emit&& emit) {
+    const V ux = m.ux, uy = m.uy;
+    const V uu = fmadd(ux, ux, uy * uy);
+    const V ninth(T(1) / T(9)), q(T(0.25));
+    if constexpr (KIND == 4) {
+        const V G0 = m.a;
+        V Px, Py, pe[4], po[4];
+        sp4_F(K, upx, upy, Px, Py);
+        const V P0 = sp4_Gs(K, S, upx, upy, Px, Py, pe, po);
+        // Eq. 28 for the unshifted f: p = 3/5 [sum f_i - (2/3) u.u + tau_g G_0]
+        const V p3 = V(T(3)) * (V(T(0.6)) * fmadd(V(K.tau), G0, fmadd(V(T(-2) / T(3)), uu, sp_rest(g))));
+        const V om(K.om), half(T(0.5));
+        const V uu15 = V(T(-1.5)) * uu, b = p3 + uu15;   // 3 p - 1.5 u.u
+        const V geq0 = fmadd(V(T(4.0 / 9.0 - 1.0)), p3, V(T(4) / T(9)) * uu15);
+        emit(0, sp_relax(K.om, g[0], fmadd(om, geq0, fmadd(half, G0 - P0, G0))), V(T(0)));
+        const V ga = ninth * b, gd = q * ga;
+        const V up = q * (ux + uy), um = q * (uy - ux);
+        const V hx = half * ux, hy = half * uy;
+        const V ge[4] = {fmadd(hx, ux, ga), fmadd(hy, uy, ga), fmadd(V(T(2)) * up, up, gd),
+                         fmadd(V(T(2)) * um, um, gd)};
+        V ax, ay, dx, dy;
+        sp_odd(hx, ax, dx);
+        sp_odd(hy, ay, dy);
+        const V go[4] = {ax, ay, dx + dy, dy - dx};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = pair2(k), j = sopp(i);
+            // om g^eq_i - G_i(t - 1) / 2, even and odd parts
+            const V A = fmadd(om, ge[k], V(T(-0.5)) * pe[k]), B = fmadd(om, go[k], V(T(-0.5)) * po[k]);
+            const V Gi = nb(i - 1, 0, 0), Gj = nb(j - 1, 0, 0);
+            const V ni = nb(i - 1, sx(i), sy(i)), nj = nb(j - 1, sx(j), sy(j));
+            // without G_i(x + c_i) / 2
+            const V pi = sp_relax(K.om, g[i], Gi + (A + B)), pj = sp_relax(K.om, g[j], Gj + (A - B));
+            // bounce-back of f - G/2: leaves with G_i(x + c_i) / 2 less, returns as opp(i) with G_opp(x) / 2
+            emit(i, fmadd(half, ni, pi), fmadd(half, Gj, pi));
+            emit(j, fmadd(half, nj, pj), fmadd(half, Gi, pj));
+        }
+        return;
+    } else {
+        V Vx, Vy, Tx, Ty, Ea, Ed, r0;   // Tx, Ty: (om a u + sg F) / 2
+        const V uF = fmadd(ux, V(K.fx), uy * V(K.fy));
+        if constexpr (KIND == 3) {
+            // Eq. 28: p = 3/5 [sum g_i + S/2 - (2/3) u.u + (tau_g - 1/2) G_0]
+            const V t = V(T(-3)) * uF;
+            const V G0 = fmadd(S, V(K.k0), V(T(4) / T(9)) * t);
+            const V p3 = V(T(3)) * (V(T(0.6)) * fmadd(V(K.tgm), G0, fmadd(V(T(-2) / T(3)), uu,
+                                                                          fmadd(V(T(0.5)), S, sp_rest(g)))));
+            const V omp = V(K.om) * p3;
+            const V b0 = fmadd(V(K.om), V(T(-1.5)) * uu, V(K.sg) * t), b = omp + b0;
+            Vx = fmadd(V(K.om_h), ux, V(K.sgfx));
+            Vy = fmadd(V(K.om_h), uy, V(K.sgfy));
+            Tx = fmadd(V(K.om_h), ux, V(K.hsgfx));
+            Ty = fmadd(V(K.om_h), uy, V(K.hsgfy));
+            Ea = fmadd(S, V(K.ska), ninth * b);
+            Ed = fmadd(S, V(K.skd), V(T(1) / T(36)) * b);
+            r0 = fmadd(V(T(4.0 / 9.0 - 1.0)), omp, fmadd(S, V(K.sk0), V(T(4) / T(9)) * b0));
+        } else {
+            // 12 div u (Eq. 30a)
+            const V sa = nb(0, 1, 1) - nb(0, -1, -1), sb = nb(0, -1, 1) - nb(0, 1, -1);
+            const V ta = nb(1, 1, 1) - nb(1, -1, -1), tb = nb(1, -1, 1) - nb(1, 1, -1);
+            const V ax = nb(0, 1, 0) - nb(0, -1, 0), ay = nb(1, 0, 1) - nb(1, 0, -1);
+            const V div = fmadd(V(T(4)), ax + ay, (sa - sb) + (ta + tb));
+            const V gq = fmadd(m.b, V(K.q), V(K.q0)) * div;          // sg Q div u
+            const V Sg = V(K.sc) * S, om(K.om), sg(K.sg);
+            const V h = V(K.om_h) * m.b;                              // om a / 2
+            V hA, S2;
+            if constexpr (KIND == 1) {                                // with the u u S of Remark 1
+                hA = h - V(T(0.5)) * (sg * Sg);
+                S2 = fmadd(V(T(1.5)) * uu, Sg, Sg);
+            } else {
+                hA = h;
+                S2 = Sg;
+            }
+            Vx = fmadd(hA, ux, V(K.sgfx));
+            Vy = fmadd(hA, uy, V(K.sgfy));
+            if constexpr (KIND == 2) {   // (om p_0 / 2, a constant, rounded would be a bias of every step)
+                Tx = fmadd(V(K.om_h), m.b * ux, V(K.hsgfx));
+                Ty = fmadd(V(K.om_h), m.b * uy, V(K.hsgfy));
+            } else {
+                Tx = fmadd(h, ux, V(K.hsgfx));
+                Ty = fmadd(h, uy, V(K.hsgfy));
+            }
+            const V b = fmadd(om, fmadd(V(T(-1.5)) * m.b, uu, m.a), sg * fmadd(V(T(-3)), uF, S2));
+            Ea = ninth * fmadd(V(T(1.5)), gq, b);
+            Ed = V(T(1) / T(36)) * fmadd(V(T(6)), gq, b);
+            r0 = V(T(4) / T(9)) * fmadd(V(T(-3)), gq, b);
+        }
+        auto out = [&](int i, V v) { emit(i, v, v); };
+        out(0, sp_relax(K.om, g[0], r0));
+        auto pair = [&](int i, int j, V E, V O) {
+            out(i, sp_relax(K.om, g[i], E + O));
+            out(j, sp_relax(K.om, g[j], E - O));
+        };
+        V ox, oy, dx, dy;
+        sp_odd(Tx, ox, dx);
+        sp_odd(Ty, oy, dy);
+        pair(1, 3, fmadd(ux, Vx, Ea), ox);
+        pair(2, 4, fmadd(uy, Vy, Ea), oy);
+        pair(5, 7, fmadd(q * (ux + uy), Vx + Vy, Ed), dx + dy);
+        pair(6, 8, fmadd(q * (uy - ux), Vy - Vx, Ed), dy - dx);
+    }
+}
+
+// Push-streaming of a unit at column x of row y: into its neighbours, or back
+// reversed from a wall (halfway bounce-back). 32-bit offsets: 9 nx ny < 2^31.
+template <typename V>
+struct SpPush {
+    using U = Unit<V>;
+    typename U::R* out;
+    int N, nx, x, y, up, dn;
+    bool bot, top;
+    template <typename T>
+    __device__ __forceinline__ SpPush(const SpK<T>& K, typename U::R* out_, int N_, int x_, int y_)
+        : out(out_), N(N_), nx(K.nx), x(x_), y(y_) {
+        bot = K.walls && y == 0;
+        top = K.walls && y == K.ny - 1;
+        dn = y == 0 ? K.ny - 1 : y - 1;   // (not used at a wall)
+        up = y == K.ny - 1 ? 0 : y + 1;
+    }
+    __device__ __forceinline__ void operator()(int i, V v, V w) const {
+        if ((sy(i) > 0 && top) || (sy(i) < 0 && bot)) {
+            U::st(out + sopp(i) * N + y * nx + x, w);
+            return;
+        }
+        U::push(out + i * N + (sy(i) == 0 ? y : (sy(i) > 0 ? up : dn)) * nx, x, nx, sx(i), v);
+    }
+};
+
+// Remark 3, large domains: nothing of a neighbour is needed, one unit a thread.
+// 4096 x 4096 FP32 186 us a step (1.0 of the copy bandwidth); FP64 bound by its
+// FP64 operations: 2048 x 2048 1235 -> 638 us with the opposite pairs' even and odd
+// parts.
+template <typename V>
+__global__ void __launch_bounds__(256, 4) sp_cell_kernel(const typename Unit<V>::R* __restrict__ gin,
+                                                      typename Unit<V>::R* __restrict__ gout,
+                                                      const typename Unit<V>::R* __restrict__ src, int N,
+                                                      SpK<typename Unit<V>::R> K) {
+    using U = Unit<V>;
+    const int c = U::cells * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (c >= N) return;
+    const int y = c / K.nx, x = c - y * K.nx;
+    V g[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) g[i] = U::ld(gin + i * N + c);
+    const V S = U::ld(src + c);
+    SpMom<V> m;
+    sp_moments_of<3>(K, g, S, m, [](int, V) {});
+    sp_collide<3>(K, g, S, m, V(), V(), [](int, int, int) { return V(); }, SpPush<V>(K, gout, N, x, y));
+}
+
+// ---- One pass a step: row marches of Remarks 1, 2 and 4 ----
+// These models couple a cell to its neighbours only through functions of the
+// neighbours' own populations (u in div u; G_i at x + c_i), so a step is one
+// kernel: a block owns a strip of columns and marches over a run of rows, keeping
+// what the neighbours need of three rows in a shared-memory ring and the
+// populations of the collision row and the next one in registers. Per row: the
+// loads of the row after the next are issued, the next row's ring values formed,
+// one barrier, the collision. Every population is read once: in FP32 76 bytes a
+// cell for Remarks 1 and 2 (two kernels, one writing u, moved 132), 92 for Remark
+// 4 (160: of t - 1 it keeps u, two planes updated in place, and forms F(u) again).
+// 4096 x 4096 FP32, two kernels -> here, us a step: Remark 1 375 -> 206 (0.91 of
+// the copy bandwidth), 2 330 -> 217, 4 489 -> 309 (0.74: three quarters of it
+// arithmetic at 16 warps a SM); 2048 x 2048 FP64 (half the FP64 operations) 1790 ->
+// 878, 1525 -> 780, 2459 -> 1691.
+//
+// Thread t holds unit t - 1 of the strip [x0, x0 + w): the first and the last hold
+// one unit of halo, which they only prepare. Neighbouring runs march in opposite
+// directions, so that the rows both need at a shared boundary are read together.
+struct SpRun {
+    int rows, strips, w;   // rows a run, strips of w columns
+};
+struct SpMarch {   // the block's run: Y0 its first row, d its direction, n its rows
+    int x0, wc, Y0, d, n, ny, walls;
+    template <typename T>
+    __device__ __forceinline__ SpMarch(const SpK<T>& K, const SpRun& r) : ny(K.ny), walls(K.walls) {
+        const int run = blockIdx.x / r.strips, strip = blockIdx.x - run * r.strips;
+        x0 = strip * r.w;
+        wc = min(r.w, K.nx - x0);
+        const int ya = run * r.rows, yb = min(ny, ya + r.rows);
+        n = yb - ya;
+        d = (run & 1) ? 1 : -1;
+        Y0 = d > 0 ? ya : yb - 1;
+    }
+    __device__ __forceinline__ bool ghost(int y) const { return walls && (y < 0 || y >= ny); }
+    __device__ __forceinline__ int row(int y) const { return y < 0 ? y + ny : (y >= ny ? y - ny : y); }
+    __device__ __forceinline__ static int slot(int y) { return (y + 4) & 3; }
+    // ring slot of row y + r as row y's stencil sees it: the wall mirrors it onto y
+    __device__ __forceinline__ int near(int y, int r) const { return slot(ghost(y + r) ? y : y + r); }
+};
+
+constexpr int kSpThreads = 128;   // most threads of a march block, all of a tile block
+
+template <int KIND, typename V, int OCC>
+__global__ void __launch_bounds__(kSpThreads, OCC) sp_march_kernel(const typename Unit<V>::R* __restrict__ gin,
+                                                                   typename Unit<V>::R* __restrict__ gout,
+                                                                   const typename Unit<V>::R* __restrict__ src,
+                                                                   typename Unit<V>::R* __restrict__ uprev, int N,
+                                                                   SpK<typename Unit<V>::R> K, SpRun run) {
+    using U = Unit<V>;
+    __shared__ typename U::E ring[4][kRing<KIND>][kSpThreads];
+    const SpMarch A(K, run);
+    const int t = threadIdx.x, nx = K.nx;
+    const bool in = U::cells * t < A.wc + 2 * U::cells, own = t >= 1 && U::cells * t < A.wc + U::cells;
+    int x = A.x0 + U::cells * (t - 1);
+    x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+    auto load = [&](int y, V (&g)[kQ], V& S) {
+        if (!in || A.ghost(y)) return;
+        const int c = A.row(y) * nx + x;
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) g[i] = U::ld(gin + i * N + c);
+        S = U::ld(src + c);
+    };
+    auto prepare = [&](int y, const V (&g)[kQ], V S, SpMom<V>& m) {
+        if (!in || A.ghost(y)) return;
+        auto& slot = ring[A.slot(y)];
+        sp_moments_of<KIND>(K, g, S, m, [&](int r, V v) { slot[r][t] = U::pack(v); });
+    };
+    V g[kQ], S, gn[kQ], Sn;
+    SpMom<V> m, mn;
+    load(A.Y0 - A.d, gn, Sn);
+    load(A.Y0, g, S);
+    prepare(A.Y0 - A.d, gn, Sn, mn);
+    prepare(A.Y0, g, S, m);
+    load(A.Y0 + A.d, gn, Sn);
+    for (int k = 0; k < A.n; ++k) {
+        const int y = A.Y0 + k * A.d, c = y * nx + x;
+        V upx, upy;
+        if (KIND == 4 && own) {
+            upx = U::ld(uprev + c);
+            upy = U::ld(uprev + N + c);
+        }
+        prepare(y + A.d, gn, Sn, mn);
+        V gx[kQ], Sx;
+        if (k + 1 < A.n) load(y + 2 * A.d, gx, Sx);
+        __syncthreads();
+        if (own) {
+            if constexpr (KIND == 4) {
+                U::st(uprev + c, m.ux);
+                U::st(uprev + N + c, m.uy);
+            }
+            sp_collide<KIND>(K, g, S, m, upx, upy,
+                             [&](int r, int dx, int dy) { return U::at(ring[A.near(y, dy)][r], t, dx); },
+                             SpPush<V>(K, gout, N, x, y));
+        }
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            g[i] = gn[i];
+            gn[i] = gx[i];
+        }
+        S = Sn;
+        Sn = Sx;
+        m = mn;
+    }
+}
+
+// ---- Small domains: several steps in one cooperative launch over tiles ----
+// As step_kernel_tile (lbm_tile.cuh): tiles of at most 128 units, all rows at
+// once, an item's step waiting only for the items within 3 cells. Up to where the
+// marches above fill the GPU, a launch a step costs more than the step.
+struct SpTileArgs {
+    const void *g0, *g1;   // buffer sets: step s reads g0 when s is even
+    const void* src;
+    void* uprev;
+    int N, nitems, nsteps, ulog, wait_limit;
+    const lbm::WorkItem* work;
+    const int* nbr;
+    int *done, *status;
+};
+
+template <int KIND, typename V, int OCC>
+__global__ void __launch_bounds__(kSpThreads, OCC) sp_tile_kernel(const SpTileArgs a, SpK<typename Unit<V>::R> K) {
+    using U = Unit<V>;
+    using R = typename U::R;
+    // (2^u + 2) x (rows + 2) units: at most 34 x 6 over the shapes 2^u x 128 / 2^u
+    constexpr int NR = kRing<KIND> > 0 ? kRing<KIND> : 1;
+    __shared__ typename U::E ring[NR][208];
+    __shared__ int s_bad;
+    const int tid = threadIdx.x, nx = K.nx, ny = K.ny, N = a.N;
+    const int W = (1 << a.ulog) + 2;
+    const R* src = static_cast<const R*>(a.src);
+    R* uprev = static_cast<R*>(a.uprev);
+    for (int s = 0; s < a.nsteps; ++s) {
+        const R* gin = static_cast<const R*>((s & 1) ? a.g1 : a.g0);
+        R* gout = static_cast<R*>(const_cast<void*>((s & 1) ? a.g0 : a.g1));
+        for (int item = blockIdx.x; item < a.nitems; item += gridDim.x) {
+            const lbm::WorkItem wk = a.work[item];
+            if (s > 0 && !lbm::tile_wait(a.done, a.nbr + item * lbm::kMaxTileNbr, s, a.wait_limit, a.status,
+                                         a.done + a.nitems, &s_bad, tid))
+                return;
+            const int nu = wk.dir / U::cells, rows = wk.nrows;
+            const int tx = tid & (W - 3), ty = tid >> a.ulog;
+            const bool act = tx < nu && ty < rows;
+            auto prepare = [&](int ry, int rx, V (&g)[kQ], V& S, SpMom<V>& m) {   // unit rx of row ry, from -1
+                int x = wk.x0 + rx * U::cells, y = wk.ystart + ry;
+                x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+                if (K.walls) y = y < 0 ? 0 : (y >= ny ? ny - 1 : y);   // the wall mirrors its row
+                else y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+                const int c = y * nx + x, at = (ry + 1) * W + rx + 1;
+#pragma unroll
+                for (int i = 0; i < kQ; ++i) g[i] = U::ld(gin + i * N + c);
+                S = U::ld(src + c);
+                sp_moments_of<KIND>(K, g, S, m, [&](int r, V v) { ring[r][at] = U::pack(v); });
+            };
+            V g[kQ], S, upx, upy;
+            SpMom<V> m;
+            const int x = wk.x0 + tx * U::cells, y = wk.ystart + ty, c = y * nx + x;
+            if (act) {
+                if (KIND == 4) {
+                    upx = U::ld(uprev + c);
+                    upy = U::ld(uprev + N + c);
+                }
+                prepare(ty, tx, g, S, m);
+            }
+            if constexpr (KIND != 3) {
+                const int ownth = rows << a.ulog, halo = 2 * (nu + 2) + 2 * rows;
+                for (int k = tid >= ownth ? tid - ownth : tid + kSpThreads - ownth; k < halo; k += kSpThreads) {
+                    const int cap = 2 * (nu + 2), q = k - cap;
+                    const int ry = k < cap ? (k < nu + 2 ? -1 : rows) : q >> 1;
+                    const int rx = k < cap ? (k < nu + 2 ? k : k - nu - 2) - 1 : ((q & 1) ? nu : -1);
+                    V gh[kQ], Sh;
+                    SpMom<V> mh;
+                    prepare(ry, rx, gh, Sh, mh);
+                }
+                __syncthreads();
+            }
+            if (act) {
+                if constexpr (KIND == 4) {
+                    U::st(uprev + c, m.ux);
+                    U::st(uprev + N + c, m.uy);
+                }
+                const int at = (ty + 1) * W + tx + 1;
+                sp_collide<KIND>(K, g, S, m, upx, upy,
+                                 [&](int r, int dx, int dy) { return U::at(ring[r], at + dy * W, dx); },
+                                 SpPush<V>(K, gout, N, x, y));
+            }
+            __syncthreads();   // every thread's stores of the step issued, the ring free
+            if (tid == 0 && a.nsteps > 1) {
+                __threadfence();
+                atomicExch(a.done + item, s + 1);
+            }
+        }
+    }
 }
 
 }  // namespace
@@ -692,9 +794,7 @@ struct lbm_sp_ctx {
     long long N = 0;
     void* g[2] = {nullptr, nullptr};
     void* src = nullptr;
-    void* ufield = nullptr;            // Remark 1: u of the current step (2 planes);
-                                       // Remark 4 scheme: u, F(u) at t and t - 1 (2 x 4 planes)
-    int uprev = 0;                     // Remark 4 scheme: which half of ufield holds u at t - 1
+    void* ufield = nullptr;            // Remark 4 scheme: u of the step before (2 planes)
     double* d_tmp = nullptr;           // staging for inputs and outputs
     int cur = 0;
     bool ready = false;
@@ -702,6 +802,20 @@ struct lbm_sp_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     SpConst K{};
+    SpK<float> kf;                     // the step's constants in the arithmetic type
+    SpK<double> kd;
+    int kind = 3;                      // 1, 2, 3: Remarks; 4: the Remark 4 scheme
+    int cells = 1;                     // cells a unit: 2 in FP32 with nx even
+    const void* kernel = nullptr;      // one step a launch: row march, Remark 3 one unit a thread
+    SpRun run{};
+    int threads = kSpThreads;
+    const void* tile = nullptr;        // small domains: several steps a launch (null: not taken)
+    int tile_items = 0, tile_grid = 0, tile_ulog = 0;
+    void* d_tile = nullptr;            // items, neighbours, step counters and abort flag
+    lbm::WorkItem* d_tile_work = nullptr;
+    int* d_tile_nbr = nullptr;
+    int* d_tile_done = nullptr;
+    int* d_status = nullptr;           // set by a bounded wait that ran out
     std::string err;
 };
 
@@ -722,35 +836,168 @@ void sp_release(lbm_sp_ctx* c) {
     cudaFree(c->g[1]);
     cudaFree(c->src);
     cudaFree(c->ufield);
+    cudaFree(c->d_tile);
+    cudaFree(c->d_status);
     cudaFree(c->d_tmp);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
 }
 
-// Remarks 1 and 2: u, then the collision
-template <int M>
-void sp1_enqueue(lbm_sp_ctx* c) {
-    if (c->form == LBM_F64) {
-        const double* gi = static_cast<const double*>(c->g[c->cur]);
-        double* uf = static_cast<double*>(c->ufield);
-        sp1_moments_kernel<M, double><<<blocks(c->N), 256, 0, c->stream>>>(
-            gi, static_cast<const double*>(c->src), c->N, c->K, uf);
-        sp1_step_kernel<M, double><<<blocks(c->N), 256, 0, c->stream>>>(
-            gi, static_cast<double*>(c->g[1 - c->cur]), static_cast<const double*>(c->src), uf, c->N, c->K);
-        return;
+// The step kernels of a model for unit type V, and the resident blocks of 128
+// threads a SM their registers are sized for. The row march holds two rows of
+// populations and a third in flight. Measured at 4096 x 4096, pairs, us a step:
+// Remark 1 220 / 206 / 282 with 4 / 5 / 6 blocks, Remark 2 216 / 217 / 235, Remark 4
+// 330 / 309 / 367 with 3 / 4 / 5; FP64 the same with 2 to 4 (bound by its FP64
+// operations).
+template <typename V>
+void sp_kernels(int kind, const void** step, const void** tile) {
+    constexpr bool f64 = sizeof(typename Unit<V>::R) == 8, pair = Unit<V>::cells == 2;
+    constexpr int m = f64 ? 3 : pair ? 5 : 6, m2 = f64 ? 3 : pair ? 4 : 6, m4 = f64 ? 3 : pair ? 4 : 6;
+    constexpr int o = f64 ? 3 : pair ? 4 : 6;
+    switch (kind) {
+        case 1:
+            *step = (const void*)sp_march_kernel<1, V, m>;
+            *tile = (const void*)sp_tile_kernel<1, V, o>;
+            break;
+        case 2:
+            *step = (const void*)sp_march_kernel<2, V, m2>;
+            *tile = (const void*)sp_tile_kernel<2, V, o>;
+            break;
+        case 4:
+            *step = (const void*)sp_march_kernel<4, V, m4>;
+            *tile = (const void*)sp_tile_kernel<4, V, o>;
+            break;
+        default:
+            *step = (const void*)sp_cell_kernel<V>;
+            *tile = (const void*)sp_tile_kernel<3, V, o>;
     }
-    const float* gi = static_cast<const float*>(c->g[c->cur]);
-    float* uf = static_cast<float*>(c->ufield);
-    if (c->p.nx % 2 == 0) {   // two cells a thread
-        sp1_moments_x2_kernel<M><<<blocks(c->N / 2), 256, 0, c->stream>>>(
-            gi, static_cast<const float*>(c->src), c->N, c->K, uf);
-        sp1_step_x2_kernel<M><<<blocks(c->N / 2), 256, 0, c->stream>>>(
-            gi, static_cast<float*>(c->g[1 - c->cur]), static_cast<const float*>(c->src), uf, c->N, c->K);
-    } else {
-        sp1_moments_kernel<M, float><<<blocks(c->N), 256, 0, c->stream>>>(
-            gi, static_cast<const float*>(c->src), c->N, c->K, uf);
-        sp1_step_kernel<M, float><<<blocks(c->N), 256, 0, c->stream>>>(
-            gi, static_cast<float*>(c->g[1 - c->cur]), static_cast<const float*>(c->src), uf, c->N, c->K);
+}
+
+// Chooses the step kernels and their launch shapes.
+lbm_status sp_plan(lbm_sp_ctx* c) {
+    c->kind = c->p.scheme == LBM_SP_SCHEME_REMARK4 ? 4
+              : c->p.model == LBM_SP_NEARLY_INCOMPRESSIBLE ? 1
+              : c->p.model == LBM_SP_HE_INCOMPRESSIBLE ? 2 : 3;
+    c->kf = sp_consts<float>(c->K, c->p.model);
+    c->kd = sp_consts<double>(c->K, c->p.model);
+    c->cells = c->form == LBM_F32 && c->p.nx % 2 == 0 ? 2 : 1;
+    if (c->form == LBM_F64) sp_kernels<One<double>>(c->kind, &c->kernel, &c->tile);
+    else if (c->cells == 2) sp_kernels<F2>(c->kind, &c->kernel, &c->tile);
+    else sp_kernels<One<float>>(c->kind, &c->kernel, &c->tile);
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    auto slots = [&](const void* k, int threads) {
+        int occ = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, threads, 0);
+        return (long long)sms * (occ > 0 ? occ : 1);
+    };
+    const int units = c->p.nx / c->cells;
+    if (c->kind != 3) {
+        // strips of equal width, at most `threads` - 2 units; run lengths for the
+        // fewest (waves of resident blocks) x (rows + 2 for the prologue)
+        long long best = -1;
+        for (int threads = 64; threads <= kSpThreads; threads += 32) {
+            const int strips = (units + threads - 3) / (threads - 2), w = (units + strips - 1) / strips;
+            const long long target = slots(c->kernel, threads);
+            for (int r = 1; r <= c->p.ny; ++r) {
+                const int rows = (c->p.ny + r - 1) / r, runs = (c->p.ny + rows - 1) / rows;
+                const long long cost = ((long long)strips * runs + target - 1) / target * (rows + 2);
+                if (best < 0 || cost < best) {
+                    best = cost;
+                    c->threads = threads;
+                    c->run = SpRun{rows, strips, w * c->cells};
+                }
+            }
+        }
     }
+    // Tiles, several steps a launch, while every tile is resident at once (FP64:
+    // two rounds): a step of a small domain is the latency of a launch. us a step,
+    // tiles and one launch a step: 64 x 64 Remark 1 FP32 3.0 and 4.2, FP64 6.0 and
+    // 8.8; 256 x 256 3.7 and 6.2, 18.6 and 26.9; 400 x 400 (3 rounds) 8.7 and 6.2,
+    // 50.9 and 49.5.
+    auto count = [&](int u, int r) { return (long long)((units + u - 1) / u) * ((c->p.ny + r - 1) / r); };
+    int U, R;
+    lbm::tile_shape(count, sms, &U, &R);
+    const long long tslots = slots(c->tile, kSpThreads);
+    if (count(8, 16) < count(U, R) && count(U, R) > tslots) {
+        U = 8;
+        R = 16;
+    }
+    if (count(U, R) > (c->form == LBM_F64 ? 2 : 1) * tslots) {
+        c->tile = nullptr;
+        return LBM_OK;
+    }
+    lbm::TileList list;
+    lbm::add_tiles(list, 0, c->p.nx, c->p.ny, c->cells, c->p.bc_y != LBM_BC_BOUNCEBACK, U, R);
+    const size_t wb = (list.items.size() * sizeof(lbm::WorkItem) + 255) & ~size_t(255);
+    const size_t nb = (list.nbr.size() * sizeof(int) + 255) & ~size_t(255);
+    const size_t db = (list.items.size() + 1) * sizeof(int);
+    cudaError_t r = cudaMalloc(&c->d_tile, wb + nb + db);
+    if (r != cudaSuccess) return r == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
+    c->d_tile_work = static_cast<lbm::WorkItem*>(c->d_tile);
+    c->d_tile_nbr = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb);
+    c->d_tile_done = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb + nb);
+    if (cudaMemcpy(c->d_tile_work, list.items.data(), list.items.size() * sizeof(lbm::WorkItem),
+                   cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(c->d_tile_nbr, list.nbr.data(), list.nbr.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+        return LBM_ECUDA;
+    c->tile_items = (int)list.items.size();
+    c->tile_grid = (int)(c->tile_items < tslots ? c->tile_items : tslots);
+    while ((1 << c->tile_ulog) < U) ++c->tile_ulog;
+    return LBM_OK;
+}
+
+// Queues one step.
+cudaError_t sp_step_once(lbm_sp_ctx* c) {
+    const void* in = c->g[c->cur];
+    void* out = c->g[1 - c->cur];
+    int N = (int)c->N;
+    void* k = c->form == LBM_F64 ? (void*)&c->kd : (void*)&c->kf;
+    c->cur ^= 1;
+    if (c->kind == 3) {
+        void* args[] = {&in, &out, &c->src, &N, k};
+        return cudaLaunchKernel(c->kernel, dim3(blocks(c->N / c->cells)), dim3(256), args, 0, c->stream);
+    }
+    void* args[] = {&in, &out, &c->src, &c->ufield, &N, k, &c->run};
+    const int runs = (c->p.ny + c->run.rows - 1) / c->run.rows;
+    return cudaLaunchKernel(c->kernel, dim3(runs * c->run.strips), dim3(c->threads), args, 0, c->stream);
+}
+
+// Queues n steps on tiles as one cooperative launch, after zeroing the step
+// counters and the abort flag.
+cudaError_t sp_step_tiles(lbm_sp_ctx* c, int n) {
+    SpTileArgs a;
+    a.g0 = c->g[c->cur];
+    a.g1 = c->g[1 - c->cur];
+    a.src = c->src;
+    a.uprev = c->ufield;
+    a.N = (int)c->N;
+    a.nitems = c->tile_items;
+    a.nsteps = n;
+    a.ulog = c->tile_ulog;
+    a.wait_limit = lbm::kWaitLimit;
+    a.work = c->d_tile_work;
+    a.nbr = c->d_tile_nbr;
+    a.done = c->d_tile_done;
+    a.status = c->d_status;
+    if (n > 1) {
+        const cudaError_t e = cudaMemsetAsync(a.done, 0, ((size_t)c->tile_items + 1) * sizeof(int), c->stream);
+        if (e != cudaSuccess) return e;
+    }
+    void* args[] = {&a, c->form == LBM_F64 ? (void*)&c->kd : (void*)&c->kf};
+    c->cur ^= n & 1;
+    // one step: no block waits, so the grid need not be resident at once
+    return n > 1 ? cudaLaunchCooperativeKernel(c->tile, dim3(c->tile_grid), dim3(kSpThreads), args, 0, c->stream)
+                 : cudaLaunchKernel(c->tile, dim3(c->tile_grid), dim3(kSpThreads), args, 0, c->stream);
+}
+
+// After a synchronisation: a bounded wait of the tiles that ran out.
+lbm_status sp_device_status(lbm_sp_ctx* c) {
+    if (!c->tile) return LBM_OK;
+    int st = 0;
+    const cudaError_t r = cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    if (r != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) return sp_cuda(c, r, "status read-back");
+    return st == 0 ? LBM_OK : sp_fail(c, LBM_ETIMEOUT, "a bounded device wait ran out in the step kernel");
 }
 
 template <int M>
@@ -803,9 +1050,8 @@ lbm_status lbm_sp_create(const lbm_sp_params* params, int precision, void* cuda_
     if ((r = cudaMalloc(&c->g[0], kQ * c->N * e)) != cudaSuccess ||
         (r = cudaMalloc(&c->g[1], kQ * c->N * e)) != cudaSuccess ||
         (r = cudaMalloc(&c->src, c->N * e)) != cudaSuccess ||
-        ((p.model == LBM_SP_NEARLY_INCOMPRESSIBLE || p.model == LBM_SP_HE_INCOMPRESSIBLE) &&
-         (r = cudaMalloc(&c->ufield, 2 * c->N * e)) != cudaSuccess) ||
-        (p.scheme == LBM_SP_SCHEME_REMARK4 && (r = cudaMalloc(&c->ufield, 8 * c->N * e)) != cudaSuccess) ||
+        (p.scheme == LBM_SP_SCHEME_REMARK4 && (r = cudaMalloc(&c->ufield, 2 * c->N * e)) != cudaSuccess) ||
+        (r = cudaMalloc((void**)&c->d_status, sizeof(int))) != cudaSuccess ||
         (r = cudaMalloc((void**)&c->d_tmp, kQ * c->N * sizeof(double))) != cudaSuccess) {
         sp_release(c);
         delete c;
@@ -819,6 +1065,12 @@ lbm_status lbm_sp_create(const lbm_sp_params* params, int precision, void* cuda_
         sp_release(c);
         delete c;
         return LBM_ECUDA;
+    }
+    const lbm_status st = sp_plan(c);
+    if (st != LBM_OK) {
+        sp_release(c);
+        delete c;
+        return st;
     }
     *out = c;
     return LBM_OK;
@@ -843,21 +1095,10 @@ lbm_status lbm_sp_init(lbm_sp_ctx* c, const double* source_host) {
     if ((r = cudaMemsetAsync(c->g[0], 0, kQ * c->N * sp_elem(c->form), c->stream)) != cudaSuccess)
         return sp_cuda(c, r, "state reset");
     // Remark 4 scheme: u at t = -1 is u at t = 0 = 0
-    c->uprev = 0;
     if (c->p.scheme == LBM_SP_SCHEME_REMARK4 &&
-        (r = cudaMemsetAsync(c->ufield, 0, 8 * c->N * sp_elem(c->form), c->stream)) != cudaSuccess)
+        (r = cudaMemsetAsync(c->ufield, 0, 2 * c->N * sp_elem(c->form), c->stream)) != cudaSuccess)
         return sp_cuda(c, r, "state reset");
-    if (c->p.scheme == LBM_SP_SCHEME_REMARK4) {   // F(u = 0) = F_0 at t = -1
-        const double F0[2] = {c->p.force_x, c->p.force_y};
-        for (int a = 0; a < 2; ++a) {
-            if (c->form == LBM_F64)
-                sp_fill_kernel<double><<<blocks(c->N), 256, 0, c->stream>>>(
-                    static_cast<double*>(c->ufield) + (2 + a) * c->N, F0[a], c->N);
-            else
-                sp_fill_kernel<float><<<blocks(c->N), 256, 0, c->stream>>>(
-                    static_cast<float*>(c->ufield) + (2 + a) * c->N, F0[a], c->N);
-        }
-    }
+    if ((r = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream)) != cudaSuccess) return sp_cuda(c, r, "state reset");
     if ((r = cudaStreamSynchronize(c->stream)) != cudaSuccess) return sp_cuda(c, r, "init");
     if ((r = cudaGetLastError()) != cudaSuccess) return sp_cuda(c, r, "init kernel");
     c->ready = true;
@@ -869,51 +1110,11 @@ lbm_status lbm_sp_step(lbm_sp_ctx* c, int nsteps) {
     if (!c) return LBM_EINVAL;
     if (nsteps < 0) return sp_fail(c, LBM_EINVAL, "nsteps < 0");
     if (!c->ready) return sp_fail(c, LBM_ESTATE, "not initialised");
-    const bool m1 = c->p.model == LBM_SP_NEARLY_INCOMPRESSIBLE, m2 = c->p.model == LBM_SP_HE_INCOMPRESSIBLE;
-    const bool r4 = c->p.scheme == LBM_SP_SCHEME_REMARK4;
-    for (int s = 0; s < nsteps; ++s) {
-        if (r4) {
-            const long long h = 4 * c->N;
-            const int un = 1 - c->uprev;
-            if (c->form == LBM_F64) {
-                const double* fi = static_cast<const double*>(c->g[c->cur]);
-                double* u = static_cast<double*>(c->ufield);
-                sp4_moments_kernel<double><<<blocks(c->N), 256, 0, c->stream>>>(fi, c->N, c->K, u + un * h);
-                sp4_step_kernel<double><<<blocks(c->N), 256, 0, c->stream>>>(
-                    fi, static_cast<double*>(c->g[1 - c->cur]), static_cast<const double*>(c->src), u + un * h,
-                    u + c->uprev * h, c->N, c->K);
-            } else {
-                const float* fi = static_cast<const float*>(c->g[c->cur]);
-                float* u = static_cast<float*>(c->ufield);
-                if (c->p.nx % 2 == 0) {   // two cells a thread
-                    sp4_moments_x2_kernel<<<blocks(c->N / 2), 256, 0, c->stream>>>(fi, c->N, c->K, u + un * h);
-                    sp4_step_x2_kernel<<<blocks(c->N / 2), 256, 0, c->stream>>>(
-                        fi, static_cast<float*>(c->g[1 - c->cur]), static_cast<const float*>(c->src), u + un * h,
-                        u + c->uprev * h, c->N, c->K);
-                } else {
-                    sp4_moments_kernel<float><<<blocks(c->N), 256, 0, c->stream>>>(fi, c->N, c->K, u + un * h);
-                    sp4_step_kernel<float><<<blocks(c->N), 256, 0, c->stream>>>(
-                        fi, static_cast<float*>(c->g[1 - c->cur]), static_cast<const float*>(c->src), u + un * h,
-                        u + c->uprev * h, c->N, c->K);
-                }
-            }
-            c->uprev = un;
-        } else if (m1) {
-            sp1_enqueue<1>(c);
-        } else if (m2) {
-            sp1_enqueue<2>(c);        } else if (c->form == LBM_F64)
-            sp_step_kernel<double><<<blocks(c->N), 256, 0, c->stream>>>(
-                static_cast<const double*>(c->g[c->cur]), static_cast<double*>(c->g[1 - c->cur]),
-                static_cast<const double*>(c->src), c->N, c->K);
-        else if (c->p.nx % 2 == 0)   // two cells a thread
-            sp_step_x2_kernel<<<blocks(c->N / 2), 256, 0, c->stream>>>(
-                static_cast<const float*>(c->g[c->cur]), static_cast<float*>(c->g[1 - c->cur]),
-                static_cast<const float*>(c->src), c->N, c->K);
-        else
-            sp_step_kernel<float><<<blocks(c->N), 256, 0, c->stream>>>(
-                static_cast<const float*>(c->g[c->cur]), static_cast<float*>(c->g[1 - c->cur]),
-                static_cast<const float*>(c->src), c->N, c->K);
-        c->cur ^= 1;
+    for (int s = 0; s < nsteps;) {
+        const int n = c->tile ? (nsteps - s < 256 ? nsteps - s : 256) : 1;
+        const cudaError_t e = c->tile ? sp_step_tiles(c, n) : sp_step_once(c);
+        if (e != cudaSuccess) return sp_cuda(c, e, "step kernel");
+        s += n;
     }
     c->time += nsteps;
     const cudaError_t r = cudaGetLastError();
@@ -949,7 +1150,7 @@ lbm_status lbm_sp_get_fields(lbm_sp_ctx* c, unsigned mask, double* host_out) {
                              c->stream)) != cudaSuccess)
         return sp_cuda(c, r, "fields read-back");
     if ((r = cudaStreamSynchronize(c->stream)) != cudaSuccess) return sp_cuda(c, r, "fields");
-    return LBM_OK;
+    return sp_device_status(c);
 }
 
 lbm_status lbm_sp_get_populations(lbm_sp_ctx* c, double* host_g) {
@@ -973,7 +1174,7 @@ lbm_status lbm_sp_get_populations(lbm_sp_ctx* c, double* host_g) {
     if ((r = cudaMemcpyAsync(host_g, c->d_tmp, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
         return sp_cuda(c, r, "populations read-back");
     if ((r = cudaStreamSynchronize(c->stream)) != cudaSuccess) return sp_cuda(c, r, "populations");
-    return LBM_OK;
+    return sp_device_status(c);
 }
 
 const char* lbm_sp_last_error(const lbm_sp_ctx* c) { return c ? c->err.c_str() : "null context"; }

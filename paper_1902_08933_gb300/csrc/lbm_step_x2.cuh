@@ -522,12 +522,6 @@ __global__ void __launch_bounds__(TX, X2Occ<FORM, TX>::value) step_kernel_x2(con
     x2_item<FORM, MON>(a, blockIdx.x, smem_raw, threadIdx.x, 0, 0, TX);
 }
 
-__device__ __forceinline__ int ld_acquire_gpu(const int* p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // ---------------------------------------------------------------------------
 // Several steps of one plan of work items in one persistent launch (the
 // LBM_PIPELINE_PERSISTENT plan of a context whose items all fit on the GPU at

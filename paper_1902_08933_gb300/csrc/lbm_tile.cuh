@@ -319,37 +319,9 @@ __global__ void __launch_bounds__(kTileThreads, OCC) step_kernel_tile(const Step
                 inst = wk.inst;
                 C.load(a.inst[inst]);
             }
-            if (s > 0) {
-                if (tid < 32) {
-                    int ok = 1;
-                    const int n = tid < kMaxTileNbr ? a.nbr[item * kMaxTileNbr + tid] : -1;
-                    if (n >= 0) {
-                        const int need = s + a.wait_extra;
-                        ok = 0;
-                        for (int it = 0; it < a.wait_limit; ++it) {
-                            if (ld_acquire_gpu(a.done + n) >= need) {
-                                ok = 1;
-                                break;
-                            }
-                            if (it >= 256) {   // neighbours are within a step of each other: rarely
-                                if (*reinterpret_cast<volatile int*>(abort_flag)) break;
-                                __nanosleep(64);
-                            }
-                        }
-                        __threadfence();
-                    }
-                    const unsigned bad = __ballot_sync(0xffffffffu, !ok);
-                    if (tid == 0) {
-                        if (bad) {
-                            atomicExch(a.status, kStatusTimeout);
-                            atomicExch(abort_flag, 1);
-                        }
-                        s_bad = bad != 0;
-                    }
-                }
-                __syncthreads();
-                if (s_bad) return;
-            }
+            if (s > 0 && !tile_wait(a.done, a.nbr + item * kMaxTileNbr, s + a.wait_extra, a.wait_limit, a.status,
+                                    abort_flag, &s_bad, tid))
+                return;
             if constexpr (PAIR) tile_item_x2<FORM>(a, C, wk, a.tile_ulog, sm, tid, (s & 1) != 0);
             else tile_item_1<FORM>(a, C, wk, a.tile_ulog, sm, tid, (s & 1) != 0);
             __syncthreads();   // every thread's stores of the step issued, the rings free
