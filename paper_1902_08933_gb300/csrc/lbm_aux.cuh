@@ -92,38 +92,37 @@ __global__ void phi_pass(const AuxArgs a) {
     }
 }
 
-template <typename R>
-__device__ __forceinline__ void gather(const double* f, int nx, int ny, int walls, int x, int y,
-                                       Nbr<R>& nb) {
-    for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-            int yy = y + dy, xx = x + dx;
-            xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-            if (walls) yy = yy < 0 ? -1 - yy : (yy >= ny ? 2 * ny - 1 - yy : yy);
-            else yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
-            nb.z[dy + 1][dx + 1] = R(f[yy * nx + xx]);
-        }
+// 3x3 neighbourhood of a field (x periodic; y periodic or mirrored at walls)
+template <typename T>
+__device__ __forceinline__ void gather(const T* f, int nx, int ny, int walls, int x, int y, Nbr<double>& nb) {
+    const int xs[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
+    const int ys[3] = {y == 0 ? (walls ? 0 : ny - 1) : y - 1, y, y == ny - 1 ? (walls ? ny - 1 : 0) : y + 1};
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) nb.z[dy][dx] = double(f[ys[dy] * nx + xs[dx]]);
 }
 
 template <int FORM>
 __global__ void mu_pass(const AuxArgs a) {
-    using R = double;
-    Consts<R> C;
+    Consts<double> C;
     C.load(a.inst[a.instance]);
     const int n = C.nx * C.ny;
     for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n; cell += gridDim.x * blockDim.x) {
-        Nbr<R> nb;
+        Nbr<double> nb;
         gather(a.tmp_phi, C.nx, C.ny, C.walls, cell % C.nx, cell / C.nx, nb);
-        a.tmp_mu[cell] = double(chem_pot(C, nb.z[1][1], nb.lap()));
+        a.tmp_mu[cell] = chem_pot_f64(C, nb);
     }
 }
 
-// Everything one cell's macroscopic stage produces, plus the Laplace-law P of Sec. 4.2.
-template <int FORM>
+// Everything one cell's macroscopic stage produces, plus (PLAP) the Laplace-law P
+// of Sec. 4.2. FIN: also whether every population is finite. Bound by its FP64
+// operations (macroscopic_f64), like the FP64 step: what is not asked for is not
+// formed.
+template <int FORM, bool PLAP, bool FIN>
 __device__ __forceinline__ void cell_fields(const AuxArgs& a, const Consts<double>& C, int cell, double out[7],
                                             bool& finite) {
     using F = Form<FORM>;
-    using R = double;
     using SR = typename F::R;   // the storage form's arithmetic type: the values as loaded
     using AT = typename F::AT;
     PopIO<F> io;
@@ -133,56 +132,50 @@ __device__ __forceinline__ void cell_fields(const AuxArgs& a, const Consts<doubl
     io.S = a.S; io.hs = SR(C.hs); io.ihs = SR(C.ihs); io.gs = SR(C.gs); io.igs = SR(C.igs);
     const int x = cell % C.nx, y = cell / C.nx;
     const long long c = C.base + cell;
-    Nbr<R> nphi, nmu;
+    Nbr<double> nphi, nmu, np;
     gather(a.tmp_phi, C.nx, C.ny, C.walls, x, y, nphi);
     gather(a.tmp_mu, C.nx, C.ny, C.walls, x, y, nmu);
-    Nbr<R> np;
-    const AT* pp = static_cast<const AT*>(a.p_prev) + C.base;
-    for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-            int yy = y + dy, xx = x + dx;
-            xx = xx < 0 ? xx + C.nx : (xx >= C.nx ? xx - C.nx : xx);
-            if (C.walls) yy = yy < 0 ? -1 - yy : (yy >= C.ny ? 2 * C.ny - 1 - yy : yy);
-            else yy = yy < 0 ? yy + C.ny : (yy >= C.ny ? yy - C.ny : yy);
-            np.z[dy + 1][dx + 1] = R(pp[yy * C.nx + xx]);
-        }
-    R g[9];
-    SR hv[9], lo;
-    io.phi_of(c, hv, lo);
-    finite = isfinite(lo);
+    gather(static_cast<const AT*>(a.p_prev) + C.base, C.nx, C.ny, C.walls, x, y, np);
+    double g[9];
+    finite = true;
+    g[0] = 0.0;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        g[i] = R(io.load_g(i, c));   // exact: FP16 or FP32 times a power of two
-        finite = finite && isfinite(g[i]) && isfinite(hv[i]);
+    for (int i = FIN ? 0 : 1; i < 9; ++i) {   // g_0 enters no field
+        g[i] = double(io.load_g(i, c));       // exact: FP16 or FP32 times a power of two
+        if constexpr (FIN) finite = finite && isfinite(g[i]);
     }
-    R gphix, gphiy, gmux, gmuy, gpx, gpy;
-    nphi.grad(gphix, gphiy);
-    nmu.grad(gmux, gmuy);
-    np.grad(gpx, gpy);
-    const R phi = nphi.z[1][1], mu = nmu.z[1][1];
-    const Macro<R> m = macroscopic(C, g, phi, mu, gphix, gphiy, gmux, gmuy, nmu.lap(), gpx, gpy);
-    // P = p_0 - kappa phi lap(phi) + kappa |grad phi|^2 / 2 + p, p_0 = phi psi' - psi (Sec. 4.2)
-    const R psi = C.beta * phi * phi * (phi - R(1)) * (phi - R(1));
-    const R dpsi = R(2) * C.beta * phi * (phi - R(1)) * (R(2) * phi - R(1));
-    const R Plap = (phi * dpsi - psi) - C.kappa * phi * nphi.lap() +
-                   R(0.5) * C.kappa * (gphix * gphix + gphiy * gphiy) + m.p;
-    out[0] = phi; out[1] = m.ux; out[2] = m.uy; out[3] = m.p; out[4] = m.rho; out[5] = mu;
-    out[6] = Plap;
+    if constexpr (FIN) {
+        SR hv[9], lo;
+        io.phi_of(c, hv, lo);
+        finite = finite && isfinite(lo);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) finite = finite && isfinite(hv[i]);
+    }
+    const MacroD m = macroscopic_f64(C, g, nphi, nmu, np);
+    const double phi = nphi.z[1][1];
+    out[0] = phi; out[1] = m.ux.v; out[2] = m.uy.v; out[3] = m.p.v; out[4] = m.rho.v; out[5] = nmu.z[1][1];
+    out[6] = 0.0;
+    if constexpr (PLAP) {
+        // P = p_0 - kappa phi lap(phi) + kappa |grad phi|^2 / 2 + p, p_0 = phi psi' - psi (Sec. 4.2)
+        const double psi = C.beta * phi * phi * (phi - 1.0) * (phi - 1.0);
+        const double dpsi = 2.0 * C.beta * phi * (phi - 1.0) * (2.0 * phi - 1.0);
+        out[6] = (phi * dpsi - psi) - C.kappa6 * phi * lap6(nphi).v +
+                 (0.5 / 144.0) * C.kappa * fmadd(m.Gx, m.Gx, m.Gy * m.Gy).v + m.p.v;
+    }
 }
 
-template <int FORM>
+template <int FORM, bool PLAP>
 __global__ void fields_pass(const AuxArgs a) {
-    using R = double;
-    Consts<R> C;
+    Consts<double> C;
     C.load(a.inst[a.instance]);
     const int n = C.nx * C.ny;
     for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n; cell += gridDim.x * blockDim.x) {
-        R v[7];
+        double v[7];
         bool fin;
-        cell_fields<FORM>(a, C, cell, v, fin);
+        cell_fields<FORM, PLAP, false>(a, C, cell, v, fin);
         int k = 0;
         for (int b = 0; b < 7; ++b)
-            if (a.mask & (1u << b)) a.out[(long long)(k++) * n + cell] = double(v[b]);
+            if (a.mask & (1u << b)) a.out[(long long)(k++) * n + cell] = v[b];
     }
 }
 
@@ -203,19 +196,17 @@ __device__ __forceinline__ double warp_max(double v) {
 
 template <int FORM>
 __global__ void __launch_bounds__(256) diag_pass(const AuxArgs a) {
-    using R = double;
-    Consts<R> C;
+    Consts<double> C;
     C.load(a.inst[a.instance]);
     const int n = C.nx * C.ny;
     double acc[kDiagQuantities];
 #pragma unroll
     for (int q = 0; q < kDiagQuantities; ++q) acc[q] = 0.0;
     for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n; cell += gridDim.x * blockDim.x) {
-        R v[7];
+        double v[7];
         bool fin;
-        cell_fields<FORM>(a, C, cell, v, fin);
-        const double phi = double(v[0]), ux = double(v[1]), uy = double(v[2]);
-        const double rho = double(v[4]), P = double(v[6]);
+        cell_fields<FORM, true, true>(a, C, cell, v, fin);
+        const double phi = v[0], ux = v[1], uy = v[2], rho = v[4], P = v[6];
         const double x = double(cell % C.nx), y = double(cell / C.nx);
         const double uu = ux * ux + uy * uy;
         acc[0] += phi;

@@ -2,6 +2,7 @@
 // Included by lbm_form<N>.cu, which instantiates them for its form.
 #pragma once
 
+#include "lbm.h"
 #include "lbm_aux.cuh"
 #include "lbm_device.cuh"
 #include "lbm_step_tma.cuh"
@@ -333,7 +334,8 @@ cudaError_t launch_fields_t(const AuxArgs& a, int ncells, cudaStream_t s) {
     const int g = grid_for(ncells, 256);
     phi_pass<FORM><<<g, 256, 0, s>>>(a);
     mu_pass<FORM><<<g, 256, 0, s>>>(a);
-    fields_pass<FORM><<<g, 256, 0, s>>>(a);
+    if (a.mask & LBM_FIELD_PLAP) fields_pass<FORM, true><<<g, 256, 0, s>>>(a);
+    else fields_pass<FORM, false><<<g, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
