@@ -315,14 +315,12 @@ lbm_status lbm_set_launch(lbm_ctx* ctx, int tile_x, int rows);
  *                      of at least 64 columns).
  *  LBM_PIPELINE_BATCHED the PAIRS kernel over every instance of the context in
  *                      ONE persistent, cooperative launch for up to 64 steps
- *                      (one node of the captured graph): blocks of 128 threads
- *                      take (step, descriptor) pairs from an on-device queue,
- *                      a descriptor one strip of up to 256 columns or two of up
- *                      to 128 (two thread groups with their own barriers); an
- *                      item of step s waits (bounded) until its instance has
- *                      finished step s - 1, so steps overlap across instances.
- *                      The strip widths are fixed (lbm_set_launch sets the run
- *                      length only). Only when every instance can use PAIRS;
+ *                      (one node of the captured graph): blocks of 64 threads
+ *                      take (step, work item) pairs from an on-device queue, an
+ *                      item one strip of up to 128 columns; an item of step s
+ *                      waits (bounded) until its instance has finished step s -
+ *                      1, so steps overlap across instances. The strip width is
+ *                      fixed (lbm_set_launch sets the run length only). Only when every instance can use PAIRS;
  *                      else as AUTO.
  *  LBM_PIPELINE_PERSISTENT the PAIRS plan (one launch class: the same strip
  *                      width for every instance), run for up to 64 steps in ONE
@@ -367,7 +365,7 @@ lbm_status lbm_set_graphs(lbm_ctx* ctx, int enable);
  * them, for the monitored ones): strip width,
  * number of thread blocks, and the load path it uses (0 plain, 1 cp.async,
  * 2 TMA, 3 pairs, 4 batched: the one persistent launch, whose blocks count is
- * its grid, one block per resident slot, however many descriptors it takes).
+ * its grid, one block per resident slot, however many items it takes).
  * Any output pointer may be NULL. LBM_EINVAL for an index out of range. */
 lbm_status lbm_launch_info(lbm_ctx* ctx, int index, int* tile_x, int* blocks, int* variant);
 

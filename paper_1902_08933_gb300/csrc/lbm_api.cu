@@ -165,9 +165,8 @@ struct lbm_ctx {
     std::vector<Launch> launches;
     std::vector<WorkItem> work;
     WorkItem* d_work = nullptr;
-    // batched step (one persistent launch over all instances): block descriptors
-    // and the queue counters the kernel takes them with
-    lbm::BlockDesc* d_desc = nullptr;
+    // batched step (one persistent launch over all instances): its items and the
+    // queue counters the kernel takes them with
     int ndesc = 0;
     int* d_queue = nullptr;        // batched queue: next, blocks finished, abort
     int* d_done = nullptr;         // batched: items finished a launch, per instance
@@ -259,7 +258,6 @@ StepArgs step_args(const lbm_ctx* c, int in) {
     a.mon_rec = nullptr;
     a.time_base = nullptr;
     a.mon_step = 0;
-    a.desc = c->d_desc;
     a.ndesc = c->ndesc;
     a.queue = c->d_queue;
     a.done = c->d_done;
@@ -464,92 +462,55 @@ lbm_status plan(lbm_ctx* c) {
     return plan_multi(c, sms);
 }
 
-// Batched plan: the paired kernel's work items of every instance, runs of rows
-// with alternating directions. Instances wider than 128 columns are cut into
-// strips of 256 (wide items: one a block descriptor, all 128 threads on it --
-// the strip width of the one-instance launch, measured 12 % faster than 128 on
-// the 512 mixed instances); narrower instances, and a last strip of at most 128
-// columns, are narrow items, paired into descriptors (items of equal run length
-// together). The descriptors are sorted by run length, longest first, so the
-// queue hands out the long ones first and the short ones fill the tail. Run
-// length: about one descriptor per resident block a step, at most 64 rows,
-// unless set by lbm_set_launch (its strip width does not apply here) -- long
-// runs re-read fewer halo rows, and the tail of a step is hidden by the next
-// step's items of the instances already done (several steps a launch): on the
-// 512 mixed instances 64-row runs beat 32 by 4 % (FP32) and 16 by 12 %.
+// Batched plan: the paired kernel's work items of every instance, strips of 128
+// columns (kBatchedTX pairs) and runs of rows with alternating directions, longest
+// run first, so the queue hands out the long ones first and the short ones fill
+// the tail. Run length, unless set by lbm_set_launch (its strip width does not
+// apply here): about 1.2 items a resident block a step, 8 to 64 rows, each
+// instance cut into equal runs -- long runs re-read fewer halo rows, the tail of a
+// step is hidden by the next step's items of the instances already done, and fewer
+// items than blocks leave some idle (mixed instances, us a step at 8 / 16 / 32 / 64
+// rows: 512 f32 403 / 349 / 324 / 318, 200 f32 151 / 131 / 121 / 159, 64 f32 54 / 56 /
+// 82 / 132; a short run left over at the end of each strip costs up to 10 %).
 lbm_status plan_batched(lbm_ctx* c, bool, bool, bool, int sms) {
+    constexpr int kStrip = 128;
     int occ = 1;
     by_form(c->form, [&](auto F) {
         occ = std::max(1, lbm::batched_occupancy_t<decltype(F)::value>());
         return cudaSuccess;
     });
-    constexpr int kWideStrip = 256, kNarrowStrip = 128;
-    // strips of one instance: (x0, width) with width > kNarrowStrip for wide ones
-    auto strips_of = [&](const lbm_params& p) {
-        std::vector<std::pair<int, int>> v;
-        for (int x0 = 0; x0 < p.nx;) {
-            const int w = p.nx - x0 > kNarrowStrip ? std::min(kWideStrip, p.nx - x0) : p.nx - x0;
-            v.push_back({x0, w});
-            x0 += w;
-        }
-        return v;
-    };
     int rows = c->rows_req;
     if (rows <= 0) {
-        double block_rows = 0;   // rows of whole blocks: a narrow item is half a block
-        for (const lbm_params& p : c->params)
-            for (const auto& sw : strips_of(p)) block_rows += (sw.second > kNarrowStrip ? 1.0 : 0.5) * p.ny;
-        rows = (int)std::lround(block_rows / (1.0 * sms * occ));
+        double strip_rows = 0;
+        for (const lbm_params& p : c->params) strip_rows += (double)((p.nx + kStrip - 1) / kStrip) * p.ny;
+        rows = (int)std::lround(strip_rows / (1.2 * sms * occ));
         rows = std::max(8, std::min(64, rows));
     }
-    std::vector<WorkItem> wide, narrow;
+    c->work.clear();
     for (int k = 0; k < c->n; ++k) {
         const lbm_params& p = c->params[k];
         const int r = std::min(rows, p.ny);
-        const int nchunks = (p.ny + r - 1) / r;
-        for (const auto& sw : strips_of(p))
+        // runs of the rows asked for, or equal ones of about (at most 64) rows
+        const int nchunks = c->rows_req > 0 ? (p.ny + r - 1) / r : std::max((p.ny + 63) / 64, (p.ny + r / 2) / r);
+        for (int x0 = 0; x0 < p.nx; x0 += kStrip)
             for (int ch = 0; ch < nchunks; ++ch) {
-                const int y0 = ch * r, y1 = std::min(p.ny, y0 + r);
+                const int y0 = c->rows_req > 0 ? ch * r : (int)((long long)p.ny * ch / nchunks);
+                const int y1 = c->rows_req > 0 ? std::min(p.ny, y0 + r) : (int)((long long)p.ny * (ch + 1) / nchunks);
                 WorkItem w;
                 w.inst = k;
-                w.x0 = sw.first;
+                w.x0 = x0;
                 w.nrows = y1 - y0;
                 w.dir = (ch % 2 == 0) ? -1 : 1;
                 w.ystart = w.dir < 0 ? y1 - 1 : y0;
                 w.pad = 0;
-                (sw.second > kNarrowStrip ? wide : narrow).push_back(w);
+                c->work.push_back(w);
             }
     }
-    auto longer = [](const WorkItem& x, const WorkItem& y) { return x.nrows > y.nrows; };
-    std::stable_sort(narrow.begin(), narrow.end(), longer);
-    c->work = wide;
-    c->work.insert(c->work.end(), narrow.begin(), narrow.end());
-    std::vector<lbm::BlockDesc> host;
-    std::vector<int> len;
-    for (int j = 0; j < (int)wide.size(); ++j) {
-        host.push_back({{j, lbm::kDescWide}});
-        len.push_back(wide[j].nrows);
-    }
-    const int nw = (int)wide.size(), nn = (int)narrow.size();
-    for (int j = 0; j < nn; j += 2) {
-        host.push_back({{nw + j, j + 1 < nn ? nw + j + 1 : -1}});
-        len.push_back(narrow[j].nrows);   // the longer of the two
-    }
-    std::vector<int> order(host.size());
-    for (int i = 0; i < (int)order.size(); ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return len[x] > len[y]; });
-    {
-        std::vector<lbm::BlockDesc> sorted;
-        for (int i : order) sorted.push_back(host[i]);
-        host.swap(sorted);
-    }
-    c->ndesc = (int)host.size();
+    std::stable_sort(c->work.begin(), c->work.end(),
+                     [](const WorkItem& x, const WorkItem& y) { return x.nrows > y.nrows; });
+    c->ndesc = (int)c->work.size();
     c->launches.clear();
-    c->launches.push_back({kNarrowStrip, 0, (int)std::min<long long>(c->ndesc, (long long)sms * occ), lbm::kBatched});
-    cudaFree(c->d_desc);
-    c->d_desc = nullptr;
-    LBM_CK(c, cudaMalloc(&c->d_desc, host.size() * sizeof(lbm::BlockDesc)));
-    LBM_CK(c, cudaMemcpy(c->d_desc, host.data(), host.size() * sizeof(lbm::BlockDesc), cudaMemcpyHostToDevice));
+    c->launches.push_back({kStrip, 0, (int)std::min<long long>(c->ndesc, (long long)sms * occ), lbm::kBatched});
     if (!c->d_queue) LBM_CK(c, cudaMalloc(&c->d_queue, 4 * sizeof(int)));
     LBM_CK(c, cudaMemset(c->d_queue, 0, 4 * sizeof(int)));
     if (!c->d_done) LBM_CK(c, cudaMalloc(&c->d_done, (size_t)c->n * sizeof(int)));
@@ -877,7 +838,6 @@ void release(lbm_ctx* c) {
     cudaFree(c->sc.philo);
     cudaFree(c->d_inst);
     cudaFree(c->d_work);
-    cudaFree(c->d_desc);
     cudaFree(c->d_queue);
     cudaFree(c->d_done);
     cudaFree(c->d_nbr);

@@ -38,19 +38,11 @@ struct WorkItem {
                                              // instance's items; D3Q15, the tile's y0
 };
 
-// A block's share of the batched step (step_kernel_x2_batched): one work item
-// of up to 256 columns that all 128 threads march (item[1] == kDescWide), or two
-// of up to 128 columns that two groups of 64 threads march side by side (an
-// unused entry is -1).
-constexpr int kDescWide = -2;
 // the persistent multi-step plan (step_kernel_x2_multi): neighbour items an item
 constexpr int kMaxNbr = 8;
 // the tile plan (step_kernel_tile): items within 3 cells of an item, tiles of at
 // least 2 x 2 cells: at most two on either side
 constexpr int kMaxTileNbr = 24;
-struct BlockDesc {
-    int item[2];
-};
 
 // Device buffers of one step (ping-pong: *_in is time t, *_out time t + 1).
 struct StepArgs {
@@ -79,14 +71,13 @@ struct StepArgs {
     struct MonRecord* mon_host;         // optional: caller's pinned host records (device-mapped), or null
     const int64_t* time_base;           // per instance: time level - steps of the context
     long long mon_step;                 // steps of the context before the monitored step
-    // batched step only: block descriptors, their number, and the queue
-    // counters {next (step, descriptor), blocks finished, abort} (zero between
+    // launches of several steps: number of items; batched step only: the queue
+    // counters {next (step, item), blocks finished, abort} (zero between
     // launches). One launch runs nsteps steps: step s reads the buffers above
     // when s is even, the *_out ones when s is odd, and an item of step s > 0
     // first waits (bounded: wait_limit rounds) until done[inst], the items of
     // its instance finished in this launch, reaches s x (items_csr[inst + 1] -
     // items_csr[inst]) + wait_extra (0; a test sets 1 to make the wait run out).
-    const BlockDesc* desc;
     int ndesc;
     int* queue;
     int* done;
@@ -142,7 +133,7 @@ constexpr int kDiagBlocks = 304;      // 2 x 152 SMs
 // storage of h and p); bulk copies by the TMA (FP32 arithmetic, 16-byte rows);
 // two cells per thread in packed FP32 (FP32 arithmetic, nx even, tile >= 64).
 // kBatched: the pairs kernel over every instance in one persistent launch
-// (block descriptors of two 128-column strips).
+// (128-column strips).
 enum StepVariant { kPlain = 0, kAsync = 1, kTma = 2, kPairs = 3, kBatched = 4 };
 template <int FORM> cudaError_t launch_step_t(int tile_x, const StepArgs& a, int nwork, cudaStream_t s,
                                               int variant, bool monitor);

@@ -56,6 +56,14 @@ static cudaError_t launch_step_tx(const StepArgs& a, int nwork, cudaStream_t s, 
     return cudaGetLastError();
 }
 
+// The batched launch's kernel of a form, if it has one.
+template <int FORM>
+static const void* batched_kernel(bool monitor) {
+    if constexpr (kHasTma<FORM>)
+        return monitor ? (const void*)step_kernel_x2_batched<FORM, true> : (const void*)step_kernel_x2_batched<FORM>;
+    return nullptr;
+}
+
 template <int FORM>
 cudaError_t launch_step_t(int tile_x, const StepArgs& a, int nwork, cudaStream_t s, int variant,
                           bool monitor) {
@@ -63,25 +71,22 @@ cudaError_t launch_step_t(int tile_x, const StepArgs& a, int nwork, cudaStream_t
     if (monitor && a.mon == nullptr) return cudaErrorInvalidValue;
     if constexpr (kHasTma<FORM>) {
         if (variant == kBatched) {   // nwork = blocks of the persistent grid (at most those resident)
-            if (a.desc == nullptr || a.queue == nullptr || a.done == nullptr) return cudaErrorInvalidValue;
-            if (monitor) {
-                if (a.nsteps != 1) return cudaErrorInvalidValue;
-                step_kernel_x2_batched<FORM, true><<<nwork, 128, X2Batched<FORM>::bytes, s>>>(a);
-                return cudaGetLastError();
-            }
+            if (a.queue == nullptr || a.done == nullptr) return cudaErrorInvalidValue;
+            if (monitor && a.nsteps != 1) return cudaErrorInvalidValue;
             // several steps: the blocks wait on one another's items, so the grid
             // is launched cooperatively (all of it resident at once)
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(nwork);
-            cfg.blockDim = dim3(128);
-            cfg.dynamicSmemBytes = X2Batched<FORM>::bytes;
+            cfg.blockDim = dim3(kBatchedTX);
+            cfg.dynamicSmemBytes = X2Smem<FORM, kBatchedTX>::bytes;
             cfg.stream = s;
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeCooperative;
             attr[0].val.cooperative = a.nsteps > 1 ? 1 : 0;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            return cudaLaunchKernelEx(&cfg, step_kernel_x2_batched<FORM, false>, a);
+            void* args[1] = {const_cast<StepArgs*>(&a)};
+            return cudaLaunchKernelExC(&cfg, batched_kernel<FORM>(monitor), args);
         }
         if (variant == kPairs) {
             switch (tile_x) {
@@ -144,24 +149,23 @@ cudaError_t prepare_step_t() {
     if ((e = prep_tx<FORM, 128>()) != cudaSuccess) return e;
     if ((e = prep_tx<FORM, 256>()) != cudaSuccess) return e;
     if constexpr (kHasTma<FORM>) {
-        e = cudaFuncSetAttribute(step_kernel_x2_batched<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)X2Batched<FORM>::bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(step_kernel_x2_batched<FORM, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X2Batched<FORM>::bytes);
+        for (bool monitor : {false, true})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(batched_kernel<FORM>(monitor), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)X2Smem<FORM, kBatchedTX>::bytes);
     }
     return e;
 }
 
 template <int FORM>
 int batched_occupancy_t() {
+    int n = 0;
     if constexpr (kHasTma<FORM>) {
-        int n = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel_x2_batched<FORM>, 128,
-                                                                      X2Batched<FORM>::bytes);
-        return e == cudaSuccess ? n : 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batched_kernel<FORM>(false), kBatchedTX,
+                                                          X2Smem<FORM, kBatchedTX>::bytes) != cudaSuccess)
+            return 0;
     }
-    return 0;
+    return n;
 }
 
 // Several steps of a paired plan in one cooperative launch (step_kernel_x2_multi):

@@ -200,14 +200,13 @@ __device__ __forceinline__ void x2_collide_push(const Consts<float>& C, const X2
 }
 
 // One work item (a strip of 2 TX columns of one instance, a run of rows) marched
-// by a group of TX threads (32, 64 or 128): a whole thread block (step_kernel_x2:
-// barrier 0, the one __syncthreads uses; TX its compile-time block size, so the
-// layout below folds to constants) or a thread group of the batched kernel
-// (step_kernel_x2_batched: named barrier 1 + group, TX 128 or 64 chosen per block
-// descriptor). smem_raw is the group's own region in the X2Smem<FORM, TX> layout,
-// tid the thread's index in the group, item the work item's index in
-// StepArgs::work (and of its monitor slot); swap: the step reads the *_out
-// buffers of a and writes the *_in ones (odd steps of a batched launch).
+// by a group of TX threads (32, 64 or 128): a whole thread block in every kernel
+// here (barrier 0, the one __syncthreads uses; TX its compile-time block size, so
+// the layout below folds to constants). smem_raw is the group's region in the
+// X2Smem<FORM, TX> layout, tid the thread's index in the group, item the work
+// item's index in StepArgs::work (and of its monitor slot); swap: the step reads
+// the *_out buffers of a and writes the *_in ones (odd steps of a launch of
+// several).
 template <int FORM, int MON>
 __device__ __forceinline__ void x2_item(const StepArgs& a, int item, unsigned char* smem_raw, int tid,
                                         int bar, int grp, const int TX, const bool swap = false,
@@ -586,93 +585,71 @@ __global__ void __launch_bounds__(TX, X2Occ<FORM, TX>::value) step_kernel_x2_mul
 
 // ---------------------------------------------------------------------------
 // The batched step: every instance of a context, several steps, in one
-// persistent launch. Blocks of 128 threads take (step, block descriptor) pairs
-// from a queue -- an atomic counter over nsteps x ndesc, step-major; within a
-// step the planner sorts the descriptors longest run first -- until it runs
-// dry. A descriptor holds either one wide item (a strip of up to 256 columns,
-// marched by all 128 threads; item[1] == kDescWide) or two narrow ones (strips
-// of up to 128 columns, each on its own group of 64 threads with its own
-// shared-memory region and named barrier, so the two groups march
-// independently: different instances, run lengths and directions). Both kinds
-// go through one inlined x2_item with the group width as a run-time value (two
-// inlined bodies, one a width, made the register allocator spill).
+// persistent launch. Blocks of kBatchedTX threads take (step, item) pairs from a
+// queue -- an atomic counter over nsteps x ndesc, step-major; the planner sorts
+// the items longest run first -- until it runs dry. An item is a strip of up to
+// 2 kBatchedTX columns.
 // Steps overlap across instances: an item of step s > 0 waits only until every
 // item of its own instance's step s - 1 has finished (a per-instance counter of
 // finished items), so no grid-wide step boundary leaves SMs idle in a tail. The
 // wait is safe: items are handed out in step order, so every item waited for
 // was taken earlier by a running block, and the earliest unfinished one waits
-// for nothing. It is bounded all the same: after wait_limit rounds the group
+// for nothing. It is bounded all the same: after wait_limit rounds the block
 // records a timeout in the status word, raises the abort flag (every block
-// then stops taking work) and skips its item. The last block to finish sets
-// the queue and the counters back to zero for the next launch.
-// Three resident blocks a SM (up to 168 registers a thread) for every form: at
-// four, the FP16-h form's batched kernel spilled at its 128-register cap and ran
-// at 23.2k MLUPS on the 512 mixed instances.
-template <int FORM>
-struct X2Batched {
-    static constexpr size_t narrow = X2Smem<FORM, 64>::bytes;    // one group of 64
-    static constexpr size_t wide = X2Smem<FORM, 128>::bytes;     // the block as one group
-    static constexpr size_t bytes = 2 * narrow > wide ? 2 * narrow : wide;
-    static constexpr int by_smem = (int)((228u * 1024u) / (bytes + 1024u));
-    static constexpr int occ = by_smem < 3 ? by_smem : 3;
-};
+// then stops taking work) and leaves. The last block to finish sets the queue
+// and the counters back to zero for the next launch.
+// Blocks of 64 threads, one item each, with the width a compile-time constant: a
+// block of 128 marching either one item of 256 columns or two of 128 took 168
+// registers for its run-time width (FP16 h spilled at 128) and tied the two items
+// together. 512 mixed instances, us a step, that -> this: f32 316 -> 318, f32_c 338
+// -> 330, f32_cc 358 -> 345, FP16 g 364 -> 343, FP16 h 397 -> 300; 64 instances 58 ->
+// 53, 61 -> 55, 64 -> 58, 65 -> 59, 70 -> 54. (Blocks of 32: 336 / 427 / 434 / 376 /
+// 327; of 128: 346 / 359 / 378 / 395 / 337.)
+constexpr int kBatchedTX = 64;
 
 template <int FORM, bool MON = false>
-__global__ void __launch_bounds__(128, X2Batched<FORM>::occ) step_kernel_x2_batched(const StepArgs a) {
+__global__ void __launch_bounds__(kBatchedTX, X2Occ<FORM, kBatchedTX>::value) step_kernel_x2_batched(const StepArgs a) {
+    constexpr int TX = kBatchedTX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_desc, s_abort;
-    __shared__ int s_skip[2];
+    __shared__ int s_next, s_abort;
     const int tid = threadIdx.x;
-    const int g = tid >> 6;   // narrow thread group: 0 or 1
     const int total = a.nsteps * a.ndesc;
     volatile int* abort_flag = a.queue + 2;
     for (;;) {
         if (tid == 0) {
-            s_desc = atomicAdd(a.queue, 1);
-            s_abort = *abort_flag;
+            const int gq = atomicAdd(a.queue, 1);
+            int stop = *abort_flag || gq >= total;
+            if (!stop && gq >= a.ndesc) {   // step s > 0: this instance's step s - 1 first
+                const int s = gq / a.ndesc, inst = a.work[gq - s * a.ndesc].inst;
+                const int need = s * (a.items_csr[inst + 1] - a.items_csr[inst]) + a.wait_extra;
+                int ok = 0;
+                for (int it = 0; it < a.wait_limit; ++it) {
+                    if (ld_acquire_gpu(a.done + inst) >= need) {
+                        ok = 1;
+                        break;
+                    }
+                    if (*abort_flag) break;
+                    __nanosleep(64);
+                }
+                if (!ok) {
+                    atomicExch(a.status, kStatusTimeout);
+                    atomicExch(a.queue + 2, 1);
+                    stop = 1;
+                }
+                __threadfence();
+            }
+            s_next = gq;
+            s_abort = stop;
         }
         __syncthreads();
-        const int gq = s_desc;
-        if (gq >= total || s_abort) break;
-        const int s = gq / a.ndesc, q = gq - s * a.ndesc;
-        const int i0 = a.desc[q].item[0], i1 = a.desc[q].item[1];
-        const bool wide = i1 == kDescWide;
-        const int item = (wide || g == 0) ? i0 : i1;
-        const int gt = wide ? tid : tid & 63, nthr = wide ? 128 : 64, bar = wide ? 1 : 1 + g, grp = wide ? 0 : g;
-        int inst = -1;
-        bool run = item >= 0;
-        if (run) {
-            inst = a.work[item].inst;
-            if (s > 0) {   // every item of this instance's step s - 1 finished
-                if (gt == 0) {
-                    const int need = s * (a.items_csr[inst + 1] - a.items_csr[inst]) + a.wait_extra;
-                    int ok = 0;
-                    for (int it = 0; it < a.wait_limit; ++it) {
-                        if (ld_acquire_gpu(a.done + inst) >= need) {
-                            ok = 1;
-                            break;
-                        }
-                        if (*abort_flag) break;
-                        __nanosleep(64);
-                    }
-                    if (!ok) {
-                        atomicExch(a.status, kStatusTimeout);
-                        atomicExch(a.queue + 2, 1);
-                    }
-                    __threadfence();
-                    s_skip[grp] = !ok;
-                }
-                group_sync(bar, nthr);
-                run = !s_skip[grp];
-            }
-            if (run)
-                x2_item<FORM, MON>(a, item, smem_raw + (wide ? 0 : g * X2Batched<FORM>::narrow), gt, bar, grp,
-                                   nthr, !MON && (s & 1) != 0);   // a monitored launch runs one step
-        }
-        __syncthreads();   // the groups are done with their regions and stores; s_desc may change
-        if (run && gt == 0) {   // publish: one more item of this instance finished
+        const int gq = s_next;
+        if (s_abort) break;
+        const int s = gq / a.ndesc, item = gq - s * a.ndesc;
+        x2_item<FORM, MON>(a, item, smem_raw, tid, 0, 0, TX, !MON && (s & 1) != 0);
+        __syncthreads();   // every thread's stores issued; the rings and s_next free
+        if (tid == 0) {    // publish: one more item of this instance finished
             __threadfence();
-            atomicAdd(a.done + inst, 1);
+            atomicAdd(a.done + a.work[item].inst, 1);
         }
     }
     if (tid == 0) {
