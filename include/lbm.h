@@ -327,11 +327,12 @@ lbm_status lbm_set_launch(lbm_ctx* ctx, int tile_x, int rows);
  *                      cooperative launch with one block per work item when
  *                      every item's block fits on the GPU at once (else as
  *                      PAIRS): before step s a block waits (bounded) only for
- *                      the items within reach of its own (3 rows, 2 columns) to
+ *                      the items within reach of its own (3 cells) to
  *                      finish step s - 1, so no grid-wide step boundary remains.
  *  LBM_PIPELINE_AUTO   (default) BATCHED for contexts of several instances that
- *                      all can use it; otherwise PAIRS where available, else
- *                      ASYNC, else TMA, else PLAIN. Contexts too small to fill
+ *                      all can use it; otherwise PAIRS where available (one
+ *                      domain with the built-in launch shape: as PERSISTENT),
+ *                      else ASYNC, else TMA, else PLAIN. Contexts too small to fill
  *                      the GPU with those kernels' row runs (one 512 x 512
  *                      domain in FP32, larger in FP64; every nx even or every
  *                      nx odd) run their unmonitored steps on tiles of at most

@@ -173,7 +173,7 @@ struct lbm_ctx {
     bool multi = false;            // persistent plan: several steps a launch
     long long step_launches = 0;   // kernel launches lbm_step has issued (graph nodes counted)
     int graph_launches = 0;        // kernel nodes of the captured graph
-    int* d_nbr = nullptr;          // persistent plan: neighbour items, kMaxNbr an item
+    int* d_nbr = nullptr;          // persistent plan: neighbour items, kMaxTileNbr an item
     int* d_multi_done = nullptr;   // persistent plan: steps finished per item, then the abort flag
     double* d_mon_multi = nullptr; // persistent plan, every step monitored: [64 steps][items][kMonQ] slots
     int* d_mon_multi_cnt = nullptr;   // ... [64 steps][instances][kMonSub + 1] counters
@@ -296,10 +296,15 @@ int default_tile(int nx) {
     return 32;
 }
 
-int default_tile_pairs(int nx) {   // strip width of the paired kernel (2 columns a thread)
-    if (nx >= 256) return 256;
-    if (nx >= 128) return 128;
-    return 64;
+// Strip width of the paired kernel (2 columns a thread): 256 columns, or 128 where
+// that leaves at least 3 % fewer padded columns (what its halo costs).
+// f32_c, us a step with 256 / 128: 1024 x 4096 118 / 123, 130 x 8000 52 / 60, but 1400 x
+// 1400 (5.5 strips of 256) 66.2 / 63.5, 600 x 1400 37.4 / 31.8, 300 x 4000 60 / 49 (64:
+// 58, 48, 50 for 130, 320, 300 columns).
+int default_tile_pairs(int nx) {
+    if (nx < 128) return 64;
+    const int w256 = (nx + 255) / 256 * 256, w128 = (nx + 127) / 128 * 128;
+    return w256 * 100 <= w128 * 103 ? 256 : 128;
 }
 
 // Load path and strip width of one instance under the context's pipeline mode.
@@ -518,20 +523,33 @@ lbm_status plan_batched(lbm_ctx* c, bool, bool, bool, int sms) {
     return finish_plan(c);
 }
 
-// The persistent plan (LBM_PIPELINE_PERSISTENT): a paired plan of one launch
-// class whose blocks all fit on the GPU at once runs several steps a launch
-// (step_kernel_x2_multi). Neighbour lists: for each item, the other items of its
-// instance whose columns lie within 2 and whose rows lie within 3 of its own
+// The persistent plan (LBM_PIPELINE_PERSISTENT, and LBM_PIPELINE_AUTO for one
+// domain with the built-in launch shape): a paired plan of one launch class whose
+// blocks all fit on the GPU at once runs several steps a launch
+// (step_kernel_x2_multi), so no step ends in a tail of idle SMs. Neighbour lists:
+// for each item, the other items of its instance within 3 cells of its own
 // (periodic where the instance is; the reach of one step of the row march: lead
-// rows 2 ahead, pushes 1 row and 1 column out, the phi halo 2 columns). More
-// than kMaxNbr neighbours, or more items than resident blocks: no persistent
-// launch, the plan runs as PAIRS.
+// rows 2 ahead, the phi halo 2 columns, pushes 1 cell out of cells as far again).
+// More than kMaxTileNbr neighbours, or more items than resident blocks: no
+// persistent launch, the plan runs as PAIRS.
 // steps of one monitored persistent launch (slots and counters are kept per step)
 constexpr int kMultiSteps = 64;
 
+// Buffers of the records of every step of a persistent launch.
+lbm_status multi_monitor(lbm_ctx* c) {
+    if (!c->multi || c->d_mon_multi) return LBM_OK;
+    const size_t items = c->launches[0].count;
+    LBM_CK(c, cudaMalloc(&c->d_mon_multi, (size_t)kMultiSteps * items * lbm::kMonQ * sizeof(double)));
+    LBM_CK(c, cudaMalloc(&c->d_mon_multi_cnt, (size_t)kMultiSteps * c->n * (lbm::kMonSub + 1) * sizeof(int)));
+    LBM_CK(c, cudaMalloc(&c->d_mon_multi_sub,
+                         (size_t)kMultiSteps * c->n * lbm::kMonSub * lbm::kMonQ * sizeof(double)));
+    return LBM_OK;
+}
+
 lbm_status plan_multi(lbm_ctx* c, int sms) {
     c->multi = false;
-    if (c->d3 || c->pipeline != LBM_PIPELINE_PERSISTENT || c->launches.size() != 1 ||
+    const bool by_default = c->pipeline == LBM_PIPELINE_AUTO && c->n == 1 && !c->tile_req && !c->rows_req;
+    if (c->d3 || !(c->pipeline == LBM_PIPELINE_PERSISTENT || by_default) || c->launches.size() != 1 ||
         c->launches[0].variant != lbm::kPairs)
         return LBM_OK;
     const auto& L = c->launches[0];
@@ -555,17 +573,17 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
             if (b0 + sh * n < a1 && a0 < b1 + sh * n) return true;
         return false;
     };
-    std::vector<int> nbr((size_t)L.count * lbm::kMaxNbr, -1);
+    std::vector<int> nbr((size_t)L.count * lbm::kMaxTileNbr, -1);
     for (int k = 0; k < L.count; ++k) {
         const lbm_params& p = c->params[box[k].inst];
         const bool per_y = p.bc_y != LBM_BC_BOUNCEBACK;
         int cnt = 0;
         for (int m = 0; m < L.count; ++m) {
             if (m == k || box[m].inst != box[k].inst) continue;
-            if (!meet(box[k].x0 - 2, box[k].x1 + 2, box[m].x0, box[m].x1, p.nx, true)) continue;
+            if (!meet(box[k].x0 - 3, box[k].x1 + 3, box[m].x0, box[m].x1, p.nx, true)) continue;
             if (!meet(box[k].y0 - 3, box[k].y1 + 3, box[m].y0, box[m].y1, p.ny, per_y)) continue;
-            if (cnt == lbm::kMaxNbr) return LBM_OK;   // too many: no persistent launch
-            nbr[(size_t)k * lbm::kMaxNbr + cnt++] = m;
+            if (cnt == lbm::kMaxTileNbr) return LBM_OK;   // too many: no persistent launch
+            nbr[(size_t)k * lbm::kMaxTileNbr + cnt++] = m;
         }
     }
     cudaFree(c->d_nbr);
@@ -578,15 +596,11 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
     c->d_mon_multi_cnt = nullptr;
     cudaFree(c->d_mon_multi_sub);
     c->d_mon_multi_sub = nullptr;
-    LBM_CK(c, cudaMalloc(&c->d_mon_multi, (size_t)kMultiSteps * L.count * lbm::kMonQ * sizeof(double)));
-    LBM_CK(c, cudaMalloc(&c->d_mon_multi_cnt, (size_t)kMultiSteps * c->n * (lbm::kMonSub + 1) * sizeof(int)));
-    LBM_CK(c, cudaMalloc(&c->d_mon_multi_sub,
-                         (size_t)kMultiSteps * c->n * lbm::kMonSub * lbm::kMonQ * sizeof(double)));
     LBM_CK(c, cudaMalloc(&c->d_nbr, nbr.size() * sizeof(int)));
     LBM_CK(c, cudaMemcpy(c->d_nbr, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice));
     LBM_CK(c, cudaMalloc(&c->d_multi_done, ((size_t)L.count + 1) * sizeof(int)));
     c->multi = true;
-    return LBM_OK;
+    return c->monitor ? multi_monitor(c) : LBM_OK;
 }
 
 // The tile plan (step_kernel_tile, lbm_tile.cuh) of a context under
@@ -1104,7 +1118,7 @@ cudaError_t enqueue_multi(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, in
     if (e != cudaSuccess) return e;
     const bool monitor = host_records != nullptr;
     if (monitor) {
-        if (nsteps > kMultiSteps || !c->d_mon) return cudaErrorInvalidValue;
+        if (nsteps > kMultiSteps || !c->d_mon || !c->d_mon_multi) return cudaErrorInvalidValue;
         e = cudaMemsetAsync(c->d_mon_multi_cnt, 0, (size_t)nsteps * c->n * (lbm::kMonSub + 1) * sizeof(int),
                             c->stream);
         if (e != cudaSuccess) return e;
@@ -1229,10 +1243,6 @@ bool build_graph(lbm_ctx* c) {
             if (e == cudaSuccess) e = cudaEventRecord(c->join[i], c->side[i]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->join[i], 0);
         }
-    } else if (batched_plan(c)) {
-        e = enqueue_batched(c, 0, steps);   // one launch for all the steps
-    } else if (multi_plan(c)) {
-        e = enqueue_multi(c, 0, steps);     // one launch (after the counters' reset) for all the steps
     } else {
         for (int t = 0; t < steps && e == cudaSuccess; ++t) e = enqueue_step(c, t & 1);
     }
@@ -1253,7 +1263,7 @@ bool build_graph(lbm_ctx* c) {
     }
     c->graph = x;
     c->graph_steps = steps;
-    c->graph_launches = nl > 1 ? steps * nl : ((batched_plan(c) || multi_plan(c)) ? 1 : steps * step_kernels(c));
+    c->graph_launches = nl > 1 ? steps * nl : steps * step_kernels(c);
     return true;
 }
 }  // namespace
@@ -1278,8 +1288,9 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
         c->cur ^= n & 1;
         left -= n;
     }
-    // graph replays cover whole multiples of the captured steps from parity 0
-    if (left >= 2 && c->use_graphs) {
+    // graph replays cover whole multiples of the captured steps from parity 0 (a
+    // plan that runs several steps a launch needs none)
+    if (left >= 2 && c->use_graphs && !batched_plan(c) && !multi_plan(c)) {
         if (c->cur == 1) {
             cudaError_t e = enqueue_step(c, 1);
             if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
@@ -1296,7 +1307,7 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
             }
         }
     }
-    while (left > 0 && (batched_plan(c) || multi_plan(c))) {   // the rest in launches of up to 256 steps
+    while (left > 0 && (batched_plan(c) || (multi_plan(c) && left > 1))) {   // launches of up to 256 steps
         const int n = std::min(left, 256);
         cudaError_t e = batched_plan(c) ? enqueue_batched(c, c->cur, n) : enqueue_multi(c, c->cur, n);
         if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
@@ -1397,7 +1408,7 @@ lbm_status lbm_set_monitor(lbm_ctx* c, int enable) {
         LBM_CK(c, cudaMallocHost(&c->h_mon, sizeof(lbm_monitor)));
     }
     c->monitor = enable != 0;
-    return LBM_OK;
+    return enable && !c->plan_dirty ? multi_monitor(c) : LBM_OK;
 }
 
 lbm_status lbm_read_monitor_async(lbm_ctx* c, int instance, lbm_monitor* host_out) {
@@ -1838,7 +1849,8 @@ lbm_status lbm_autotune_shape(lbm_ctx* c, int flags, lbm_launch_shape* out) {
         // graph branches there, one after the other in direct launches
         if (c->cur == 1 && (st = lbm_step(c, 1)) != LBM_OK) break;
         if ((st = lbm_step(c, 2)) != LBM_OK) break;
-        const int nt = std::max(8, c->use_graphs && c->graph ? c->graph_steps : 0);
+        const bool several = tile_plan(c) || batched_plan(c) || multi_plan(c);   // steps a launch
+        const int nt = several ? 64 : std::max(8, c->use_graphs && c->graph ? c->graph_steps : 0);
         float ms = 1e30f;
         for (int rep = 0; rep < 3 && st == LBM_OK; ++rep) {
             cudaEventRecord(e0, c->stream);
@@ -1956,7 +1968,7 @@ lbm_status lbm_inject_batched_wait_timeout(lbm_ctx* c, int rounds) {
     lbm_status st = sticky(c);
     if (st != LBM_OK) return st;
     if (c->plan_dirty && (st = plan(c)) != LBM_OK) return st;
-    if (!batched_plan(c) && !multi_plan(c))
+    if (!batched_plan(c) && !(multi_plan(c) && c->pipeline == LBM_PIPELINE_PERSISTENT))
         return fail(c, LBM_ESTATE, "the context runs neither the batched nor the persistent launch");
     // two steps; every item of the second waits for one finished item (batched)
     // or step (persistent, and the tiles that stand in for the batched launch in

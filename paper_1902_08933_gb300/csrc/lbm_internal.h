@@ -38,10 +38,9 @@ struct WorkItem {
                                              // instance's items; D3Q15, the tile's y0
 };
 
-// the persistent multi-step plan (step_kernel_x2_multi): neighbour items an item
-constexpr int kMaxNbr = 8;
-// the tile plan (step_kernel_tile): items within 3 cells of an item, tiles of at
-// least 2 x 2 cells: at most two on either side
+// Neighbour items listed per item by the plans that run several steps a launch
+// (step_kernel_x2_multi, step_kernel_tile, sp_tile_kernel): the items within 3 cells
+// of it, at most two on either side when items are at least 2 x 2 cells.
 constexpr int kMaxTileNbr = 24;
 
 // Device buffers of one step (ping-pong: *_in is time t, *_out time t + 1).
@@ -82,7 +81,7 @@ struct StepArgs {
     int* queue;
     int* done;
     const int* items_csr;
-    const int* nbr;        // persistent multi-step plan: kMaxNbr neighbour items per item, -1 padded
+    const int* nbr;        // persistent and tile plans: kMaxTileNbr neighbour items per item, -1 padded
     long long set_delta;   // bytes from each *_in array to its *_out array (the same for all)
     int ninst;
     int nsteps;

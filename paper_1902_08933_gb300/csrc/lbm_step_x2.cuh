@@ -525,9 +525,9 @@ __global__ void __launch_bounds__(TX, X2Occ<FORM, TX>::value) step_kernel_x2(con
 // Several steps of one plan of work items in one persistent launch (the
 // LBM_PIPELINE_PERSISTENT plan of a context whose items all fit on the GPU at
 // once): block b owns work item b for every step, and before step s > 0 waits
-// only until each of its neighbour items (a.nbr[b * kMaxNbr ..], -1 padded:
-// the items whose rows and columns lie within the 3 rows and 2 columns one step
-// reads or writes around item b) has finished step s - 1, counted in a.done
+// only until each of its neighbour items (a.nbr[b * kMaxTileNbr ..], -1 padded:
+// the items within 3 cells of item b: one step reads h up to 2 cells outside it,
+// which cells up to 3 outside have pushed) has finished step s - 1, counted in a.done
 // (zeroed before the launch). Those are exactly the items that read what step
 // s of b overwrites and wrote what it reads, so no grid-wide step boundary is
 // needed; neighbours stay within one step of each other. The launch is
@@ -539,42 +539,23 @@ __global__ void __launch_bounds__(TX, X2Occ<FORM, TX>::value) step_kernel_x2(con
 template <int FORM, int TX, bool MON = false>
 __global__ void __launch_bounds__(TX, X2Occ<FORM, TX>::value) step_kernel_x2_multi(const StepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_item, s_step;
     const int b = blockIdx.x, tid = threadIdx.x;
     int* abort_flag = a.done + a.ndesc;
-    for (int s = 0; s < a.nsteps; ++s) {
-        if (s > 0) {
-            if (tid < 32) {
-                int ok = 1;
-                if (tid < kMaxNbr) {
-                    const int n = a.nbr[b * kMaxNbr + tid];
-                    if (n >= 0) {
-                        const int need = s + a.wait_extra;
-                        ok = 0;
-                        for (int it = 0; it < a.wait_limit; ++it) {
-                            if (ld_acquire_gpu(a.done + n) >= need) {
-                                ok = 1;
-                                break;
-                            }
-                            if (*reinterpret_cast<volatile int*>(abort_flag)) break;
-                            __nanosleep(64);
-                        }
-                        __threadfence();
-                    }
-                }
-                const unsigned bad = __ballot_sync(0xffffffffu, !ok);
-                if (tid == 0) {
-                    if (bad) {
-                        atomicExch(a.status, kStatusTimeout);
-                        atomicExch(abort_flag, 1);
-                    }
-                    s_bad = bad != 0;
-                }
-            }
-            __syncthreads();
-            if (s_bad) return;
+    for (int s0 = 0; s0 < a.nsteps; ++s0) {
+        // item and step through shared memory: as a block index and a loop counter
+        // they made the compiler keep what follows from them in registers across
+        // the item (FP16 h: 168 bytes of spills a thread, 155 us a step for 115)
+        if (tid == 0) {
+            s_item = b;
+            s_step = s0;
         }
-        x2_item<FORM, MON ? 2 : 0>(a, b, smem_raw, tid, 0, 0, TX, (s & 1) != 0, s);
+        __syncthreads();
+        const int item = *(volatile int*)&s_item, s = *(volatile int*)&s_step;
+        if (s > 0 && !tile_wait(a.done, a.nbr + b * kMaxTileNbr, s + a.wait_extra, a.wait_limit, a.status, abort_flag,
+                                &s_bad, tid))
+            return;
+        x2_item<FORM, MON ? 2 : 0>(a, item, smem_raw, tid, 0, 0, TX, (s & 1) != 0, s);
         __syncthreads();   // every thread's stores of step s issued
         if (!MON && tid == 0) {   // (the monitored item publishes itself, before its monitor tree)
             __threadfence();
