@@ -1077,6 +1077,10 @@ struct StepOcc {
                                      ? (sizeof(typename Form<FORM>::R) == 8 ? 384 : 1024) / TX : 1;
 };
 
+// Forms whose one-cell kernel prefetches the next row's g into L2.
+template <int FORM>
+constexpr bool kL2Prefetch = sizeof(typename Form<FORM>::R) == 4 && !Form<FORM>::g16;
+
 // The asynchronous variant needs 4- or 8-byte elements for h and p (cp.async).
 template <int FORM>
 constexpr bool kAsyncOk = sizeof(typename Form<FORM>::R) == 4 && !Form<FORM>::h16;
@@ -1284,6 +1288,31 @@ __global__ void __launch_bounds__(TX, StepOcc<FORM, TX>::value) step_kernel(cons
                              colm, colp, nphi, nmu, np, h, g, pux, puy, mon);
     };
 
+    // L2 prefetch of the g and phi*u row segments of collision row Yp (the next
+    // one), one bulk prefetch a lane over the 16-byte-aligned interior of each, as
+    // in the paired kernel. For states larger than L2 (a.l2_prefetch): 1023 x 2047
+    // f32 95.9 -> 88.5 us a step, 1399 x 4001 240 -> 221; in L2 it is only work (517 x
+    // 1033 29.2 -> 30.2), and with FP16 g the step waits for something else (f32_h16
+    // 86 -> 90).
+    auto l2_prefetch_row = [&](int Yp) {
+        if (tid >= 11 || ghost(Yp)) return;
+        const long long c = (long long)rowoff(Yp) + x0;
+        const char* src;
+        unsigned bytes;
+        if (tid < 9) {
+            src = reinterpret_cast<const char*>(io.gin + (long long)tid * S + c);
+            bytes = (unsigned)(w * sizeof(typename F::GT));
+        } else {
+            src = reinterpret_cast<const char*>(phiu + (long long)(tid - 9) * S + c);
+            bytes = (unsigned)(w * sizeof(AT));
+        }
+        const uintptr_t p0 = reinterpret_cast<uintptr_t>(src);
+        const uintptr_t lo = (p0 + 15u) & ~uintptr_t(15), hi = (p0 + bytes) & ~uintptr_t(15);
+        if (hi > lo)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((unsigned)(hi - lo))
+                         : "memory");
+    };
+
     const int Y0 = wk.ystart;
     // Prologue: phi rows Y0-2d .. Y0+d, mu rows Y0-d .. Y0, p rows Y0-d .. Y0.
     // Rows inside the domain first: a ghost row (beyond a wall, on either side
@@ -1312,6 +1341,8 @@ __global__ void __launch_bounds__(TX, StepOcc<FORM, TX>::value) step_kernel(cons
             pux = R(phiu[c]);
             puy = R(phiu[S + c]);
         }
+        if constexpr (kL2Prefetch<FORM>)
+            if (a.l2_prefetch && k + 1 < wk.nrows) l2_prefetch_row(Y + d);
         if constexpr (ASYNC) {
             lead_row_async(Y + 2 * d);
         } else {

@@ -87,6 +87,7 @@ struct StepArgs {
     int nsteps;
     int wait_limit;
     int wait_extra;
+    int l2_prefetch;       // one-cell kernel: prefetch rows into L2 (the state is larger than L2)
     int tile_ulog;         // tile plan: log2 of the units (cells or pairs) of a tile's row
 };
 
