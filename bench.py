@@ -321,7 +321,7 @@ def kernel_run(args):
         if model == 4:
             spcfg.update(scheme=1, force_x=1e-6, drag_lin=1e-3, drag_quad=0.1)
         sim = lbm.SourceFlow(spcfg, form, stream=stream.cuda_stream, source=src)
-        bpl = {0: 76, 1: 132, 2: 132, 4: 160}[model] * (2 if form == "f64" else 1)
+        bpl = {0: 76, 1: 76, 2: 76, 4: 92}[model] * (2 if form == "f64" else 1)
     if args.pipeline != "auto" and args.kernel_run in ("batched", "bubble3d"):
         lbm.lbm_set_pipeline(sim.ctx, getattr(lbm, "LBM_PIPELINE_" + args.pipeline.upper()))
     shape = None
@@ -411,12 +411,12 @@ def main():
     d = sim.diagnostics()
     sim.close()
     value = world * cells * args.steps / (ms * 1e-3) / 1e6
-    # per step: a launch of the persistent plan runs up to 64 steps, and its
+    # per step: a launch of the persistent plan runs up to 256 steps, and its
     # algorithmic bytes over its duration is this same rate
     per_step_s = ms * 1e-3 / args.steps
     achieved = ALGO_BYTES_PER_LUP[args.form] * cells / per_step_s / 1e9
     achieved_form = BYTES_PER_LUP[args.form] * cells / per_step_s / 1e9
-    persistent = (shape or {}).get("pipeline") == "persistent" or args.pipeline == "persistent"
+    persistent = variant == "pairs" and n_launches < args.steps   # no graphs: their nodes count as launches
     traffic = traffic_record(args.form + ("/persistent" if persistent else ""))
     result = {
         "metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": world,
@@ -605,16 +605,15 @@ def side_legs(args, lbm, wl, cfg, phi0, stream, hbm_peak):
     n = 4096
     src = np.ascontiguousarray(1e-4 * np.sin(2 * np.pi * np.arange(n) / n)[None, :] * np.ones((n, 1)))
     sp = {"workload": "source_flow_4096x4096", "cells": n * n}
-    # Remark 1 (two kernels a step): (9 + 1) reads + 2 writes of u, then
-    # 9 + 1 + 2 reads and 9 writes, so 264 / 132 bytes a cell
+    # one kernel a step: 9 populations and S read, 9 populations written, 76 / 152
+    # bytes a cell; the Remark 4 scheme also reads and writes the kept u, 92 / 184
     sp1 = {"workload": "source_flow_remark1_4096x4096", "cells": n * n}
     sp2 = {"workload": "source_flow_remark2_4096x4096", "cells": n * n}   # Remark 2: as Remark 1
-    # Remark 4 scheme with a drag force (two kernels): 9 reads and 4 writes (u, F),
-    # then 9 + 1 + 4 + 4 reads (f, S, u and F at t and t - 1) and 9 writes: 320 / 160
+    # Remark 4 scheme with a drag force
     sp4 = {"workload": "source_flow_remark4_drag_4096x4096", "cells": n * n}
     legs = {0: sp, 1: sp1, 2: sp2, 4: sp4}
-    for model, form, bpl in ((0, "f64", 152), (0, "f32", 76), (1, "f64", 264), (1, "f32", 132),
-                             (2, "f64", 264), (2, "f32", 132), (4, "f64", 320), (4, "f32", 160)):
+    for model, form, bpl in ((0, "f64", 152), (0, "f32", 76), (1, "f64", 152), (1, "f32", 76),
+                             (2, "f64", 152), (2, "f32", 76), (4, "f64", 184), (4, "f32", 92)):
         spcfg = dict(nx=n, ny=n, nu=0.1, model=model if model in (1, 2) else 0)
         if model == 4:
             spcfg.update(scheme=1, force_x=1e-6, drag_lin=1e-3, drag_quad=0.1)

@@ -220,7 +220,7 @@ lbm_status lbm_step_monitored(lbm_ctx* ctx, int nsteps, lbm_monitor* host_record
  * memory: host_records holds nsteps x n_instances records (pinned host memory
  * the device can write), record [k * n_instances + instance] that of step k of
  * the call (time = lbm_time before the call + k). Under the persistent plan
- * (LBM_PIPELINE_PERSISTENT) up to 64 steps run in one launch and the last
+ * (LBM_PIPELINE_PERSISTENT, or AUTO where it takes it) up to 64 steps run in one launch and the last
  * block of each step to finish reduces that step's sums while the others are
  * already on later steps, so the records cost little more than the sums;
  * otherwise each step is a monitored launch as in lbm_step_monitored. The
@@ -314,16 +314,17 @@ lbm_status lbm_set_launch(lbm_ctx* ctx, int tile_x, int rows);
  *                      (FP32-arithmetic forms, instances with nx even, strips
  *                      of at least 64 columns).
  *  LBM_PIPELINE_BATCHED the PAIRS kernel over every instance of the context in
- *                      ONE persistent, cooperative launch for up to 64 steps
- *                      (one node of the captured graph): blocks of 64 threads
+ *                      ONE persistent, cooperative launch for up to 256 steps:
+ *                      blocks of 64 threads
  *                      take (step, work item) pairs from an on-device queue, an
  *                      item one strip of up to 128 columns; an item of step s
  *                      waits (bounded) until its instance has finished step s -
  *                      1, so steps overlap across instances. The strip width is
- *                      fixed (lbm_set_launch sets the run length only). Only when every instance can use PAIRS;
+ *                      fixed (lbm_set_launch sets the run length only). Only
+ *                      when every instance can use PAIRS;
  *                      else as AUTO.
  *  LBM_PIPELINE_PERSISTENT the PAIRS plan (one launch class: the same strip
- *                      width for every instance), run for up to 64 steps in ONE
+ *                      width for every instance), run for up to 256 steps in ONE
  *                      cooperative launch with one block per work item when
  *                      every item's block fits on the GPU at once (else as
  *                      PAIRS): before step s a block waits (bounded) only for
