@@ -1472,7 +1472,7 @@ static lbm_status fields_to_device(lbm_ctx* c, int instance, unsigned mask, doub
     a.out = dev_out;
     a.mask = mask;
     cudaError_t e = by_form(c->form, [&](auto F) {
-        return lbm::launch_fields_t<decltype(F)::value>(a, p.nx * p.ny, c->stream);
+        return lbm::launch_fields_t<decltype(F)::value>(a, p.nx, p.ny, c->stream);
     });
     if (e != cudaSuccess) return cuda_fail(c, e, "fields kernels");
     return LBM_OK;

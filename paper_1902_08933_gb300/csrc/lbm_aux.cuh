@@ -68,7 +68,8 @@ __global__ void init_kernel(const StepArgs a, const double* __restrict__ phi0, i
 
 // ---------------------------------------------------------------------------
 // Macroscopic fields and diagnostics of one instance, in three passes over
-// global memory (phi, then mu, then everything else) -- off the hot loop. They
+// global memory (phi, then mu, then everything else; the fields of small domains
+// in one, fields_tile) -- off the hot loop. They
 // compute in FP64 whatever the storage form: the stored populations convert to
 // FP64 exactly (phi of the conservative forms from its two-float h_0 to about
 // 2^-48), so the fields, sums and the Laplace pressure P of Sec. 4.2 measure the
@@ -120,7 +121,8 @@ __global__ void mu_pass(const AuxArgs a) {
 // operations (macroscopic_f64), like the FP64 step: what is not asked for is not
 // formed.
 template <int FORM, bool PLAP, bool FIN>
-__device__ __forceinline__ void cell_fields(const AuxArgs& a, const Consts<double>& C, int cell, double out[7],
+__device__ __forceinline__ void cell_fields(const AuxArgs& a, const Consts<double>& C, int x, int y,
+                                            const Nbr<double>& nphi, const Nbr<double>& nmu, double out[7],
                                             bool& finite) {
     using F = Form<FORM>;
     using SR = typename F::R;   // the storage form's arithmetic type: the values as loaded
@@ -130,11 +132,8 @@ __device__ __forceinline__ void cell_fields(const AuxArgs& a, const Consts<doubl
     io.h0in = static_cast<const float2*>(a.h0);
     io.gin = static_cast<const typename F::GT*>(a.g);
     io.S = a.S; io.hs = SR(C.hs); io.ihs = SR(C.ihs); io.gs = SR(C.gs); io.igs = SR(C.igs);
-    const int x = cell % C.nx, y = cell / C.nx;
-    const long long c = C.base + cell;
-    Nbr<double> nphi, nmu, np;
-    gather(a.tmp_phi, C.nx, C.ny, C.walls, x, y, nphi);
-    gather(a.tmp_mu, C.nx, C.ny, C.walls, x, y, nmu);
+    const long long c = C.base + y * C.nx + x;
+    Nbr<double> np;
     gather(static_cast<const AT*>(a.p_prev) + C.base, C.nx, C.ny, C.walls, x, y, np);
     double g[9];
     finite = true;
@@ -164,6 +163,23 @@ __device__ __forceinline__ void cell_fields(const AuxArgs& a, const Consts<doubl
     }
 }
 
+// The same with phi and mu from the scratch planes.
+template <int FORM, bool PLAP, bool FIN>
+__device__ __forceinline__ void cell_fields_at(const AuxArgs& a, const Consts<double>& C, int cell, double out[7],
+                                               bool& finite) {
+    const int x = cell % C.nx, y = cell / C.nx;
+    Nbr<double> nphi, nmu;
+    gather(a.tmp_phi, C.nx, C.ny, C.walls, x, y, nphi);
+    gather(a.tmp_mu, C.nx, C.ny, C.walls, x, y, nmu);
+    cell_fields<FORM, PLAP, FIN>(a, C, x, y, nphi, nmu, out, finite);
+}
+
+__device__ __forceinline__ void put_fields(const AuxArgs& a, int n, int cell, const double v[7]) {
+    int k = 0;
+    for (int b = 0; b < 7; ++b)
+        if (a.mask & (1u << b)) a.out[(long long)(k++) * n + cell] = v[b];
+}
+
 template <int FORM, bool PLAP>
 __global__ void fields_pass(const AuxArgs a) {
     Consts<double> C;
@@ -172,11 +188,71 @@ __global__ void fields_pass(const AuxArgs a) {
     for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n; cell += gridDim.x * blockDim.x) {
         double v[7];
         bool fin;
-        cell_fields<FORM, PLAP, false>(a, C, cell, v, fin);
-        int k = 0;
-        for (int b = 0; b < 7; ++b)
-            if (a.mask & (1u << b)) a.out[(long long)(k++) * n + cell] = v[b];
+        cell_fields_at<FORM, PLAP, false>(a, C, cell, v, fin);
+        put_fields(a, n, cell, v);
     }
+}
+
+// The three passes in one launch, a block a tile of kFieldTX x kFieldTY cells: phi of
+// the tile and a halo of 2 cells and mu of a halo of 1 in shared memory, mirrored at
+// walls as gather() does. Three launches are most of the time of a small domain
+// (64 x 64 20.6 -> 10.4 us, 150 x 150 20.6 -> 16.5); a large one is bound by its FP64
+// operations, of which the halo adds 0.4 of the mu of a cell, and takes the passes
+// (launch_fields_t). 16 x 8 cells: enough blocks at the sizes this serves.
+constexpr int kFieldTX = 16, kFieldTY = 8;
+template <int FORM, bool PLAP>
+__global__ void __launch_bounds__(kFieldTX * kFieldTY) fields_tile(const AuxArgs a) {
+    using F = Form<FORM>;
+    using R = typename F::R;
+    constexpr int PW = kFieldTX + 4, MW = kFieldTX + 2;
+    __shared__ double s_phi[(kFieldTY + 4) * PW], s_mu[(kFieldTY + 2) * MW];
+    Consts<double> C;
+    C.load(a.inst[a.instance]);
+    const int nx = C.nx, ny = C.ny, walls = C.walls;
+    const int strips = (nx + kFieldTX - 1) / kFieldTX;
+    const int x0 = (int)blockIdx.x % strips * kFieldTX, y0 = (int)blockIdx.x / strips * kFieldTY;
+    const int w = min(kFieldTX, nx - x0), rows = min(kFieldTY, ny - y0);
+    auto wrapx = [nx](int x) { return x < 0 ? x + nx : (x >= nx ? x - nx : x); };
+    auto rowg = [ny, walls](int y) {
+        if (walls) return y < 0 ? -1 - y : (y >= ny ? 2 * ny - 1 - y : y);
+        return y < 0 ? y + ny : (y >= ny ? y - ny : y);
+    };
+    auto nbr = [](const double* f, int j, int width, Nbr<double>& n) {
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) n.z[dy][dx] = f[j + (dy - 1) * width + dx - 1];
+    };
+    PopIO<F> io;
+    io.hin = static_cast<const typename F::HT*>(a.h);
+    io.h0in = static_cast<const float2*>(a.h0);
+    io.S = a.S; io.hs = R(C.hs); io.ihs = R(C.ihs);
+    for (int k = threadIdx.x; k < (rows + 4) * PW; k += kFieldTX * kFieldTY) {
+        const int ry = k / PW - 2, rx = k % PW - 2;
+        if (rx >= w + 2) continue;
+        R hv[9], lo;
+        const R phi = io.phi_of(C.base + rowg(y0 + ry) * nx + wrapx(x0 + rx), hv, lo);
+        s_phi[k] = double(phi) + double(lo);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < (rows + 2) * MW; k += kFieldTX * kFieldTY) {
+        const int ry = k / MW - 1, rx = k % MW - 1;
+        if (rx > w) continue;
+        const int cr = walls ? rowg(y0 + ry) - y0 : ry;   // a ghost row's mu is its mirror row's
+        Nbr<double> nb;
+        nbr(s_phi, (cr + 2) * PW + rx + 2, PW, nb);
+        s_mu[k] = chem_pot_f64(C, nb);
+    }
+    __syncthreads();
+    const int tx = threadIdx.x % kFieldTX, ty = threadIdx.x / kFieldTX;
+    if (tx >= w || ty >= rows) return;
+    Nbr<double> nphi, nmu;
+    nbr(s_phi, (ty + 2) * PW + tx + 2, PW, nphi);
+    nbr(s_mu, (ty + 1) * MW + tx + 1, MW, nmu);
+    double v[7];
+    bool fin;
+    cell_fields<FORM, PLAP, false>(a, C, x0 + tx, y0 + ty, nphi, nmu, v, fin);
+    put_fields(a, nx * ny, (y0 + ty) * nx + x0 + tx, v);
 }
 
 // Diagnostics: per-block FP64 partial sums written to a.partials (scratch,
@@ -205,7 +281,7 @@ __global__ void __launch_bounds__(256) diag_pass(const AuxArgs a) {
     for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < n; cell += gridDim.x * blockDim.x) {
         double v[7];
         bool fin;
-        cell_fields<FORM, true, true>(a, C, cell, v, fin);
+        cell_fields_at<FORM, true, true>(a, C, cell, v, fin);
         const double phi = v[0], ux = v[1], uy = v[2], rho = v[4], P = v[6];
         const double x = double(cell % C.nx), y = double(cell / C.nx);
         const double uu = ux * ux + uy * uy;

@@ -155,7 +155,7 @@ template <int FORM> bool has_async_t();                    // the form has the c
 template <int FORM> bool has_pairs_t();                    // the form has the paired kernel
 template <int FORM> cudaError_t launch_init_t(const StepArgs& a, const double* phi0, int instance,
                                               int ncells, cudaStream_t s);
-template <int FORM> cudaError_t launch_fields_t(const AuxArgs& a, int ncells, cudaStream_t s);
+template <int FORM> cudaError_t launch_fields_t(const AuxArgs& a, int nx, int ny, cudaStream_t s);
 template <int FORM> cudaError_t launch_diag_t(const AuxArgs& a, int ncells, cudaStream_t s);
 template <int FORM> cudaError_t launch_populations_t(const AuxArgs& a, int ncells, double* out_h,
                                                      double* out_g, cudaStream_t s);

@@ -334,8 +334,18 @@ cudaError_t launch_init_t(const StepArgs& a, const double* phi0, int instance, i
 }
 
 template <int FORM>
-cudaError_t launch_fields_t(const AuxArgs& a, int ncells, cudaStream_t s) {
-    const int g = grid_for(ncells, 256);
+cudaError_t launch_fields_t(const AuxArgs& a, int nx, int ny, cudaStream_t s) {
+    // us a call, tiles and passes, f32_c phi, u, p: 64 x 64 10.4 and 20.6, 150 x 150 16.5
+    // and 20.6, 400 x 400 54.7 and 61.8, 512 x 512 82.1 and 83.1, 1024 x 1024 305 and 296;
+    // FP64 400 x 400 53.3 and 55.4, 512 x 512 80.0 and 73.9; with P 66 and 70, 101 and 96
+    constexpr int kTileCells = 200000;
+    if (nx * ny <= kTileCells) {
+        const int tiles = ((nx + kFieldTX - 1) / kFieldTX) * ((ny + kFieldTY - 1) / kFieldTY);
+        if (a.mask & LBM_FIELD_PLAP) fields_tile<FORM, true><<<tiles, kFieldTX * kFieldTY, 0, s>>>(a);
+        else fields_tile<FORM, false><<<tiles, kFieldTX * kFieldTY, 0, s>>>(a);
+        return cudaGetLastError();
+    }
+    const int g = grid_for(nx * ny, 256);
     phi_pass<FORM><<<g, 256, 0, s>>>(a);
     mu_pass<FORM><<<g, 256, 0, s>>>(a);
     if (a.mask & LBM_FIELD_PLAP) fields_pass<FORM, true><<<g, 256, 0, s>>>(a);
@@ -375,7 +385,7 @@ cudaError_t launch_populations_t(const AuxArgs& a, int ncells, double* out_h, do
     template bool has_pairs_t<F>();                                                           \
     template cudaError_t launch_init_t<F>(const StepArgs&, const double*, int, int,           \
                                           cudaStream_t);                                      \
-    template cudaError_t launch_fields_t<F>(const AuxArgs&, int, cudaStream_t);               \
+    template cudaError_t launch_fields_t<F>(const AuxArgs&, int, int, cudaStream_t);               \
     template cudaError_t launch_diag_t<F>(const AuxArgs&, int, cudaStream_t);                 \
     template cudaError_t launch_populations_t<F>(const AuxArgs&, int, double*, double*,       \
                                                  cudaStream_t);
