@@ -39,11 +39,10 @@
 #include "lbm.h"
 #include "lbm_mbar.cuh"
 #include "lbm_tileplan.h"
-#include "lbm_device.cuh"   // lbm::F2, two cells' FP32 values in packed instructions
+#include "lbm_device.cuh"
 
 namespace {
 
-using lbm::F2;
 constexpr int kQ = 9;
 __host__ __device__ constexpr int sx(int i) { return i == 1 || i == 5 || i == 8 ? 1 : (i == 3 || i == 6 || i == 7 ? -1 : 0); }
 __host__ __device__ constexpr int sy(int i) { return i == 2 || i == 5 || i == 6 ? 1 : (i == 4 || i == 7 || i == 8 ? -1 : 0); }
@@ -53,189 +52,15 @@ static_assert(sopp(1) == 3 && sopp(2) == 4 && sopp(5) == 7 && sopp(6) == 8 && so
 // one direction of each opposite pair (1, 2, 5, 6; their opposites 3, 4, 7, 8)
 __host__ __device__ constexpr int pair2(int q) { return q == 0 ? 1 : q == 1 ? 2 : q == 2 ? 5 : 6; }
 
-struct SpConst {
-    int nx, ny, walls;
-    double inv_tau, src, tgm, Qc, fx, fy;   // 1/tau_g, 1 - 1/(2 tau_g), tau_g - 1/2, Q, F
-    double dl, dq;                          // drag of the Remark 4 scheme: F(u) = F - (dl + dq |u|) u
-    double p0;                              // Remark 2: the constant p_0
-    // derived on the host, so that FP32 kernels do no FP64 arithmetic on them
-    double tau, Qd0;                        // tau_g; Q - (2/d) c_s^2 (the part of Q without the density)
-    double hp0, ip0, hp0fx, hp0fy;          // p_0 / 2, 1 / p_0, p_0 F_1 / 2
-};
-
-template <typename R>
-struct SpCell { R ux, uy, p; };
-
-// u (Eq. 27a, rho = 1), G_i (Remark 3) and p (Eq. 28) of one cell
-template <typename R>
-__device__ __forceinline__ SpCell<R> sp_moments(const SpConst& K, const R g[kQ], R S, R G[kQ]) {
-    SpCell<R> m;
-    R jx = R(0), jy = R(0), rest = R(0);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) {
-        if (sx(i)) jx += sx(i) > 0 ? g[i] : -g[i];
-        if (sy(i)) jy += sy(i) > 0 ? g[i] : -g[i];
-        rest += g[i];
-    }
-    const R fx = R(K.fx), fy = R(K.fy);
-    m.ux = jx + R(0.5) * fx;
-    m.uy = jy + R(0.5) * fy;
-    const R uF = m.ux * fx + m.uy * fy, uu = m.ux * m.ux + m.uy * m.uy;
-    const R QS = R(K.Qc) * S;
-    // (c c - c_s^2 I):(u F + F u + Q S I) / (2 c_s^4) = 9 (c.u)(c.F) - 3 u.F + 4.5 (|c|^2 - 2/3) Q S;
-    // for opposite directions the part even in c is shared and c.F / c_s^2 flips sign
-    G[0] = R(sw(0)) * (S - R(3) * uF + R(4.5) * (-R(2.0 / 3.0)) * QS);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = pair2(q), j = sopp(i);
-        const R cu = R(sx(i)) * m.ux + R(sy(i)) * m.uy, cF = R(sx(i)) * fx + R(sy(i)) * fy;
-        const R c2 = R(sx(i) * sx(i) + sy(i) * sy(i));
-        const R e = R(sw(i)) * (S + R(9) * cu * cF - R(3) * uF + R(4.5) * (c2 - R(2.0 / 3.0)) * QS);
-        const R o = R(sw(i)) * (R(3) * cF);
-        G[i] = e + o;
-        G[j] = e - o;
-    }
-    // Eq. 28: c_s^2 / (1 - w_0) = 3/5; s_0(u) = -w_0 u.u / (2 c_s^2) = -(2/3) u.u
-    m.p = R(0.6) * (rest + R(0.5) * S - R(2.0 / 3.0) * uu + R(K.tgm) * G[0]);
-    return m;
-}
-
-// ---- Remarks 1 and 2 (M = 1, 2) ----
-// g holds g_i - w_i a0 (a0 = 1 for Remark 1, p_0 for Remark 2: the rest state).
-// d = rho - 1 (Remark 1) or p - p_0 (Remark 2); a = rho or p_0, the factor of
-// s_i(u) in g^eq (Eq. 29bb, Eq. 29bd); both equilibria are d w_i + a s_i(u)
-// after the shift. Sg and the force Fg are in the units of g (Remark 2: p_0 S_1,
-// p_0 F_1).
-template <int M, typename R>
-__device__ __forceinline__ void sp1_moments(const SpConst& K, const R g[kQ], R S, R& d, R& a, R& ux, R& uy) {
-    R m0 = g[0], jx = R(0), jy = R(0);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) {
-        m0 += g[i];
-        if (sx(i)) jx += sx(i) > 0 ? g[i] : -g[i];
-        if (sy(i)) jy += sy(i) > 0 ? g[i] : -g[i];
-    }
-    if constexpr (M == 1) {
-        d = m0 + R(0.5) * S;                       // Eq. 27aa
-        a = R(1) + d;
-        const R ir = R(1) / a;
-        ux = (jx + R(0.5) * R(K.fx)) * ir;         // Eq. 27a
-        uy = (jy + R(0.5) * R(K.fy)) * ir;
-    } else {
-        d = m0 + R(K.hp0) * S;                     // p = sum g + p_0 S_1 / 2
-        a = R(K.p0);
-        ux = (jx + R(K.hp0fx)) * R(K.ip0);         // p_0 u = sum c g + p_0 F_1 / 2
-        uy = (jy + R(K.hp0fy)) * R(K.ip0);
-    }
-}
-
-template <int M, typename R>
-__global__ void sp1_fields_kernel(const R* __restrict__ g, const R* __restrict__ src, long long N, SpConst K,
-                                  unsigned mask, double* __restrict__ out) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    R gc[kQ], d, a, ux, uy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) gc[i] = g[i * N + c];
-    sp1_moments<M>(K, gc, src[c], d, a, ux, uy);
-    // Remark 1: p = rho c_s^2, rho = 1 + d; Remark 2: p = p_0 + d
-    const double p = M == 1 ? (1.0 + double(d)) / 3.0 : K.p0 + double(d);
-    int slot = 0;
-    if (mask & LBM_FIELD_UX) out[(slot++) * N + c] = double(ux);
-    if (mask & LBM_FIELD_UY) out[(slot++) * N + c] = double(uy);
-    if (mask & LBM_FIELD_P) out[(slot++) * N + c] = p;
-    if (M == 1 && (mask & LBM_FIELD_RHO)) out[(slot++) * N + c] = 1.0 + double(d);
-}
-
-// ---- Remark 4 scheme (on the Remark 3 model) ----
-template <typename R>
-__device__ __forceinline__ void sp4_u(const R f[kQ], R& ux, R& uy) {
-    R jx = R(0), jy = R(0);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) {
-        if (sx(i)) jx += sx(i) > 0 ? f[i] : -f[i];
-        if (sy(i)) jy += sy(i) > 0 ? f[i] : -f[i];
-    }
-    ux = jx;
-    uy = jy;
-}
-
-template <typename R>
-__device__ __forceinline__ void sp4_force(const SpConst& K, R ux, R uy, R& Fx, R& Fy) {
-    const R k = R(K.dl) + R(K.dq) * sqrt(ux * ux + uy * uy);
-    Fx = R(K.fx) - k * ux;
-    Fy = R(K.fy) - k * uy;
-}
-
-// G_i of Remark 3 with force F at velocity u, direction i
-template <typename R>
-__device__ __forceinline__ R sp4_G(const SpConst& K, int i, R S, R ux, R uy, R Fx, R Fy) {
-    const R cu = R(sx(i)) * ux + R(sy(i)) * uy, cF = R(sx(i)) * Fx + R(sy(i)) * Fy;
-    const R c2 = R(sx(i) * sx(i) + sy(i) * sy(i));
-    return R(sw(i)) * (S + R(3) * cF + R(9) * cu * cF - R(3) * (ux * Fx + uy * Fy) +
-                       R(4.5) * (c2 - R(2.0 / 3.0)) * R(K.Qc) * S);
-}
-
-template <typename R>
-__global__ void sp4_fields_kernel(const R* __restrict__ f, const R* __restrict__ src, long long N, SpConst K,
-                                  unsigned mask, double* __restrict__ out) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    R fc[kQ], ux, uy, Fx, Fy;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) fc[i] = f[i * N + c];
-    sp4_u(fc, ux, uy);
-    sp4_force(K, ux, uy, Fx, Fy);
-    R rest = R(0);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) rest += fc[i];
-    const R G0 = sp4_G(K, 0, src[c], ux, uy, Fx, Fy);
-    const R p = R(0.6) * (rest - R(2.0 / 3.0) * (ux * ux + uy * uy) + R(K.tau) * G0);
-    int slot = 0;
-    if (mask & LBM_FIELD_UX) out[(slot++) * N + c] = double(ux);
-    if (mask & LBM_FIELD_UY) out[(slot++) * N + c] = double(uy);
-    if (mask & LBM_FIELD_P) out[(slot++) * N + c] = double(p);
-}
-
-// populations g_i = stored + w_i, widened to FP64
-template <typename R>
-__global__ void sp1_widen_kernel(const R* __restrict__ in, double* __restrict__ out, long long N, double a0) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) out[i * N + c] = double(in[i * N + c]) + sw(i) * a0;
-}
-
-template <typename R>
-__global__ void sp_fields_kernel(const R* __restrict__ g, const R* __restrict__ src, long long N, SpConst K,
-                                 unsigned mask, double* __restrict__ out) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    R gc[kQ], G[kQ];
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) gc[i] = g[i * N + c];
-    const SpCell<R> m = sp_moments(K, gc, src[c], G);
-    int slot = 0;
-    if (mask & LBM_FIELD_UX) out[(slot++) * N + c] = double(m.ux);
-    if (mask & LBM_FIELD_UY) out[(slot++) * N + c] = double(m.uy);
-    if (mask & LBM_FIELD_P) out[(slot++) * N + c] = double(m.p);
-}
-
-template <typename R>
-__global__ void sp_convert_kernel(const double* __restrict__ in, R* __restrict__ out, long long n) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < n) out[c] = R(in[c]);
-}
-
-template <typename R>
-__global__ void sp_widen_kernel(const R* __restrict__ in, double* __restrict__ out, long long n) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < n) out[c] = double(in[c]);
-}
-
-// ---- The step ----
-// One cell of a unit: float or double with explicit roundings; F2 is a unit of two
-// cells (x, x + 1), x even, in packed FP32 instructions (nx even).
+// ---- Arithmetic ----
+// A unit of the step: one cell (One<float>, One<double>), or two horizontally
+// adjacent ones (x, x + 1), x even, in packed FP32 instructions (Two; nx even). No
+// sum below is left to the compiler to contract: a velocity component that the flow
+// does not have (u_y of a source that does not vary in y) is nothing but the rounding
+// residue of these sums, so which products are rounded before they are added is part
+// of the results, and the same in every kernel. For the packed instructions, which
+// the compiler contracts where it likes, that takes additions as FFMA2 with a factor
+// that it cannot know to be 1 or -1.
 template <typename T>
 struct One {
     T v;
@@ -250,11 +75,38 @@ __device__ __forceinline__ One<double> operator+(One<double> a, One<double> b) {
 __device__ __forceinline__ One<double> operator-(One<double> a, One<double> b) { return __dsub_rn(a.v, b.v); }
 __device__ __forceinline__ One<double> operator*(One<double> a, One<double> b) { return __dmul_rn(a.v, b.v); }
 __device__ __forceinline__ One<double> fmadd(One<double> a, One<double> b, One<double> c) { return __fma_rn(a.v, b.v, c.v); }
-// 1/x and sqrt(x), correctly rounded per lane
+template <typename T> __device__ __forceinline__ One<T> operator-(One<T> a) { return One<T>(-a.v); }
+
+__constant__ float2 sp_plus = {1.f, 1.f}, sp_minus = {-1.f, -1.f};   // (never written)
+struct Two {
+    float2 v;
+    Two() = default;
+    __device__ __forceinline__ Two(float s) : v(make_float2(s, s)) {}
+    __device__ __forceinline__ Two(float a, float b) : v(make_float2(a, b)) {}
+    __device__ __forceinline__ explicit Two(float2 w) : v(w) {}
+};
+__device__ __forceinline__ Two operator+(Two a, Two b) { return Two(__ffma2_rn(b.v, sp_plus, a.v)); }
+__device__ __forceinline__ Two operator-(Two a, Two b) { return Two(__ffma2_rn(b.v, sp_minus, a.v)); }
+__device__ __forceinline__ Two operator*(Two a, Two b) { return Two(__fmul2_rn(a.v, b.v)); }
+__device__ __forceinline__ Two operator-(Two a) { return Two(-a.v.x, -a.v.y); }
+__device__ __forceinline__ Two fmadd(Two a, Two b, Two c) { return Two(__ffma2_rn(a.v, b.v, c.v)); }
+
+// c + a b and c - a b, rounded once by a single cell, the product first by a pair
+template <typename T>
+__device__ __forceinline__ One<T> add_prod(One<T> c, One<T> a, One<T> b) { return fmadd(a, b, c); }
+template <typename T>
+__device__ __forceinline__ One<T> sub_prod(One<T> c, One<T> a, One<T> b) { return fmadd(-a, b, c); }
+__device__ __forceinline__ Two add_prod(Two c, Two a, Two b) { return c + a * b; }
+__device__ __forceinline__ Two sub_prod(Two c, Two a, Two b) { return c - a * b; }
+// a b - c d: the first product not rounded by a single cell, both rounded by a pair
+template <typename T>
+__device__ __forceinline__ One<T> diff_prod(One<T> a, One<T> b, One<T> c, One<T> d) { return fmadd(a, b, -(c * d)); }
+__device__ __forceinline__ Two diff_prod(Two a, Two b, Two c, Two d) { return a * b - c * d; }
+// 1/x and sqrt(x), correctly rounded per cell
 template <typename T> __device__ __forceinline__ One<T> sp_inv(One<T> x) { return One<T>(T(1) / x.v); }
 template <typename T> __device__ __forceinline__ One<T> sp_sqrt(One<T> x) { return One<T>(sqrt(x.v)); }
-__device__ __forceinline__ F2 sp_inv(F2 x) { return F2(1.f / x.v.x, 1.f / x.v.y); }
-__device__ __forceinline__ F2 sp_sqrt(F2 x) { return F2(sqrtf(x.v.x), sqrtf(x.v.y)); }
+__device__ __forceinline__ Two sp_inv(Two x) { return Two(1.f / x.v.x, 1.f / x.v.y); }
+__device__ __forceinline__ Two sp_sqrt(Two x) { return Two(sqrtf(x.v.x), sqrtf(x.v.y)); }
 
 // How a unit sits in memory: T values of one cell or a pair, one access.
 template <typename V> struct Unit;
@@ -273,19 +125,19 @@ template <typename T> struct Unit<One<T>> {
         row[X < 0 ? nx - 1 : (X == nx ? 0 : X)] = v.v;
     }
 };
-template <> struct Unit<F2> {
+template <> struct Unit<Two> {
     using R = float;
     using E = float2;
     static constexpr int cells = 2;
-    __device__ __forceinline__ static F2 ld(const float* p) { return F2(*reinterpret_cast<const float2*>(p)); }
-    __device__ __forceinline__ static void st(float* p, F2 v) { *reinterpret_cast<float2*>(p) = v.v; }
-    __device__ __forceinline__ static E pack(F2 v) { return v.v; }
-    __device__ __forceinline__ static F2 at(const E* row, int t, int dx) {
-        if (dx < 0) return F2(row[t - 1].y, row[t].x);
-        if (dx > 0) return F2(row[t].y, row[t + 1].x);
-        return F2(row[t]);
+    __device__ __forceinline__ static Two ld(const float* p) { return Two(*reinterpret_cast<const float2*>(p)); }
+    __device__ __forceinline__ static void st(float* p, Two v) { *reinterpret_cast<float2*>(p) = v.v; }
+    __device__ __forceinline__ static E pack(Two v) { return v.v; }
+    __device__ __forceinline__ static Two at(const E* row, int t, int dx) {
+        if (dx < 0) return Two(row[t - 1].y, row[t].x);
+        if (dx > 0) return Two(row[t].y, row[t + 1].x);
+        return Two(row[t]);
     }
-    __device__ __forceinline__ static void push(float* row, int x, int nx, int dx, F2 v) {
+    __device__ __forceinline__ static void push(float* row, int x, int nx, int dx, Two v) {
         if (dx == 0) {   // keeps the pair together
             st(row + x, v);
         } else {
@@ -295,253 +147,339 @@ template <> struct Unit<F2> {
     }
 };
 
-// Constants of the step in the arithmetic type, derived on the host (SpConst) so
-// that the kernels convert and combine nothing. F is in the units of g (Remark 2:
-// p_0 F_1); ka, kd, k0: 1 + 4.5 (|c|^2 - 2/3) Q of the axes, the diagonals and the
-// rest direction (Remark 3), times w_i.
+// Constants of a model: FP64, and for FP32 contexts converted on the host, so that
+// their kernels do no FP64 arithmetic.
 template <typename T>
-struct SpK {
+struct SpConst {
     int nx, ny, walls;
-    T om, sg, om_h;            // 1/tau_g, 1 - 1/(2 tau_g), om / 2
-    T fx, fy, hfx, hfy;        // F, F / 2
-    T sgfx, sgfy, hsgfx, hsgfy;   // sg F, sg F / 2
-    T ka, kd, k0, ska, skd, sk0;  // Remark 3, Remark 4; s..: times sg
-    T tgm, tau;
-    T sc, hS, p0, ip0;         // Remarks 1, 2: units of S; S / 2 in them; p_0, 1 / p_0 (Remark 1: unused)
-    T q, q0;                   // gs Q = (a q + q0) 12 div u
-    T dl, dq;                  // drag
+    T inv_tau, src, tgm, Qc, fx, fy;   // 1/tau_g, 1 - 1/(2 tau_g), tau_g - 1/2, Q, F
+    T dl, dq;                          // drag of the Remark 4 scheme: F(u) = F - (dl + dq |u|) u
+    T p0;                              // Remark 2: the constant p_0
+    T tau, Qd0;                        // tau_g; Q - (2/d) c_s^2 (the part of Q without the density)
+    T hp0, ip0, hp0fx, hp0fy;          // p_0 / 2, 1 / p_0, p_0 F_1 / 2
 };
-
 template <typename T>
-SpK<T> sp_consts(const SpConst& K, int model) {
-    SpK<T> k;
-    const double sc = model == 2 ? K.p0 : 1.0, fx = sc * K.fx, fy = sc * K.fy, om = K.inv_tau, sg = K.src;
-    const double ka = (1.0 + 1.5 * K.Qc) / 9.0, kd = (1.0 + 6.0 * K.Qc) / 36.0, k0 = (1.0 - 3.0 * K.Qc) * 4.0 / 9.0;
-    k.nx = K.nx; k.ny = K.ny; k.walls = K.walls;
-    k.om = T(om); k.sg = T(sg); k.om_h = T(0.5 * om);
-    k.fx = T(fx); k.fy = T(fy); k.hfx = T(0.5 * fx); k.hfy = T(0.5 * fy);
-    k.sgfx = T(sg * fx); k.sgfy = T(sg * fy); k.hsgfx = T(0.5 * sg * fx); k.hsgfy = T(0.5 * sg * fy);
-    k.ka = T(ka); k.kd = T(kd); k.k0 = T(k0); k.ska = T(sg * ka); k.skd = T(sg * kd); k.sk0 = T(sg * k0);
-    k.tgm = T(K.tgm); k.tau = T(K.tau);
-    k.sc = T(sc); k.hS = T(0.5 * sc); k.p0 = T(K.p0); k.ip0 = T(K.ip0);
-    k.q = T(sg / 36.0); k.q0 = T(sg * K.Qd0 / 12.0);
-    k.dl = T(K.dl); k.dq = T(K.dq);
-    return k;
+SpConst<T> sp_const_as(const SpConst<double>& K) {
+    return SpConst<T>{K.nx, K.ny, K.walls, T(K.inv_tau), T(K.src), T(K.tgm), T(K.Qc), T(K.fx), T(K.fy),
+                      T(K.dl), T(K.dq), T(K.p0), T(K.tau), T(K.Qd0), T(K.hp0), T(K.ip0), T(K.hp0fx), T(K.hp0fy)};
+}
+// 4.5 (|c_i|^2 - 2/3), rounded in the arithmetic type
+template <typename T>
+__device__ __forceinline__ constexpr T sp_c2(int i) {
+    return T(4.5) * (T(sx(i) * sx(i) + sy(i) * sy(i)) - T(2.0 / 3.0));
 }
 
+// ---- Moments, of the step and of the read-back: the u handed out is the u the step
+// collides with ----
+// sum c_i g_i, one population after the other
+template <typename V>
+__device__ __forceinline__ void sp_j(const V (&g)[kQ], V& jx, V& jy) {
+    jx = g[1];
+    jy = g[2];
+#pragma unroll
+    for (int i = 3; i < kQ; ++i) {
+        if (sx(i)) jx = sx(i) > 0 ? jx + g[i] : jx - g[i];
+        if (sy(i)) jy = sy(i) > 0 ? jy + g[i] : jy - g[i];
+    }
+}
+template <typename V>
+__device__ __forceinline__ V sp_rest(const V (&g)[kQ]) {
+    V s = g[1];
+#pragma unroll
+    for (int i = 2; i < kQ; ++i) s = s + g[i];
+    return s;
+}
+
+// Remark 3: u (Eq. 27a, rho = 1), u.F, u.u, G_0 and p (Eq. 28)
+template <typename V>
+struct SpCell { V ux, uy, uF, uu, G0, p; };
+template <typename V, typename T>
+__device__ __forceinline__ SpCell<V> sp3_moments(const SpConst<T>& K, const V (&g)[kQ], V S) {
+    SpCell<V> m;
+    V jx, jy;
+    sp_j(g, jx, jy);
+    m.ux = jx + V(T(0.5) * K.fx);
+    m.uy = jy + V(T(0.5) * K.fy);
+    m.uF = fmadd(m.ux, V(K.fx), m.uy * V(K.fy));
+    m.uu = fmadd(m.ux, m.ux, m.uy * m.uy);
+    m.G0 = V(T(sw(0))) * fmadd(V(sp_c2<T>(0)), V(K.Qc) * S, sub_prod(S, V(T(3)), m.uF));
+    // c_s^2 / (1 - w_0) = 3/5; s_0(u) = -w_0 u.u / (2 c_s^2) = -(2/3) u.u
+    m.p = V(T(0.6)) * fmadd(V(K.tgm), m.G0, sub_prod(sp_rest(g) + V(T(0.5)) * S, V(T(2.0 / 3.0)), m.uu));
+    return m;
+}
+
+// Remarks 1 and 2 (M = 1, 2): g holds g_i - w_i a0 (a0 = 1 for Remark 1, p_0 for
+// Remark 2: the rest state). d = rho - 1 (Remark 1) or p - p_0 (Remark 2); a = rho or
+// p_0, the factor of s_i(u) in g^eq (Eq. 29bb, Eq. 29bd); both equilibria are d w_i +
+// a s_i(u) after the shift.
+template <int M, typename V, typename T>
+__device__ __forceinline__ void sp1_moments(const SpConst<T>& K, const V (&g)[kQ], V S, V& d, V& a, V& ux, V& uy) {
+    V m0 = g[0], jx, jy;
+    sp_j(g, jx, jy);
+#pragma unroll
+    for (int i = 1; i < kQ; ++i) m0 = m0 + g[i];
+    if constexpr (M == 1) {
+        d = m0 + V(T(0.5)) * S;                       // Eq. 27aa
+        a = V(T(1)) + d;
+        const V ir = sp_inv(a);
+        ux = (jx + V(T(0.5) * K.fx)) * ir;            // Eq. 27a
+        uy = (jy + V(T(0.5) * K.fy)) * ir;
+    } else {
+        d = fmadd(V(K.hp0), S, m0);                   // p = sum g + p_0 S_1 / 2
+        a = V(K.p0);
+        ux = (jx + V(K.hp0fx)) * V(K.ip0);            // p_0 u = sum c g + p_0 F_1 / 2
+        uy = (jy + V(K.hp0fy)) * V(K.ip0);
+    }
+}
+
+// Remark 4 scheme: F(u)
+template <typename V, typename T>
+__device__ __forceinline__ void sp4_force(const SpConst<T>& K, V ux, V uy, V& Fx, V& Fy) {
+    const V k = fmadd(V(K.dq), sp_sqrt(fmadd(ux, ux, uy * uy)), V(K.dl));
+    Fx = sub_prod(V(K.fx), k, ux);
+    Fy = sub_prod(V(K.fy), k, uy);
+}
+// G_0 / w_0
+template <typename V, typename T>
+__device__ __forceinline__ V sp4_G0w(const SpConst<T>& K, V S, V uF) {
+    return fmadd(V(sp_c2<T>(0) * K.Qc), S, sub_prod(S, V(T(3)), uF));
+}
+// p (Eq. 28 for the unshifted f, tau_g G_0)
+template <typename V, typename T>
+__device__ __forceinline__ V sp4_p(const SpConst<T>& K, const V (&f)[kQ], V uu, V G0) {
+    return V(T(0.6)) * fmadd(V(K.tau), G0, sub_prod(sp_rest(f), V(T(2.0 / 3.0)), uu));
+}
+
+// ---- Read-back ----
+template <int M, typename R>
+__global__ void sp1_fields_kernel(const R* __restrict__ g, const R* __restrict__ src, long long N, SpConst<R> K,
+                                  double p0, unsigned mask, double* __restrict__ out) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= N) return;
+    One<R> gc[kQ], d, a, ux, uy;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) gc[i] = g[i * N + c];
+    sp1_moments<M>(K, gc, One<R>(src[c]), d, a, ux, uy);
+    // Remark 1: p = rho c_s^2, rho = 1 + d; Remark 2: p = p_0 + d
+    const double p = M == 1 ? (1.0 + double(d.v)) / 3.0 : p0 + double(d.v);
+    int slot = 0;
+    if (mask & LBM_FIELD_UX) out[(slot++) * N + c] = double(ux.v);
+    if (mask & LBM_FIELD_UY) out[(slot++) * N + c] = double(uy.v);
+    if (mask & LBM_FIELD_P) out[(slot++) * N + c] = p;
+    if (M == 1 && (mask & LBM_FIELD_RHO)) out[(slot++) * N + c] = 1.0 + double(d.v);
+}
+
+// Remark 3, or (R4) the Remark 4 scheme
+template <bool R4, typename R>
+__global__ void sp_fields_kernel(const R* __restrict__ g, const R* __restrict__ src, long long N, SpConst<R> K,
+                                 unsigned mask, double* __restrict__ out) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= N) return;
+    One<R> gc[kQ], ux, uy, p;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) gc[i] = g[i * N + c];
+    const One<R> S(src[c]);
+    if constexpr (R4) {
+        One<R> Fx, Fy;
+        sp_j(gc, ux, uy);
+        sp4_force(K, ux, uy, Fx, Fy);
+        const One<R> G0 = One<R>(R(sw(0))) * sp4_G0w(K, S, fmadd(ux, Fx, uy * Fy));
+        p = sp4_p(K, gc, fmadd(ux, ux, uy * uy), G0);
+    } else {
+        const SpCell<One<R>> m = sp3_moments(K, gc, S);
+        ux = m.ux;
+        uy = m.uy;
+        p = m.p;
+    }
+    int slot = 0;
+    if (mask & LBM_FIELD_UX) out[(slot++) * N + c] = double(ux.v);
+    if (mask & LBM_FIELD_UY) out[(slot++) * N + c] = double(uy.v);
+    if (mask & LBM_FIELD_P) out[(slot++) * N + c] = double(p.v);
+}
+
+// populations g_i = stored + w_i, widened to FP64
+template <typename R>
+__global__ void sp1_widen_kernel(const R* __restrict__ in, double* __restrict__ out, long long N, double a0) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= N) return;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) out[i * N + c] = double(in[i * N + c]) + sw(i) * a0;
+}
+
+template <typename R>
+__global__ void sp_convert_kernel(const double* __restrict__ in, R* __restrict__ out, long long n) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < n) out[c] = R(in[c]);
+}
+
+template <typename R>
+__global__ void sp_widen_kernel(const R* __restrict__ in, double* __restrict__ out, long long n) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < n) out[c] = double(in[c]);
+}
+
+// ---- The step ----
 // The four models by one number: Remarks 1, 2, 3 and the Remark 4 scheme.
 // What a cell's neighbours need of it (values of the shared-memory ring): u for
-// div u (Remarks 1, 2), G_1 .. G_8 for G_i at x + c_i (Remark 4), nothing (3).
+// div u (Remarks 1, 2), G_i / w_i, i = 1 .. 8, for G_i at x + c_i (Remark 4),
+// nothing (3).
 template <int KIND> constexpr int kRing = KIND == 4 ? 8 : (KIND == 3 ? 0 : 2);
 
 // A cell's own values besides its populations and S.
 template <typename V>
-struct SpMom { V ux, uy, a, b; };   // u; Remarks 1, 2: d and a of the equilibrium; Remark 4: a = G_0
+struct SpMom { V ux, uy, a, b; };   // u; Remarks 1, 2: d and a of the equilibrium; Remark 4: F(u)
 
+// c_i.(x, y) of the directions 1, 2, 5, 6
 template <typename V>
-__device__ __forceinline__ void sp_j(const V (&g)[kQ], V& jx, V& jy) {
-    const V a = g[5] - g[7], b = g[6] - g[8];
-    jx = (g[1] - g[3]) + (a - b);
-    jy = (g[2] - g[4]) + (a + b);
-}
-template <typename V>
-__device__ __forceinline__ V sp_rest(const V (&g)[kQ]) {
-    return ((g[1] + g[2]) + (g[3] + g[4])) + ((g[5] + g[6]) + (g[7] + g[8]));
-}
-
-// (1 - om) g + x. In FP32 as x - om g, then + g: 1 - om rounded to FP32 would
-// give every step a bias of up to 2^-25 of the momentum. (FP64: one operation.)
-template <typename T>
-__device__ __forceinline__ One<T> sp_relax(T om, One<T> g, One<T> x) {
-    if constexpr (sizeof(T) == 8) return fmadd(One<T>(T(1) - om), g, x);
-    else return fmadd(One<T>(-om), g, x) + g;
-}
-__device__ __forceinline__ F2 sp_relax(float om, F2 g, F2 x) { return fmadd(F2(-om), g, x) + g; }
-// The odd parts 3 w_i c.T of a vector T over the axes (a) and, as components, the
-// diagonals (d = a / 4), from T / 2. The FP32 constants here and below (w_i, w_0 -
-// 1, 3/5 and 3 p from p) are the roundings of the remarks' own factors: products
-// of them rounded once instead, or sums that conserve the momentum exactly, are
-// closer to FP64 but drift from these by up to 1e-4 of a weak velocity component
-// in 200 steps.
-template <typename V>
-__device__ __forceinline__ void sp_odd(V half, V& a, V& d) {
-    using T = typename Unit<V>::R;
-    a = V(T(1) / T(9)) * (V(T(6)) * half);
-    d = V(T(0.25)) * a;
-}
-
-// Remark 4: F(u), and the parts of G_i even and odd in c of the pairs (1, 3),
-// (2, 4), (5, 7), (6, 8); G_0 returned.
-template <typename V, typename T>
-__device__ __forceinline__ void sp4_F(const SpK<T>& K, V ux, V uy, V& Fx, V& Fy) {
-    const V k = fmadd(V(K.dq), sp_sqrt(fmadd(ux, ux, uy * uy)), V(K.dl));
-    Fx = V(K.fx) - k * ux;
-    Fy = V(K.fy) - k * uy;
-}
-template <typename V, typename T>
-__device__ __forceinline__ V sp4_Gs(const SpK<T>& K, V S, V ux, V uy, V Fx, V Fy, V (&e)[4], V (&o)[4]) {
-    const V t = V(T(-3)) * fmadd(ux, Fx, uy * Fy);
-    const V ea = fmadd(S, V(K.ka), V(T(1) / T(9)) * t), ed = fmadd(S, V(K.kd), V(T(1) / T(36)) * t);
-    const V up = V(T(0.25)) * (ux + uy), um = V(T(0.25)) * (uy - ux), Fp = Fx + Fy, Fm = Fy - Fx;
-    e[0] = fmadd(ux, Fx, ea);
-    e[1] = fmadd(uy, Fy, ea);
-    e[2] = fmadd(up, Fp, ed);
-    e[3] = fmadd(um, Fm, ed);
-    V dx, dy;
-    sp_odd(V(T(0.5)) * Fx, o[0], dx);
-    sp_odd(V(T(0.5)) * Fy, o[1], dy);
-    o[2] = dx + dy;
-    o[3] = dy - dx;
-    return fmadd(S, V(K.k0), V(T(4) / T(9)) * t);
-}
+__device__ __forceinline__ V sp_dot(int i, V x, V y) { return i == 1 ? x : i == 2 ? y : i == 5 ? x + y : y - x; }
 
 // u and what the neighbours need (put(r, value): ring value r).
 template <int KIND, typename V, typename T, typename Put>
-__device__ __forceinline__ void sp_moments_of(const SpK<T>& K, const V (&g)[kQ], V S, SpMom<V>& m, Put&& put) {
-    V jx, jy;
-    sp_j(g, jx, jy);
-    if constexpr (KIND == 1) {                       // rho - 1 (Eq. 27aa), rho; u (Eq. 27a)
-        m.a = fmadd(V(K.hS), S, g[0] + sp_rest(g));
-        m.b = V(T(1)) + m.a;
-        const V ir = sp_inv(m.b);
-        m.ux = (jx + V(K.hfx)) * ir;
-        m.uy = (jy + V(K.hfy)) * ir;
-    } else if constexpr (KIND == 2) {                // p - p_0, p_0
-        m.a = fmadd(V(K.hS), S, g[0] + sp_rest(g));
-        m.b = V(K.p0);
-        m.ux = (jx + V(K.hfx)) * V(K.ip0);
-        m.uy = (jy + V(K.hfy)) * V(K.ip0);
-    } else if constexpr (KIND == 3) {
-        m.ux = jx + V(K.hfx);
-        m.uy = jy + V(K.hfy);
-    } else {                                         // Remark 4: u = sum c f, G_i with F(u)
-        m.ux = jx;
-        m.uy = jy;
-        V Fx, Fy, e[4], o[4];
-        sp4_F(K, jx, jy, Fx, Fy);
-        m.a = sp4_Gs(K, S, jx, jy, Fx, Fy, e, o);
+__device__ __forceinline__ void sp_moments_of(const SpConst<T>& K, const V (&g)[kQ], V S, SpMom<V>& m, Put&& put) {
+    if constexpr (KIND == 4) {
+        sp_j(g, m.ux, m.uy);   // u = sum c f
+        sp4_force(K, m.ux, m.uy, m.a, m.b);
+        const V uF = fmadd(m.ux, m.a, m.uy * m.b), three(T(3));
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            put(pair2(k) - 1, e[k] + o[k]);
-            put(sopp(pair2(k)) - 1, e[k] - o[k]);
+        for (int q = 0; q < 4; ++q) {
+            const int i = pair2(q);
+            const V cu9 = V(T(9)) * sp_dot(i, m.ux, m.uy), cF = sp_dot(i, m.a, m.b), cQ(sp_c2<T>(i) * K.Qc);
+            put(i - 1, fmadd(cQ, S, sub_prod(fmadd(cu9, cF, fmadd(three, cF, S)), three, uF)));
+            put(sopp(i) - 1, fmadd(cQ, S, sub_prod(fmadd(cu9, cF, fmadd(-three, cF, S)), three, uF)));
         }
-    }
-    if constexpr (KIND == 1 || KIND == 2) {
+    } else if constexpr (KIND != 3) {
+        sp1_moments<KIND>(K, g, S, m.a, m.b, m.ux, m.uy);
         put(0, m.ux);
         put(1, m.uy);
     }
 }
 
-// Collision (Eq. 24 with the remark's equilibrium and force term). Opposite
-// directions share the part even in c: with sg = 1 - 1/(2 tau_g) and om = 1/tau_g,
-//   g_i* = (1 - om) g_i + E_i +- O_i,  E_i = (c.u)(c.V) + E0,  O_i = 3 w_i c.T,
-// V = w_i (4.5 (om a [- sg S]) u + 9 sg F), T = om a u + sg F; the axes' weights
-// are four times the diagonals'. nb(r, dx, dy): ring value r of a
-// neighbour (mirrored about a wall); up: u at t - 1 (Remark 4); emit(i, value,
-// wall value): the population leaving in direction i, and what returns if a wall
-// reflects it (the same but for Remark 4).
+// Remark 4: the parts of G_i even in c and of c_i.F / c_s^2 (o, without w_i) at velocity u
+template <typename V, typename T>
+__device__ __forceinline__ void sp4_parts(const SpConst<T>& K, int i, V S, V ux, V uy, V Fx, V Fy, V uF, V& e, V& o) {
+    const V cF = sp_dot(i, Fx, Fy), cQ(sp_c2<T>(i) * K.Qc);
+    const V b = sub_prod(fmadd(V(T(9)) * sp_dot(i, ux, uy), cF, S), V(T(3)), uF);
+    e = V(T(sw(i))) * (i >= 5 ? b + cQ * S : fmadd(cQ, S, b));
+    o = V(T(3)) * cF;
+}
+
+// Collision (Eq. 24 with the remark's equilibrium and force term) in opposite pairs of
+// directions: the parts of s_i and G_i even in c shared, the odd parts flipped.
+// nb(r, dx, dy): ring value r of a neighbour (mirrored about a wall); up: u at t - 1
+// (Remark 4); emit(i, value, wall): the population leaving in direction i, and a
+// function giving what returns if a wall reflects it (the same but for Remark 4).
+// (c c - c_s^2 I):(u F + F u [- u u S] + Q D I) / (2 c_s^4) = 9 (c.u)(c.F) - 3 u.F
+// [- 4.5 ((c.u)^2 - u.u / 3) S] + 4.5 (|c|^2 - 2/3) Q D; D = S, or div u (Remarks 1, 2).
 template <int KIND, typename V, typename T, typename Nb, typename Emit>
-__device__ __forceinline__ void sp_collide(const SpK<T>& K, const V (&g)[kQ], V S, const SpMom<V>& m, V upx, V upy,
+__device__ __forceinline__ void sp_collide(const SpConst<T>& K, const V (&g)[kQ], V S, const SpMom<V>& m, V upx, V upy,
                                            Nb&& nb, Emit&& emit) {
-    const V ux = m.ux, uy = m.uy;
-    const V uu = fmadd(ux, ux, uy * uy);
-    const V ninth(T(1) / T(9)), q(T(0.25));
-    if constexpr (KIND == 4) {
-        const V G0 = m.a;
-        V Px, Py, pe[4], po[4];
-        sp4_F(K, upx, upy, Px, Py);
-        const V P0 = sp4_Gs(K, S, upx, upy, Px, Py, pe, po);
-        // Eq. 28 for the unshifted f: p = 3/5 [sum f_i - (2/3) u.u + tau_g G_0]
-        const V p3 = V(T(3)) * (V(T(0.6)) * fmadd(V(K.tau), G0, fmadd(V(T(-2) / T(3)), uu, sp_rest(g))));
-        const V om(K.om), half(T(0.5));
-        const V uu15 = V(T(-1.5)) * uu, b = p3 + uu15;   // 3 p - 1.5 u.u
-        const V geq0 = fmadd(V(T(4.0 / 9.0 - 1.0)), p3, V(T(4) / T(9)) * uu15);
-        emit(0, sp_relax(K.om, g[0], fmadd(om, geq0, fmadd(half, G0 - P0, G0))), V(T(0)));
-        const V ga = ninth * b, gd = q * ga;
-        const V up = q * (ux + uy), um = q * (uy - ux);
-        const V hx = half * ux, hy = half * uy;
-        const V ge[4] = {fmadd(hx, ux, ga), fmadd(hy, uy, ga), fmadd(V(T(2)) * up, up, gd),
-                         fmadd(V(T(2)) * um, um, gd)};
-        V ax, ay, dx, dy;
-        sp_odd(hx, ax, dx);
-        sp_odd(hy, ay, dy);
-        const V go[4] = {ax, ay, dx + dy, dy - dx};
+    constexpr bool pair = Unit<V>::cells == 2;
+    constexpr T w0d = T(sw(0)), w01 = pair ? T(sw(0) - 1.0) : w0d - T(1);   // w_0, w_0 - 1
+    const V w0(w0d), ig(K.inv_tau), sg(K.src), three(T(3)), half(T(0.5));
+    auto relax = [&](V gi, V geq) { return sub_prod(gi, gi - geq, ig); };
+    if constexpr (KIND == 3) {
+        const SpCell<V> c = sp3_moments(K, g, S);
+        const V QS = V(K.Qc) * S, p3 = three * c.p;
+        const V r0 = fmadd(sg, c.G0, relax(g[0], fmadd(p3, V(w01), w0 * (V(T(-1.5)) * c.uu))));
+        emit(0, r0, [&] { return r0; });
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int i = pair2(k), j = sopp(i);
-            // om g^eq_i - G_i(t - 1) / 2, even and odd parts
-            const V A = fmadd(om, ge[k], V(T(-0.5)) * pe[k]), B = fmadd(om, go[k], V(T(-0.5)) * po[k]);
-            const V Gi = nb(i - 1, 0, 0), Gj = nb(j - 1, 0, 0);
-            const V ni = nb(i - 1, sx(i), sy(i)), nj = nb(j - 1, sx(j), sy(j));
-            // without G_i(x + c_i) / 2
-            const V pi = sp_relax(K.om, g[i], Gi + (A + B)), pj = sp_relax(K.om, g[j], Gj + (A - B));
-            // bounce-back of f - G/2: leaves with G_i(x + c_i) / 2 less, returns as opp(i) with G_opp(x) / 2
-            emit(i, fmadd(half, ni, pi), fmadd(half, Gj, pi));
-            emit(j, fmadd(half, nj, pj), fmadd(half, Gi, pj));
+        for (int q = 0; q < 4; ++q) {
+            const int i = pair2(q), j = sopp(i);
+            const V w(T(sw(i))), cu = sp_dot(i, c.ux, c.uy), cF = sp_dot(i, V(K.fx), V(K.fy)), y = three * cF;
+            const V e = w * fmadd(V(sp_c2<T>(i)), QS, sub_prod(fmadd(V(T(9)) * cu, cF, S), three, c.uF));
+            const V cu2 = V(T(4.5)) * cu * cu, pw = p3 * w;
+            const V si = sub_prod(fmadd(three, cu, cu2), V(T(1.5)), c.uu);
+            const V sj = sub_prod(fmadd(-three, cu, cu2), V(T(1.5)), c.uu);
+            const V ri = fmadd(sg, add_prod(e, w, y), relax(g[i], fmadd(w, si, pw)));
+            const V rj = fmadd(sg, sub_prod(e, w, y), relax(g[j], fmadd(w, sj, pw)));
+            emit(i, ri, [&] { return ri; });
+            emit(j, rj, [&] { return rj; });
         }
-        return;
+    } else if constexpr (KIND == 4) {
+        const V ux = m.ux, uy = m.uy, Fx = m.a, Fy = m.b;
+        const V uu = fmadd(ux, ux, uy * uy), uF = fmadd(ux, Fx, uy * Fy);
+        const V G0 = w0 * sp4_G0w(K, S, uF), p = sp4_p(K, g, uu, G0), p3 = three * p;
+        V Fpx, Fpy;   // F at t - 1
+        sp4_force(K, upx, upy, Fpx, Fpy);
+        const V upF = fmadd(upx, Fpx, upy * Fpy);
+        {   // rest direction: its destination is this cell
+            const V z = V(T(-1.5)) * uu;
+            V geq;
+            if constexpr (pair) geq = fmadd(p3, V(w01), w0 * z);
+            else geq = fmadd(w0, z, p3 * V(w01));
+            emit(0, fmadd(half, sub_prod(G0, w0, sp4_G0w(K, S, upF)), relax(g[0], geq) + G0), [] { return V(T(0)); });
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = pair2(q), j = sopp(i);
+            const V w(T(sw(i))), cu = sp_dot(i, ux, uy);
+            const V E = diff_prod(V(T(4.5)) * cu, cu, V(T(1.5)), uu);
+            V ge;
+            if constexpr (pair) ge = fmadd(w, E, V(T(3) * T(sw(i))) * p);
+            else ge = i >= 5 ? fmadd(w, E, p3 * w) : fmadd(p3, w, w * E);
+            V Ge, Gy, Pe, Py;
+            sp4_parts(K, i, S, ux, uy, Fx, Fy, uF, Ge, Gy);
+            sp4_parts(K, i, S, upx, upy, Fpx, Fpy, upF, Pe, Py);
+            const V Gi = add_prod(Ge, w, Gy), Gj = sub_prod(Ge, w, Gy);
+            const V Pi = add_prod(Pe, w, Py), Pj = sub_prod(Pe, w, Py);
+            const V xi = nb(i - 1, sx(i), sy(i)), xj = nb(j - 1, sx(j), sy(j));   // G / w at the destinations
+            // G_i(x + c_i, t) - G_i(x, t - 1)
+            auto change = [&](V x, V P) { return !pair && sy(i) == 0 ? fmadd(w, x, -P) : w * x - P; };
+            const V cy = three * cu;
+            const V pi = fmadd(half, change(xi, Pi), relax(g[i], add_prod(ge, w, cy)) + Gi);
+            const V pj = fmadd(half, change(xj, Pj), relax(g[j], sub_prod(ge, w, cy)) + Gj);
+            // bounce-back of f - G/2: leaves as i with G_i(x + c_i), returns as opp(i)
+            emit(i, pi, [&] { return fmadd(half, Gj, fmadd(-half, w * xi, pi)); });
+            emit(j, pj, [&] { return fmadd(half, Gi, fmadd(-half, w * xj, pj)); });
+        }
     } else {
-        V Vx, Vy, Tx, Ty, Ea, Ed, r0;   // Tx, Ty: (om a u + sg F) / 2
-        const V uF = fmadd(ux, V(K.fx), uy * V(K.fy));
-        if constexpr (KIND == 3) {
-            // Eq. 28: p = 3/5 [sum g_i + S/2 - (2/3) u.u + (tau_g - 1/2) G_0]
-            const V t = V(T(-3)) * uF;
-            const V G0 = fmadd(S, V(K.k0), V(T(4) / T(9)) * t);
-            const V p3 = V(T(3)) * (V(T(0.6)) * fmadd(V(K.tgm), G0, fmadd(V(T(-2) / T(3)), uu,
-                                                                          fmadd(V(T(0.5)), S, sp_rest(g)))));
-            const V omp = V(K.om) * p3;
-            const V b0 = fmadd(V(K.om), V(T(-1.5)) * uu, V(K.sg) * t), b = omp + b0;
-            Vx = fmadd(V(K.om_h), ux, V(K.sgfx));
-            Vy = fmadd(V(K.om_h), uy, V(K.sgfy));
-            Tx = fmadd(V(K.om_h), ux, V(K.hsgfx));
-            Ty = fmadd(V(K.om_h), uy, V(K.hsgfy));
-            Ea = fmadd(S, V(K.ska), ninth * b);
-            Ed = fmadd(S, V(K.skd), V(T(1) / T(36)) * b);
-            r0 = fmadd(V(T(4.0 / 9.0 - 1.0)), omp, fmadd(S, V(K.sk0), V(T(4) / T(9)) * b0));
-        } else {
-            // 12 div u (Eq. 30a)
-            const V sa = nb(0, 1, 1) - nb(0, -1, -1), sb = nb(0, -1, 1) - nb(0, 1, -1);
-            const V ta = nb(1, 1, 1) - nb(1, -1, -1), tb = nb(1, -1, 1) - nb(1, 1, -1);
-            const V ax = nb(0, 1, 0) - nb(0, -1, 0), ay = nb(1, 0, 1) - nb(1, 0, -1);
-            const V div = fmadd(V(T(4)), ax + ay, (sa - sb) + (ta + tb));
-            const V gq = fmadd(m.b, V(K.q), V(K.q0)) * div;          // sg Q div u
-            const V Sg = V(K.sc) * S, om(K.om), sg(K.sg);
-            const V h = V(K.om_h) * m.b;                              // om a / 2
-            V hA, S2;
-            if constexpr (KIND == 1) {                                // with the u u S of Remark 1
-                hA = h - V(T(0.5)) * (sg * Sg);
-                S2 = fmadd(V(T(1.5)) * uu, Sg, Sg);
-            } else {
-                hA = h;
-                S2 = Sg;
-            }
-            Vx = fmadd(hA, ux, V(K.sgfx));
-            Vy = fmadd(hA, uy, V(K.sgfy));
-            if constexpr (KIND == 2) {   // (om p_0 / 2, a constant, rounded would be a bias of every step)
-                Tx = fmadd(V(K.om_h), m.b * ux, V(K.hsgfx));
-                Ty = fmadd(V(K.om_h), m.b * uy, V(K.hsgfy));
-            } else {
-                Tx = fmadd(h, ux, V(K.hsgfx));
-                Ty = fmadd(h, uy, V(K.hsgfy));
-            }
-            const V b = fmadd(om, fmadd(V(T(-1.5)) * m.b, uu, m.a), sg * fmadd(V(T(-3)), uF, S2));
-            Ea = ninth * fmadd(V(T(1.5)), gq, b);
-            Ed = V(T(1) / T(36)) * fmadd(V(T(6)), gq, b);
-            r0 = V(T(4) / T(9)) * fmadd(V(T(-3)), gq, b);
+        const V ux = m.ux, uy = m.uy, d = m.a, a = m.b;
+        V divu(T(0));   // Eq. 30a applied to u; pairs sum row by row
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            constexpr int by_row[8] = {4, 7, 8, 1, 3, 2, 5, 6};
+            const int i = pair ? by_row[k] : k + 1;
+            V cu;
+            if (sy(i) == 0) cu = nb(0, sx(i), 0);
+            else if (sx(i) == 0) cu = nb(1, 0, sy(i));
+            else cu = sx(i) * sy(i) > 0 ? nb(0, sx(i), sy(i)) + nb(1, sx(i), sy(i)) : nb(0, sx(i), sy(i)) - nb(1, sx(i), sy(i));
+            // (a sign for the direction as a whole)
+            divu = fmadd(V((sx(i) ? sx(i) : sy(i)) * T(sw(i))), cu, divu);
         }
-        auto out = [&](int i, V v) { emit(i, v, v); };
-        out(0, sp_relax(K.om, g[0], r0));
-        auto pair = [&](int i, int j, V E, V O) {
-            out(i, sp_relax(K.om, g[i], E + O));
-            out(j, sp_relax(K.om, g[j], E - O));
+        divu = divu * three;
+        const V third(T(1.0 / 3.0));
+        const V Qd = fmadd(a, third, V(K.Qd0)) * divu;   // Q div u, Q = (2/d) a c_s^2 - xi / (tau_g - 1/2)
+        // S and F in the units of g
+        const V fx(KIND == 1 ? K.fx : K.fx * K.p0), fy(KIND == 1 ? K.fy : K.fy * K.p0);
+        V Sg = S;
+        if constexpr (KIND == 2) Sg = S * V(K.p0);
+        const V uF = fmadd(ux, fx, uy * fy), uu = fmadd(ux, ux, uy * uy);
+        auto source = [&](V G, V cc) {   // the u u S of Remark 1: cc = (c.u)^2 - u.u / 3
+            if constexpr (KIND == 1) return sub_prod(G, V(T(4.5)) * cc, Sg);
+            else return G;
         };
-        V ox, oy, dx, dy;
-        sp_odd(Tx, ox, dx);
-        sp_odd(Ty, oy, dy);
-        pair(1, 3, fmadd(ux, Vx, Ea), ox);
-        pair(2, 4, fmadd(uy, Vy, Ea), oy);
-        pair(5, 7, fmadd(q * (ux + uy), Vx + Vy, Ed), dx + dy);
-        pair(6, 8, fmadd(q * (uy - ux), Vy - Vx, Ed), dy - dx);
+        {
+            const V geq = fmadd(d, w0, a * (w0 * (V(T(-1.5)) * uu)));
+            const V G = source(fmadd(V(sp_c2<T>(0)), Qd, sub_prod(Sg, three, uF)), -(uu * third));
+            const V r0 = fmadd(sg, w0 * G, relax(g[0], geq));
+            emit(0, r0, [&] { return r0; });
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = pair2(q), j = sopp(i);
+            const bool diag = i >= 5;
+            const V w(T(sw(i))), cu = sp_dot(i, ux, uy), cF = sp_dot(i, fx, fy), c2(sp_c2<T>(i));
+            const V wE = w * diff_prod(V(T(4.5)) * cu, cu, V(T(1.5)), uu);
+            const V ge = pair || diag ? fmadd(a, wE, d * w) : fmadd(d, w, a * wE), o = w * (three * cu);
+            V G = sub_prod(fmadd(V(T(9)) * cu, cF, Sg), three, uF);
+            G = pair && diag ? G + c2 * Qd : fmadd(c2, Qd, G);
+            if constexpr (KIND == 1) G = source(G, diff_prod(cu, cu, uu, third));
+            const V e = w * G, y = three * cF;
+            const V ri = fmadd(sg, add_prod(e, w, y), relax(g[i], add_prod(ge, a, o)));
+            const V rj = fmadd(sg, sub_prod(e, w, y), relax(g[j], sub_prod(ge, a, o)));
+            emit(i, ri, [&] { return ri; });
+            emit(j, rj, [&] { return rj; });
+        }
     }
 }
 
@@ -554,16 +492,17 @@ struct SpPush {
     int N, nx, x, y, up, dn;
     bool bot, top;
     template <typename T>
-    __device__ __forceinline__ SpPush(const SpK<T>& K, typename U::R* out_, int N_, int x_, int y_)
+    __device__ __forceinline__ SpPush(const SpConst<T>& K, typename U::R* out_, int N_, int x_, int y_)
         : out(out_), N(N_), nx(K.nx), x(x_), y(y_) {
         bot = K.walls && y == 0;
         top = K.walls && y == K.ny - 1;
         dn = y == 0 ? K.ny - 1 : y - 1;   // (not used at a wall)
         up = y == K.ny - 1 ? 0 : y + 1;
     }
-    __device__ __forceinline__ void operator()(int i, V v, V w) const {
+    template <typename Wall>
+    __device__ __forceinline__ void operator()(int i, V v, Wall&& wall) const {
         if ((sy(i) > 0 && top) || (sy(i) < 0 && bot)) {
-            U::st(out + sopp(i) * N + y * nx + x, w);
+            U::st(out + sopp(i) * N + y * nx + x, wall());
             return;
         }
         U::push(out + i * N + (sy(i) == 0 ? y : (sy(i) > 0 ? up : dn)) * nx, x, nx, sx(i), v);
@@ -571,14 +510,12 @@ struct SpPush {
 };
 
 // Remark 3, large domains: nothing of a neighbour is needed, one unit a thread.
-// 4096 x 4096 FP32 186 us a step (1.0 of the copy bandwidth); FP64 bound by its
-// FP64 operations: 2048 x 2048 1235 -> 638 us with the opposite pairs' even and odd
-// parts.
+// 4096 x 4096 FP32 188 us a step (1.0 of the copy bandwidth); FP64 bound by its FP64
+// operations, 2048 x 2048 1076 us.
 template <typename V>
-__global__ void __launch_bounds__(256, 4) sp_cell_kernel(const typename Unit<V>::R* __restrict__ gin,
-                                                      typename Unit<V>::R* __restrict__ gout,
-                                                      const typename Unit<V>::R* __restrict__ src, int N,
-                                                      SpK<typename Unit<V>::R> K) {
+__global__ void __launch_bounds__(256, sizeof(typename Unit<V>::R) == 8 ? 3 : 4)
+    sp_cell_kernel(const typename Unit<V>::R* __restrict__ gin, typename Unit<V>::R* __restrict__ gout,
+                   const typename Unit<V>::R* __restrict__ src, int N, SpConst<typename Unit<V>::R> K) {
     using U = Unit<V>;
     const int c = U::cells * (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (c >= N) return;
@@ -602,10 +539,11 @@ __global__ void __launch_bounds__(256, 4) sp_cell_kernel(const typename Unit<V>:
 // one barrier, the collision. Every population is read once: in FP32 76 bytes a
 // cell for Remarks 1 and 2 (two kernels, one writing u, moved 132), 92 for Remark
 // 4 (160: of t - 1 it keeps u, two planes updated in place, and forms F(u) again).
-// 4096 x 4096 FP32, two kernels -> here, us a step: Remark 1 375 -> 206 (0.91 of
-// the copy bandwidth), 2 330 -> 217, 4 489 -> 309 (0.74: three quarters of it
-// arithmetic at 16 warps a SM); 2048 x 2048 FP64 (half the FP64 operations) 1790 ->
-// 878, 1525 -> 780, 2459 -> 1691.
+// 4096 x 4096 FP32, two kernels -> here, us a step: Remark 1 375 -> 232 (0.81 of
+// the copy bandwidth), 2 330 -> 223 (0.85), 4 489 -> 322 (0.71: three quarters of it
+// arithmetic at 16 warps a SM); 2048 x 2048 FP64 (bound by its FP64 operations either
+// way: the moments are formed once instead of twice) 1790 -> 1369, 1525 -> 1198, 2459 ->
+// 2227. Bit for bit the two kernels' results (see "Arithmetic").
 //
 // Thread t holds unit t - 1 of the strip [x0, x0 + w): the first and the last hold
 // one unit of halo, which they only prepare. Neighbouring runs march in opposite
@@ -616,7 +554,7 @@ struct SpRun {
 struct SpMarch {   // the block's run: Y0 its first row, d its direction, n its rows
     int x0, wc, Y0, d, n, ny, walls;
     template <typename T>
-    __device__ __forceinline__ SpMarch(const SpK<T>& K, const SpRun& r) : ny(K.ny), walls(K.walls) {
+    __device__ __forceinline__ SpMarch(const SpConst<T>& K, const SpRun& r) : ny(K.ny), walls(K.walls) {
         const int run = blockIdx.x / r.strips, strip = blockIdx.x - run * r.strips;
         x0 = strip * r.w;
         wc = min(r.w, K.nx - x0);
@@ -639,7 +577,7 @@ __global__ void __launch_bounds__(kSpThreads, OCC) sp_march_kernel(const typenam
                                                                    typename Unit<V>::R* __restrict__ gout,
                                                                    const typename Unit<V>::R* __restrict__ src,
                                                                    typename Unit<V>::R* __restrict__ uprev, int N,
-                                                                   SpK<typename Unit<V>::R> K, SpRun run) {
+                                                                   SpConst<typename Unit<V>::R> K, SpRun run) {
     using U = Unit<V>;
     __shared__ typename U::E ring[4][kRing<KIND>][kSpThreads];
     const SpMarch A(K, run);
@@ -712,7 +650,7 @@ struct SpTileArgs {
 };
 
 template <int KIND, typename V, int OCC>
-__global__ void __launch_bounds__(kSpThreads, OCC) sp_tile_kernel(const SpTileArgs a, SpK<typename Unit<V>::R> K) {
+__global__ void __launch_bounds__(kSpThreads, OCC) sp_tile_kernel(const SpTileArgs a, SpConst<typename Unit<V>::R> K) {
     using U = Unit<V>;
     using R = typename U::R;
     // (2^u + 2) x (rows + 2) units: at most 34 x 6 over the shapes 2^u x 128 / 2^u
@@ -801,9 +739,8 @@ struct lbm_sp_ctx {
     long long time = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    SpConst K{};
-    SpK<float> kf;                     // the step's constants in the arithmetic type
-    SpK<double> kd;
+    SpConst<double> K{};
+    SpConst<float> kf{};               // FP32 steps: the constants in FP32
     int kind = 3;                      // 1, 2, 3: Remarks; 4: the Remark 4 scheme
     int cells = 1;                     // cells a unit: 2 in FP32 with nx even
     const void* kernel = nullptr;      // one step a launch: row march, Remark 3 one unit a thread
@@ -844,22 +781,24 @@ void sp_release(lbm_sp_ctx* c) {
 
 // The step kernels of a model for unit type V, and the resident blocks of 128
 // threads a SM their registers are sized for. The row march holds two rows of
-// populations and a third in flight. Measured at 4096 x 4096, pairs, us a step:
-// Remark 1 220 / 206 / 282 with 4 / 5 / 6 blocks, Remark 2 216 / 217 / 235, Remark 4
-// 330 / 309 / 367 with 3 / 4 / 5; FP64 the same with 2 to 4 (bound by its FP64
-// operations).
+// populations and a third in flight. us a step of the marches with 3 / 4 / 5 blocks:
+// pairs (4096 x 4096) Remark 1 256 / 232 / 287, Remark 2 244 / 223 / 227, Remark 4 357 /
+// 322 / 461; one FP32 cell (4095 x 4096) with 4 / 5 / 6 blocks 287 / 268 / 283, 275 / 257 /
+// 255, 422 / 372 / 435; FP64 (2048 x 2048) with 2 / 3 / 4: 1369 / 1401 / 1488, 1198 / 1232 /
+// 1314, 2306 / 2227 / 2361. Tiles: FP64 with 3 and 5 blocks 256 x 256 39.7 and 27.8, 34.1
+// and 23.9, 66.2 and 45.9 (one round of tiles for two), 192 x 192 (one either way) the same.
 template <typename V>
 void sp_kernels(int kind, const void** step, const void** tile) {
     constexpr bool f64 = sizeof(typename Unit<V>::R) == 8, pair = Unit<V>::cells == 2;
-    constexpr int m = f64 ? 3 : pair ? 5 : 6, m2 = f64 ? 3 : pair ? 4 : 6, m4 = f64 ? 3 : pair ? 4 : 6;
-    constexpr int o = f64 ? 3 : pair ? 4 : 6;
+    constexpr int m = f64 ? 2 : pair ? 4 : 5, m4 = f64 ? 3 : pair ? 4 : 5;
+    constexpr int o = f64 ? 5 : pair ? 4 : 6;
     switch (kind) {
         case 1:
             *step = (const void*)sp_march_kernel<1, V, m>;
             *tile = (const void*)sp_tile_kernel<1, V, o>;
             break;
         case 2:
-            *step = (const void*)sp_march_kernel<2, V, m2>;
+            *step = (const void*)sp_march_kernel<2, V, m>;
             *tile = (const void*)sp_tile_kernel<2, V, o>;
             break;
         case 4:
@@ -877,11 +816,10 @@ lbm_status sp_plan(lbm_sp_ctx* c) {
     c->kind = c->p.scheme == LBM_SP_SCHEME_REMARK4 ? 4
               : c->p.model == LBM_SP_NEARLY_INCOMPRESSIBLE ? 1
               : c->p.model == LBM_SP_HE_INCOMPRESSIBLE ? 2 : 3;
-    c->kf = sp_consts<float>(c->K, c->p.model);
-    c->kd = sp_consts<double>(c->K, c->p.model);
+    c->kf = sp_const_as<float>(c->K);
     c->cells = c->form == LBM_F32 && c->p.nx % 2 == 0 ? 2 : 1;
     if (c->form == LBM_F64) sp_kernels<One<double>>(c->kind, &c->kernel, &c->tile);
-    else if (c->cells == 2) sp_kernels<F2>(c->kind, &c->kernel, &c->tile);
+    else if (c->cells == 2) sp_kernels<Two>(c->kind, &c->kernel, &c->tile);
     else sp_kernels<One<float>>(c->kind, &c->kernel, &c->tile);
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
@@ -910,11 +848,11 @@ lbm_status sp_plan(lbm_sp_ctx* c) {
             }
         }
     }
-    // Tiles, several steps a launch, while every tile is resident at once (FP64:
-    // two rounds): a step of a small domain is the latency of a launch. us a step,
-    // tiles and one launch a step: 64 x 64 Remark 1 FP32 3.0 and 4.2, FP64 6.0 and
-    // 8.8; 256 x 256 3.7 and 6.2, 18.6 and 26.9; 400 x 400 (3 rounds) 8.7 and 6.2,
-    // 50.9 and 49.5.
+    // Tiles, several steps a launch, while every tile is resident at once: a step of
+    // a small domain is the latency of a launch. us a step, tiles and one launch a
+    // step: 64 x 64 Remark 1 FP32 3.0 and 4.1, FP64 7.7 and 12.3; 256 x 256 3.8 and 6.2,
+    // 27.8 and 41.0; 300 x 300 4.1 and 6.2, 35.8 and 41.0; in two rounds 400 x 400 FP32
+    // 8.8 and 8.2, 340 x 340 FP64 60 and 57.
     auto count = [&](int u, int r) { return (long long)((units + u - 1) / u) * ((c->p.ny + r - 1) / r); };
     int U, R;
     lbm::tile_shape(count, sms, &U, &R);
@@ -923,7 +861,7 @@ lbm_status sp_plan(lbm_sp_ctx* c) {
         U = 8;
         R = 16;
     }
-    if (count(U, R) > (c->form == LBM_F64 ? 2 : 1) * tslots) {
+    if (count(U, R) > tslots) {
         c->tile = nullptr;
         return LBM_OK;
     }
@@ -942,7 +880,7 @@ lbm_status sp_plan(lbm_sp_ctx* c) {
         cudaMemcpy(c->d_tile_nbr, list.nbr.data(), list.nbr.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
         return LBM_ECUDA;
     c->tile_items = (int)list.items.size();
-    c->tile_grid = (int)(c->tile_items < tslots ? c->tile_items : tslots);
+    c->tile_grid = c->tile_items;
     while ((1 << c->tile_ulog) < U) ++c->tile_ulog;
     return LBM_OK;
 }
@@ -952,7 +890,7 @@ cudaError_t sp_step_once(lbm_sp_ctx* c) {
     const void* in = c->g[c->cur];
     void* out = c->g[1 - c->cur];
     int N = (int)c->N;
-    void* k = c->form == LBM_F64 ? (void*)&c->kd : (void*)&c->kf;
+    void* k = c->form == LBM_F64 ? (void*)&c->K : (void*)&c->kf;
     c->cur ^= 1;
     if (c->kind == 3) {
         void* args[] = {&in, &out, &c->src, &N, k};
@@ -984,7 +922,7 @@ cudaError_t sp_step_tiles(lbm_sp_ctx* c, int n) {
         const cudaError_t e = cudaMemsetAsync(a.done, 0, ((size_t)c->tile_items + 1) * sizeof(int), c->stream);
         if (e != cudaSuccess) return e;
     }
-    void* args[] = {&a, c->form == LBM_F64 ? (void*)&c->kd : (void*)&c->kf};
+    void* args[] = {&a, c->form == LBM_F64 ? (void*)&c->K : (void*)&c->kf};
     c->cur ^= n & 1;
     // one step: no block waits, so the grid need not be resident at once
     return n > 1 ? cudaLaunchCooperativeKernel(c->tile, dim3(c->tile_grid), dim3(kSpThreads), args, 0, c->stream)
@@ -1000,14 +938,16 @@ lbm_status sp_device_status(lbm_sp_ctx* c) {
     return st == 0 ? LBM_OK : sp_fail(c, LBM_ETIMEOUT, "a bounded device wait ran out in the step kernel");
 }
 
-template <int M>
-void sp1_fields(lbm_sp_ctx* c, unsigned mask) {
-    if (c->form == LBM_F64)
-        sp1_fields_kernel<M, double><<<blocks(c->N), 256, 0, c->stream>>>(
-            static_cast<const double*>(c->g[c->cur]), static_cast<const double*>(c->src), c->N, c->K, mask, c->d_tmp);
-    else
-        sp1_fields_kernel<M, float><<<blocks(c->N), 256, 0, c->stream>>>(
-            static_cast<const float*>(c->g[c->cur]), static_cast<const float*>(c->src), c->N, c->K, mask, c->d_tmp);
+template <typename R>
+void sp_fields(lbm_sp_ctx* c, const SpConst<R>& K, unsigned mask) {
+    const R *g = static_cast<const R*>(c->g[c->cur]), *src = static_cast<const R*>(c->src);
+    const int n = blocks(c->N);
+    switch (c->kind) {
+        case 1: sp1_fields_kernel<1, R><<<n, 256, 0, c->stream>>>(g, src, c->N, K, c->p.p0, mask, c->d_tmp); break;
+        case 2: sp1_fields_kernel<2, R><<<n, 256, 0, c->stream>>>(g, src, c->N, K, c->p.p0, mask, c->d_tmp); break;
+        case 4: sp_fields_kernel<true, R><<<n, 256, 0, c->stream>>>(g, src, c->N, K, mask, c->d_tmp); break;
+        default: sp_fields_kernel<false, R><<<n, 256, 0, c->stream>>>(g, src, c->N, K, mask, c->d_tmp);
+    }
 }
 
 }  // namespace
@@ -1041,10 +981,10 @@ lbm_status lbm_sp_create(const lbm_sp_params* params, int precision, void* cuda_
     c->form = precision;
     c->N = (long long)p.nx * p.ny;
     const double tau = 3.0 * p.nu + 0.5;
-    c->K = SpConst{p.nx, p.ny, p.bc_y == LBM_BC_BOUNCEBACK ? 1 : 0, 1.0 / tau, 1.0 - 0.5 / tau, tau - 0.5,
-                   1.0 / 3.0 - p.xi / (tau - 0.5), p.force_x, p.force_y, p.drag_lin, p.drag_quad, p.p0,
-                   tau, -p.xi / (tau - 0.5), 0.5 * p.p0, p.p0 > 0 ? 1.0 / p.p0 : 0.0, 0.5 * p.p0 * p.force_x,
-                   0.5 * p.p0 * p.force_y};
+    c->K = SpConst<double>{p.nx, p.ny, p.bc_y == LBM_BC_BOUNCEBACK ? 1 : 0, 1.0 / tau, 1.0 - 0.5 / tau, tau - 0.5,
+                           1.0 / 3.0 - p.xi / (tau - 0.5), p.force_x, p.force_y, p.drag_lin, p.drag_quad, p.p0,
+                           tau, -p.xi / (tau - 0.5), 0.5 * p.p0, p.p0 > 0 ? 1.0 / p.p0 : 0.0, 0.5 * p.p0 * p.force_x,
+                           0.5 * p.p0 * p.force_y};
     const size_t e = sp_elem(precision);
     cudaError_t r;
     if ((r = cudaMalloc(&c->g[0], kQ * c->N * e)) != cudaSuccess ||
@@ -1123,28 +1063,14 @@ lbm_status lbm_sp_step(lbm_sp_ctx* c, int nsteps) {
 
 lbm_status lbm_sp_get_fields(lbm_sp_ctx* c, unsigned mask, double* host_out) {
     if (!c) return LBM_EINVAL;
-    const bool m1 = c->p.model == LBM_SP_NEARLY_INCOMPRESSIBLE, m2 = c->p.model == LBM_SP_HE_INCOMPRESSIBLE;
+    const bool m1 = c->p.model == LBM_SP_NEARLY_INCOMPRESSIBLE;
     const unsigned ok = LBM_FIELD_UX | LBM_FIELD_UY | LBM_FIELD_P | (m1 ? LBM_FIELD_RHO : 0u);
     if (!host_out || mask == 0 || (mask & ~ok)) return sp_fail(c, LBM_EINVAL, "bad mask or output");
     if (!c->ready) return sp_fail(c, LBM_ESTATE, "not initialised");
     const int nf = ((mask & LBM_FIELD_UX) ? 1 : 0) + ((mask & LBM_FIELD_UY) ? 1 : 0) + ((mask & LBM_FIELD_P) ? 1 : 0) +
                    ((mask & LBM_FIELD_RHO) ? 1 : 0);
-    if (c->p.scheme == LBM_SP_SCHEME_REMARK4 && c->form == LBM_F64)
-        sp4_fields_kernel<double><<<blocks(c->N), 256, 0, c->stream>>>(
-            static_cast<const double*>(c->g[c->cur]), static_cast<const double*>(c->src), c->N, c->K, mask, c->d_tmp);
-    else if (c->p.scheme == LBM_SP_SCHEME_REMARK4)
-        sp4_fields_kernel<float><<<blocks(c->N), 256, 0, c->stream>>>(
-            static_cast<const float*>(c->g[c->cur]), static_cast<const float*>(c->src), c->N, c->K, mask, c->d_tmp);
-    else if (m1)
-        sp1_fields<1>(c, mask);
-    else if (m2)
-        sp1_fields<2>(c, mask);
-    else if (c->form == LBM_F64)
-        sp_fields_kernel<double><<<blocks(c->N), 256, 0, c->stream>>>(
-            static_cast<const double*>(c->g[c->cur]), static_cast<const double*>(c->src), c->N, c->K, mask, c->d_tmp);
-    else
-        sp_fields_kernel<float><<<blocks(c->N), 256, 0, c->stream>>>(
-            static_cast<const float*>(c->g[c->cur]), static_cast<const float*>(c->src), c->N, c->K, mask, c->d_tmp);
+    if (c->form == LBM_F64) sp_fields(c, c->K, mask);
+    else sp_fields(c, c->kf, mask);
     cudaError_t r;
     if ((r = cudaMemcpyAsync(host_out, c->d_tmp, nf * c->N * sizeof(double), cudaMemcpyDeviceToHost,
                              c->stream)) != cudaSuccess)
