@@ -383,6 +383,7 @@ int march_rows(int ny, int strips, long long target, long long* cost) {
 }
 
 lbm_status plan(lbm_ctx* c) {
+    c->multi = false;   // (plan_multi sets it for the plans that it makes; the batched plan does not come to it)
     if (c->d3) return plan_d3(c);
     const int tiles[4] = {32, 64, 128, 256};
     auto tile_index = [&](int tx) {
@@ -555,7 +556,6 @@ lbm_status multi_monitor(lbm_ctx* c) {
 }
 
 lbm_status plan_multi(lbm_ctx* c, int sms) {
-    c->multi = false;
     const bool by_default = c->pipeline == LBM_PIPELINE_AUTO && c->n == 1 && !c->tile_req && !c->rows_req;
     if (c->d3 || !(c->pipeline == LBM_PIPELINE_PERSISTENT || by_default) || c->launches.size() != 1 ||
         c->launches[0].variant != lbm::kPairs)
@@ -1115,7 +1115,9 @@ cudaError_t enqueue_batched(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, 
 }
 
 // The plan runs several steps a launch, one block per work item (plan_multi).
-bool multi_plan(const lbm_ctx* c) { return c->multi && !c->d3 && c->launches.size() == 1; }
+bool multi_plan(const lbm_ctx* c) {
+    return c->multi && !c->d3 && c->launches.size() == 1 && c->launches[0].variant == lbm::kPairs;
+}
 
 // Queues `nsteps` steps of a persistent plan as one cooperative launch, the
 // first reading buffer set `in`, after zeroing the per-item step counters and
