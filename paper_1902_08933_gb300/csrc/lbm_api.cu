@@ -13,6 +13,7 @@
 #include "lbm.h"
 #include "lbm_internal.h"
 #include "lbm_mbar.cuh"
+#include "lbm_monbuf.h"
 #include "lbm_tileplan.h"
 
 using lbm::AuxArgs;
@@ -176,9 +177,7 @@ struct lbm_ctx {
     int graph_launches = 0;        // kernel nodes of the captured graph
     int* d_nbr = nullptr;          // persistent plan: neighbour items, kMaxTileNbr an item
     int* d_multi_done = nullptr;   // persistent plan: steps finished per item, then the abort flag
-    double* d_mon_multi = nullptr; // persistent plan, every step monitored: [64 steps][items][kMonQ] slots
-    int* d_mon_multi_cnt = nullptr;   // ... [64 steps][instances][kMonSub + 1] counters
-    double* d_mon_multi_sub = nullptr;  // ... and [64 steps][instances][kMonSub][kMonQ] sub-group slots
+    lbm::MultiMonitor mon_multi;   // persistent plan, every step of a launch monitored (kMultiSteps of them)
     // tile plan (plan_tile): items, neighbours and step counters in one allocation
     int tile_items = 0, tile_grid = 0, tile_ulog = 0, tile_occ = 0;
     bool tile_pair = false;
@@ -544,15 +543,15 @@ lbm_status plan_batched(lbm_ctx* c, bool, bool, bool, int sms) {
 // steps of one monitored persistent launch (slots and counters are kept per step)
 constexpr int kMultiSteps = 64;
 
-// Buffers of the records of every step of a persistent launch.
-lbm_status multi_monitor(lbm_ctx* c) {
-    if (!c->multi || c->d_mon_multi) return LBM_OK;
-    const size_t items = c->launches[0].count;
-    LBM_CK(c, cudaMalloc(&c->d_mon_multi, (size_t)kMultiSteps * items * lbm::kMonQ * sizeof(double)));
-    LBM_CK(c, cudaMalloc(&c->d_mon_multi_cnt, (size_t)kMultiSteps * c->n * (lbm::kMonSub + 1) * sizeof(int)));
-    LBM_CK(c, cudaMalloc(&c->d_mon_multi_sub,
-                         (size_t)kMultiSteps * c->n * lbm::kMonSub * lbm::kMonQ * sizeof(double)));
-    return LBM_OK;
+// Buffers of the records of every step of a persistent launch. Where they cannot be
+// had, every step is a monitored launch of its own.
+void multi_monitor(lbm_ctx* c) {
+    if (!c->multi || c->mon_multi.slots) return;
+    c->mon_multi.allocate(kMultiSteps, c->launches[0].count, c->n, [](void** p, size_t bytes) {
+        if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    });
 }
 
 lbm_status plan_multi(lbm_ctx* c, int sms) {
@@ -598,17 +597,14 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
     c->d_nbr = nullptr;
     cudaFree(c->d_multi_done);
     c->d_multi_done = nullptr;
-    cudaFree(c->d_mon_multi);
-    c->d_mon_multi = nullptr;
-    cudaFree(c->d_mon_multi_cnt);
-    c->d_mon_multi_cnt = nullptr;
-    cudaFree(c->d_mon_multi_sub);
-    c->d_mon_multi_sub = nullptr;
+    cudaFree(c->mon_multi.slots);
+    c->mon_multi = lbm::MultiMonitor();
     LBM_CK(c, cudaMalloc(&c->d_nbr, nbr.size() * sizeof(int)));
     LBM_CK(c, cudaMemcpy(c->d_nbr, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice));
     LBM_CK(c, cudaMalloc(&c->d_multi_done, ((size_t)L.count + 1) * sizeof(int)));
     c->multi = true;
-    return c->monitor ? multi_monitor(c) : LBM_OK;
+    if (c->monitor) multi_monitor(c);
+    return LBM_OK;
 }
 
 // The tile plan (step_kernel_tile, lbm_tile.cuh) of a context under
@@ -865,9 +861,7 @@ void release(lbm_ctx* c) {
     cudaFree(c->d_nbr);
     cudaFree(c->d_multi_done);
     cudaFree(c->d_tile);
-    cudaFree(c->d_mon_multi);
-    cudaFree(c->d_mon_multi_cnt);
-    cudaFree(c->d_mon_multi_sub);
+    cudaFree(c->mon_multi.slots);
     cudaFree(c->d_tmp);
     cudaFree(c->d_out);
     cudaFree(c->d_partials);
@@ -1131,8 +1125,8 @@ cudaError_t enqueue_multi(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, in
     if (e != cudaSuccess) return e;
     const bool monitor = host_records != nullptr;
     if (monitor) {
-        if (nsteps > kMultiSteps || !c->d_mon || !c->d_mon_multi) return cudaErrorInvalidValue;
-        e = cudaMemsetAsync(c->d_mon_multi_cnt, 0, (size_t)nsteps * c->n * (lbm::kMonSub + 1) * sizeof(int),
+        if (nsteps > kMultiSteps || !c->d_mon || !c->mon_multi.slots) return cudaErrorInvalidValue;
+        e = cudaMemsetAsync(c->mon_multi.count, 0, (size_t)nsteps * c->n * (lbm::kMonSub + 1) * sizeof(int),
                             c->stream);
         if (e != cudaSuccess) return e;
     }
@@ -1145,9 +1139,9 @@ cudaError_t enqueue_multi(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, in
     a.wait_extra = wait_extra;
     a.wait_limit = wait_limit;
     if (monitor) {
-        a.mon = c->d_mon_multi;
-        a.mon_sub = c->d_mon_multi_sub;
-        a.mon_count = c->d_mon_multi_cnt;
+        a.mon = c->mon_multi.slots;
+        a.mon_sub = c->mon_multi.sub;
+        a.mon_count = c->mon_multi.count;
         a.mon_csr = c->d_mon_csr;
         a.mon_n = c->n;
         a.mon_rec = reinterpret_cast<lbm::MonRecord*>(c->d_mon);
@@ -1386,7 +1380,7 @@ lbm_status lbm_step_monitored_all(lbm_ctx* c, int nsteps, lbm_monitor* host_reco
     if (c->plan_dirty && (st = plan(c)) != LBM_OK) return st;
     lbm::MonRecord* hd = static_cast<lbm::MonRecord*>(dptr);
     for (int done = 0; done < nsteps;) {
-        if (multi_plan(c)) {   // up to 64 steps a launch, every step's record from it
+        if (multi_plan(c) && c->mon_multi.slots) {   // up to 64 steps a launch, every step's record from it
             const int k = std::min(nsteps - done, kMultiSteps);
             cudaError_t e = enqueue_multi(c, c->cur, k, 0, lbm::kWaitLimit, hd + (long long)done * c->n);
             if (e != cudaSuccess) return cuda_fail(c, e, "monitored step launch");
@@ -1416,12 +1410,11 @@ lbm_status lbm_set_monitor(lbm_ctx* c, int enable) {
     if (!c) return LBM_EINVAL;
     if (c->d3 && enable) return fail(c, LBM_EINVAL, "the per-step monitor serves D2Q9 contexts");
     LBM_CK(c, cudaSetDevice(c->device));
-    if (enable && !c->d_mon) {
-        LBM_CK(c, cudaMalloc(&c->d_mon, (size_t)c->n * sizeof(lbm_monitor)));
-        LBM_CK(c, cudaMallocHost(&c->h_mon, sizeof(lbm_monitor)));
-    }
+    if (enable && !c->h_mon) LBM_CK(c, cudaMallocHost(&c->h_mon, sizeof(lbm_monitor)));
+    if (enable && !c->d_mon) LBM_CK(c, cudaMalloc(&c->d_mon, (size_t)c->n * sizeof(lbm_monitor)));
     c->monitor = enable != 0;
-    return enable && !c->plan_dirty ? multi_monitor(c) : LBM_OK;
+    if (enable && !c->plan_dirty) multi_monitor(c);
+    return LBM_OK;
 }
 
 lbm_status lbm_read_monitor_async(lbm_ctx* c, int instance, lbm_monitor* host_out) {
