@@ -566,33 +566,11 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
         return cudaSuccess;
     });
     if (occ <= 0 || (long long)L.count > (long long)sms * occ) return LBM_OK;
-    struct Box { int inst, x0, x1, y0, y1; };
-    std::vector<Box> box(L.count);
-    for (int k = 0; k < L.count; ++k) {
-        const WorkItem& w = c->work[L.offset + k];
-        const lbm_params& p = c->params[w.inst];
-        const int y0 = w.dir < 0 ? w.ystart - w.nrows + 1 : w.ystart;
-        box[k] = {w.inst, w.x0, std::min(p.nx, w.x0 + L.tx), y0, y0 + w.nrows};
-    }
-    // [a0, a1) and [b0, b1) meet, with b shifted by -n, 0, +n when periodic
-    auto meet = [](int a0, int a1, int b0, int b1, int n, bool periodic) {
-        for (int sh = periodic ? -1 : 0; sh <= (periodic ? 1 : 0); ++sh)
-            if (b0 + sh * n < a1 && a0 < b1 + sh * n) return true;
-        return false;
+    std::vector<int> nbr;
+    auto domain = [&](int k) {
+        return lbm::Domain{c->params[k].nx, c->params[k].ny, c->params[k].bc_y != LBM_BC_BOUNCEBACK};
     };
-    std::vector<int> nbr((size_t)L.count * lbm::kMaxTileNbr, -1);
-    for (int k = 0; k < L.count; ++k) {
-        const lbm_params& p = c->params[box[k].inst];
-        const bool per_y = p.bc_y != LBM_BC_BOUNCEBACK;
-        int cnt = 0;
-        for (int m = 0; m < L.count; ++m) {
-            if (m == k || box[m].inst != box[k].inst) continue;
-            if (!meet(box[k].x0 - 3, box[k].x1 + 3, box[m].x0, box[m].x1, p.nx, true)) continue;
-            if (!meet(box[k].y0 - 3, box[k].y1 + 3, box[m].y0, box[m].y1, p.ny, per_y)) continue;
-            if (cnt == lbm::kMaxTileNbr) return LBM_OK;   // too many: no persistent launch
-            nbr[(size_t)k * lbm::kMaxTileNbr + cnt++] = m;
-        }
-    }
+    if (!lbm::march_neighbours(c->work.data() + L.offset, L.count, L.tx, domain, nbr)) return LBM_OK;
     cudaFree(c->d_nbr);
     c->d_nbr = nullptr;
     cudaFree(c->d_multi_done);

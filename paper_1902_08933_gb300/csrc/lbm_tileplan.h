@@ -1,5 +1,6 @@
-// lbm_tileplan.h -- host side of the tile plans (step_kernel_tile, sp_tile_kernel):
-// domains cut into tiles and each tile's neighbours.
+// lbm_tileplan.h -- host side of the plans that run several steps a launch: domains
+// cut into tiles (step_kernel_tile, sp_tile_kernel), and the neighbours of each tile
+// and of each item of a row march (step_kernel_x2_multi).
 #pragma once
 
 #include <algorithm>
@@ -53,6 +54,46 @@ inline void add_tiles(TileList& out, int inst, int nx, int ny, int cpt, bool per
                     if (ii != i || jj != j) out.nbr.push_back(first + jj * kx + ii);
             out.nbr.resize(at + kMaxTileNbr, -1);   // at most 5 x 5 - 1
         }
+}
+
+struct Domain {
+    int nx, ny;
+    bool per_y;   // periodic in y (in x always)
+};
+
+// Neighbours of the items of a row march, strips of tx columns (dom(instance): its
+// Domain): for each item the other items of its instance within the 3 cells that a
+// step reaches -- it reads h up to 2 cells outside the item, which cells up to 3
+// outside have pushed --, kMaxTileNbr an item, -1 padded. A last strip may be as
+// narrow as 2 columns, so the item beyond it counts too. False: one has more.
+template <typename Dom>
+bool march_neighbours(const WorkItem* items, int count, int tx, Dom&& dom, std::vector<int>& nbr) {
+    struct Box { int inst, x0, x1, y0, y1; };
+    std::vector<Box> box(count);
+    for (int k = 0; k < count; ++k) {
+        const WorkItem& w = items[k];
+        const int y0 = w.dir < 0 ? w.ystart - w.nrows + 1 : w.ystart;
+        box[k] = {w.inst, w.x0, std::min(dom(w.inst).nx, w.x0 + tx), y0, y0 + w.nrows};
+    }
+    // [a0, a1) and [b0, b1) meet, with b shifted by -n, 0, +n when periodic
+    auto meet = [](int a0, int a1, int b0, int b1, int n, bool periodic) {
+        for (int sh = periodic ? -1 : 0; sh <= (periodic ? 1 : 0); ++sh)
+            if (b0 + sh * n < a1 && a0 < b1 + sh * n) return true;
+        return false;
+    };
+    nbr.assign((size_t)count * kMaxTileNbr, -1);
+    for (int k = 0; k < count; ++k) {
+        const Domain d = dom(box[k].inst);
+        int cnt = 0;
+        for (int m = 0; m < count; ++m) {
+            if (m == k || box[m].inst != box[k].inst) continue;
+            if (!meet(box[k].x0 - 3, box[k].x1 + 3, box[m].x0, box[m].x1, d.nx, true)) continue;
+            if (!meet(box[k].y0 - 3, box[k].y1 + 3, box[m].y0, box[m].y1, d.ny, d.per_y)) continue;
+            if (cnt == kMaxTileNbr) return false;
+            nbr[(size_t)k * kMaxTileNbr + cnt++] = m;
+        }
+    }
+    return true;
 }
 
 // The smallest of 8 x 4, 8 x 8 and 16 x 8 units whose tiles (count(U, R) of them)

@@ -53,3 +53,101 @@ int main() {
     return 0;
 }
 """)
+
+
+NEIGHBOURS = r"""
+#include <cstdio>
+#include <set>
+#include "lbm_tileplan.h"
+using lbm::WorkItem;
+// The items' neighbour lists against every pair of cells within 3 of one another.
+struct Rect { int x0, x1, y0, y1; };
+static int check(const std::vector<Rect>& r, const std::vector<int>& nbr, int nx, int ny, bool per_y) {
+    std::vector<int> owner((size_t)nx * ny, -1);
+    for (int k = 0; k < (int)r.size(); ++k)
+        for (int y = r[k].y0; y < r[k].y1; ++y)
+            for (int x = r[k].x0; x < r[k].x1; ++x) {
+                if (owner[y * nx + x] >= 0) return 1;
+                owner[y * nx + x] = k;
+            }
+    std::vector<std::set<int>> want(r.size());
+    for (int y = 0; y < ny; ++y)
+        for (int x = 0; x < nx; ++x) {
+            if (owner[y * nx + x] < 0) return 2;
+            for (int dy = -3; dy <= 3; ++dy)
+                for (int dx = -3; dx <= 3; ++dx) {
+                    int Y = y + dy;
+                    if (!per_y && (Y < 0 || Y >= ny)) continue;
+                    Y = (Y + 2 * ny) % ny;
+                    want[owner[y * nx + x]].insert(owner[Y * nx + (x + dx + 2 * nx) % nx]);
+                }
+        }
+    for (int k = 0; k < (int)r.size(); ++k) {
+        std::set<int> got;
+        for (int j = 0; j < lbm::kMaxTileNbr; ++j)
+            if (nbr[(size_t)k * lbm::kMaxTileNbr + j] >= 0) got.insert(nbr[(size_t)k * lbm::kMaxTileNbr + j]);
+        want[k].erase(k);
+        if (got != want[k]) {
+            std::printf("%d x %d periodic %d: item %d has %zu neighbours for %zu\n", nx, ny, per_y, k, got.size(), want[k].size());
+            return 3;
+        }
+    }
+    return 0;
+}
+"""
+
+
+def test_march_neighbours_are_the_items_within_three_cells(tmp_path):
+    # a last strip of 1 to 4 columns beside whole ones, one strip, runs of few rows
+    run_cpp(tmp_path, NEIGHBOURS + r"""
+int main() {
+    for (int tx : {64, 128, 256})
+        for (int nx : {tx, tx + 2, tx + 4, 2 * tx + 2, 3 * tx + 2, 2 * tx, tx / 2, 6, 3})
+            for (int rows : {8, 9, 5, 3})
+                for (int ny : {3, 8, 16, 17, 40})
+                    for (bool per_y : {false, true}) {
+                        std::vector<WorkItem> w;
+                        std::vector<Rect> r;
+                        for (int x0 = 0; x0 < nx; x0 += tx)
+                            for (int y0 = 0, k = 0; y0 < ny; y0 += rows, ++k) {
+                                const int y1 = std::min(ny, y0 + rows);
+                                WorkItem i{};
+                                i.x0 = x0;
+                                i.nrows = y1 - y0;
+                                i.dir = k % 2 ? 1 : -1;
+                                i.ystart = i.dir < 0 ? y1 - 1 : y0;
+                                w.push_back(i);
+                                r.push_back({x0, std::min(nx, x0 + tx), y0, y1});
+                            }
+                        std::vector<int> nbr;
+                        if (!lbm::march_neighbours(w.data(), (int)w.size(), tx, [&](int) { return lbm::Domain{nx, ny, per_y}; }, nbr))
+                            return 9;
+                        if (int e = check(r, nbr, nx, ny, per_y)) return e;
+                    }
+    return 0;
+}
+""")
+
+
+def test_tile_neighbours_are_the_tiles_within_three_cells(tmp_path):
+    run_cpp(tmp_path, NEIGHBOURS + r"""
+int main() {
+    const int shapes[4][2] = {{8, 4}, {8, 8}, {16, 8}, {8, 16}};
+    for (auto& s : shapes)
+        for (int cpt : {1, 2})
+            for (int nx = 3; nx < 75; nx += nx < 40 ? 1 : 7)
+                for (int ny : {3, 4, 5, 7, 8, 9, 15, 16, 17, 18, 33, 34, 50})
+                    for (bool per_y : {false, true}) {
+                        if (nx % cpt) continue;
+                        lbm::TileList list;
+                        lbm::add_tiles(list, 0, nx, ny, cpt, per_y, s[0], s[1]);
+                        std::vector<Rect> r;
+                        for (const WorkItem& w : list.items) {
+                            if (w.dir > s[0] * cpt || w.nrows > s[1]) return 9;
+                            r.push_back({w.x0, w.x0 + w.dir, w.ystart, w.ystart + w.nrows});
+                        }
+                        if (int e = check(r, list.nbr, nx, ny, per_y)) return e;
+                    }
+    return 0;
+}
+""")
