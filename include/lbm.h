@@ -487,6 +487,13 @@ lbm_status lbm_inject_wait_timeout(lbm_ctx* ctx, int rounds);
  * initialised, or the plan is not the batched launch), LBM_ECUDA. */
 lbm_status lbm_inject_batched_wait_timeout(lbm_ctx* ctx, int rounds);
 
+/* The same for whichever plan the context has that runs several steps a launch:
+ * the batched launch, the persistent plan (LBM_PIPELINE_PERSISTENT, or
+ * LBM_PIPELINE_AUTO where it takes it) or the tiles of small contexts. Every wait
+ * of the second of two steps is for one step or item more than there is. Errors
+ * as above; LBM_ESTATE also when every step is a launch of its own. */
+lbm_status lbm_inject_step_wait_timeout(lbm_ctx* ctx, int rounds);
+
 /* Waits for all queued work. Returns LBM_ECUDA if it failed, LBM_ETIMEOUT if a
  * bounded device wait of the step kernel ran out (the state is then suspect;
  * the status stays set until lbm_load replaces the whole state). lbm_get_fields
@@ -573,6 +580,12 @@ lbm_status lbm_sp_get_fields(lbm_sp_ctx* ctx, unsigned mask, double* host_out);
  * Remarks 1 and 2: as they are; Remark 4 scheme: the unshifted f). Synchronises. */
 lbm_status lbm_sp_get_populations(lbm_sp_ctx* ctx, double* host_g);
 
+/* As lbm_inject_step_wait_timeout, for a single-phase context whose steps run on
+ * tiles (several in one launch): afterwards lbm_sp_get_fields and
+ * lbm_sp_get_populations return LBM_ETIMEOUT until lbm_sp_init. Errors: LBM_EINVAL
+ * (NULL context, rounds out of 1 .. 2^21), LBM_ESTATE (not initialised, or the
+ * context runs a launch a step), LBM_ECUDA. */
+lbm_status lbm_sp_inject_wait_timeout(lbm_sp_ctx* ctx, int rounds);
 const char* lbm_sp_last_error(const lbm_sp_ctx* ctx);
 void lbm_sp_destroy(lbm_sp_ctx* ctx);
 

@@ -1942,7 +1942,9 @@ __global__ void wait_timeout_kernel(int rounds, int* status) {
 
 }  // namespace
 
-lbm_status lbm_inject_batched_wait_timeout(lbm_ctx* c, int rounds) {
+// Both hooks of the several-step launches; named: only plans that the caller asked
+// for by name (or several instances).
+static lbm_status inject_step_timeout(lbm_ctx* c, int rounds, bool named) {
     if (!c) return LBM_EINVAL;
     if (rounds < 1 || rounds > lbm::kWaitLimit)
         return fail(c, LBM_EINVAL, "rounds must be in 1 .. 2^21");
@@ -1952,17 +1954,21 @@ lbm_status lbm_inject_batched_wait_timeout(lbm_ctx* c, int rounds) {
     lbm_status st = sticky(c);
     if (st != LBM_OK) return st;
     if (c->plan_dirty && (st = plan(c)) != LBM_OK) return st;
-    if (!batched_plan(c) && !(multi_plan(c) && c->pipeline == LBM_PIPELINE_PERSISTENT))
-        return fail(c, LBM_ESTATE, "the context runs neither the batched nor the persistent launch");
+    if (named ? !batched_plan(c) && !(multi_plan(c) && c->pipeline == LBM_PIPELINE_PERSISTENT)
+              : !tile_plan(c) && !batched_plan(c) && !multi_plan(c))
+        return fail(c, LBM_ESTATE, named ? "the context runs neither the batched nor the persistent launch"
+                                         : "the context runs no launch of several steps");
     // two steps; every item of the second waits for one finished item (batched)
-    // or step (persistent, and the tiles that stand in for the batched launch in
-    // small contexts) more than there are, so each of those waits runs out after
-    // `rounds` rounds
+    // or step (persistent, tiles) more than there are, so each of those waits runs
+    // out after `rounds` rounds
     LBM_CK(c, tile_plan(c)      ? enqueue_tile(c, c->cur, 2, 1, rounds)
               : batched_plan(c) ? enqueue_batched(c, c->cur, 2, 1, rounds)
                                 : enqueue_multi(c, c->cur, 2, 1, rounds));
     return LBM_OK;
 }
+
+lbm_status lbm_inject_batched_wait_timeout(lbm_ctx* c, int rounds) { return inject_step_timeout(c, rounds, true); }
+lbm_status lbm_inject_step_wait_timeout(lbm_ctx* c, int rounds) { return inject_step_timeout(c, rounds, false); }
 
 lbm_status lbm_inject_wait_timeout(lbm_ctx* c, int rounds) {
     if (!c) return LBM_EINVAL;

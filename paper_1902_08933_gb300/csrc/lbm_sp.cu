@@ -643,7 +643,7 @@ struct SpTileArgs {
     const void *g0, *g1;   // buffer sets: step s reads g0 when s is even
     const void* src;
     void* uprev;
-    int N, nitems, nsteps, ulog, wait_limit;
+    int N, nitems, nsteps, ulog, wait_limit, wait_extra;   // wait_*: as in StepArgs
     const lbm::WorkItem* work;
     const int* nbr;
     int *done, *status;
@@ -666,8 +666,8 @@ __global__ void __launch_bounds__(kSpThreads, OCC) sp_tile_kernel(const SpTileAr
         R* gout = static_cast<R*>(const_cast<void*>((s & 1) ? a.g0 : a.g1));
         for (int item = blockIdx.x; item < a.nitems; item += gridDim.x) {
             const lbm::WorkItem wk = a.work[item];
-            if (s > 0 && !lbm::tile_wait(a.done, a.nbr + item * lbm::kMaxTileNbr, s, a.wait_limit, a.status,
-                                         a.done + a.nitems, &s_bad, tid))
+            if (s > 0 && !lbm::tile_wait(a.done, a.nbr + item * lbm::kMaxTileNbr, s + a.wait_extra, a.wait_limit,
+                                         a.status, a.done + a.nitems, &s_bad, tid))
                 return;
             const int nu = wk.dir / U::cells, rows = wk.nrows;
             const int tx = tid & (W - 3), ty = tid >> a.ulog;
@@ -902,8 +902,8 @@ cudaError_t sp_step_once(lbm_sp_ctx* c) {
 }
 
 // Queues n steps on tiles as one cooperative launch, after zeroing the step
-// counters and the abort flag.
-cudaError_t sp_step_tiles(lbm_sp_ctx* c, int n) {
+// counters and the abort flag; wait_extra / wait_limit as in StepArgs.
+cudaError_t sp_step_tiles(lbm_sp_ctx* c, int n, int wait_extra = 0, int wait_limit = lbm::kWaitLimit) {
     SpTileArgs a;
     a.g0 = c->g[c->cur];
     a.g1 = c->g[1 - c->cur];
@@ -913,7 +913,8 @@ cudaError_t sp_step_tiles(lbm_sp_ctx* c, int n) {
     a.nitems = c->tile_items;
     a.nsteps = n;
     a.ulog = c->tile_ulog;
-    a.wait_limit = lbm::kWaitLimit;
+    a.wait_limit = wait_limit;
+    a.wait_extra = wait_extra;
     a.work = c->d_tile_work;
     a.nbr = c->d_tile_nbr;
     a.done = c->d_tile_done;
@@ -1101,6 +1102,15 @@ lbm_status lbm_sp_get_populations(lbm_sp_ctx* c, double* host_g) {
         return sp_cuda(c, r, "populations read-back");
     if ((r = cudaStreamSynchronize(c->stream)) != cudaSuccess) return sp_cuda(c, r, "populations");
     return sp_device_status(c);
+}
+
+lbm_status lbm_sp_inject_wait_timeout(lbm_sp_ctx* c, int rounds) {
+    if (!c) return LBM_EINVAL;
+    if (rounds < 1 || rounds > lbm::kWaitLimit) return sp_fail(c, LBM_EINVAL, "rounds must be in 1 .. 2^21");
+    if (!c->ready) return sp_fail(c, LBM_ESTATE, "not initialised");
+    if (!c->tile) return sp_fail(c, LBM_ESTATE, "the context runs a launch a step");
+    const cudaError_t e = sp_step_tiles(c, 2, 1, rounds);   // every wait of the second step runs out
+    return e == cudaSuccess ? LBM_OK : sp_cuda(c, e, "step kernel");
 }
 
 const char* lbm_sp_last_error(const lbm_sp_ctx* c) { return c ? c->err.c_str() : "null context"; }

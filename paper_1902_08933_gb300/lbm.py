@@ -127,6 +127,7 @@ SIGNATURES = [
     ("lbm_reduce_fields_noalloc", ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, _VP, _VP]),
     ("lbm_inject_wait_timeout", ctypes.c_int, [_VP, ctypes.c_int]),
     ("lbm_inject_batched_wait_timeout", ctypes.c_int, [_VP, ctypes.c_int]),
+    ("lbm_inject_step_wait_timeout", ctypes.c_int, [_VP, ctypes.c_int]),
     ("lbm_sync", ctypes.c_int, [_VP]),
     ("lbm_last_error", ctypes.c_char_p, [_VP]),
     ("lbm_destroy", None, [_VP]),
@@ -136,6 +137,7 @@ SIGNATURES = [
     ("lbm_sp_step", ctypes.c_int, [_VP, ctypes.c_int]),
     ("lbm_sp_get_fields", ctypes.c_int, [_VP, ctypes.c_uint, _DP]),
     ("lbm_sp_get_populations", ctypes.c_int, [_VP, _DP]),
+    ("lbm_sp_inject_wait_timeout", ctypes.c_int, [_VP, ctypes.c_int]),
     ("lbm_sp_last_error", ctypes.c_char_p, [_VP]),
     ("lbm_sp_destroy", None, [_VP]),
 ]
@@ -364,6 +366,10 @@ def lbm_inject_batched_wait_timeout(ctx, rounds: int):
     _check(library().lbm_inject_batched_wait_timeout(ctx, int(rounds)), ctx)
 
 
+def lbm_inject_step_wait_timeout(ctx, rounds: int):
+    _check(library().lbm_inject_step_wait_timeout(ctx, int(rounds)), ctx)
+
+
 def lbm_sync(ctx):
     _check(library().lbm_sync(ctx), ctx)
 
@@ -446,6 +452,10 @@ def _check_sp(st, ctx=None):
     if st != LBM_OK:
         msg = library().lbm_sp_last_error(ctx).decode() if ctx else ""
         raise LbmError(st, msg)
+
+
+def lbm_sp_inject_wait_timeout(ctx, rounds: int):
+    _check_sp(library().lbm_sp_inject_wait_timeout(ctx, int(rounds)), ctx)
 
 
 class SourceFlow:
