@@ -934,8 +934,9 @@ cudaError_t sp_step_tiles(lbm_sp_ctx* c, int n, int wait_extra = 0, int wait_lim
 lbm_status sp_device_status(lbm_sp_ctx* c) {
     if (!c->tile) return LBM_OK;
     int st = 0;
-    const cudaError_t r = cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (r != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) return sp_cuda(c, r, "status read-back");
+    cudaError_t r = cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    if (r == cudaSuccess) r = cudaStreamSynchronize(c->stream);
+    if (r != cudaSuccess) return sp_cuda(c, r, "status read-back");
     return st == 0 ? LBM_OK : sp_fail(c, LBM_ETIMEOUT, "a bounded device wait ran out in the step kernel");
 }
 
