@@ -696,21 +696,12 @@ template <> struct MonAcc<F2> {
 // flag, the status word and the time level). Every sum has a fixed order, so the
 // record does not depend on which blocks finish last.
 //
-// The group of threads doing this is a whole block (bar 0, grp 0) or one of the
-// thread groups of the batched kernel (named barrier `bar`, group `grp` < 4,
-// nthr threads, tid its index in the group); item is the work item whose slot
-// the group writes, pos its position within its instance's items.
-__device__ __forceinline__ void group_sync(int bar, int nthr) {
-    if (bar == 0) {   // the whole block (a compile-time 0 wherever a kernel passes it)
-        __syncthreads();
-    } else {
-        asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
-    }
-}
+// The whole block does this (nthr threads); item is the work item whose slot it
+// writes, pos its position within its instance's items.
 
-// Sums (max for q = 2) of four quantities over a group, fixed tree; result in
-// thread 0's v. red: the group's [4][8] shared scratch.
-__device__ __forceinline__ void group_reduce4(double v[4], int tid, int nthr, int bar, double (*red)[8]) {
+// Sums (max for q = 2) of four quantities over a block, fixed tree; result in
+// thread 0's v. red: [quantity][warp], up to 8 warps.
+__device__ __forceinline__ void block_reduce4(double v[4], int tid, int nthr, double (&red)[4][8]) {
     const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -719,9 +710,9 @@ __device__ __forceinline__ void group_reduce4(double v[4], int tid, int nthr, in
         v[2] = fmax(v[2], __shfl_down_sync(0xffffffffu, v[2], o));
         v[3] += __shfl_down_sync(0xffffffffu, v[3], o);
     }
-    group_sync(bar, nthr);   // red[] may still be read by an earlier use
+    __syncthreads();   // red[] may still be read by an earlier use
     if (lane == 0) { red[0][warp] = v[0]; red[1][warp] = v[1]; red[2][warp] = v[2]; red[3][warp] = v[3]; }
-    group_sync(bar, nthr);
+    __syncthreads();
     if (tid == 0)
         for (int w = 1; w < nwarps; ++w) {
             v[0] += red[0][w];
@@ -785,15 +776,13 @@ __device__ __forceinline__ bool tile_wait(const int* done, const int* nbr, int n
 
 template <typename R>
 __device__ __forceinline__ void mon_block_store(const MonAcc<R>& acc, const StepArgs& a, int inst, int item,
-                                                int pos, int tid, int nthr, int bar, int grp) {
-    __shared__ double red_all[4][4][8];   // [group][quantity][warp]: up to 8 warps a group
-    __shared__ int flag_all[4];
-    double (*red)[8] = red_all[grp];
-    int& flag = flag_all[grp];
+                                                int pos, int tid, int nthr) {
+    __shared__ double red[4][8];
+    __shared__ int flag;
     double v[4];
     acc.result(v[0], v[1], v[2]);
     v[3] = 0.0;
-    group_reduce4(v, tid, nthr, bar, red);
+    block_reduce4(v, tid, nthr, red);
     const int* idx = a.mon_csr + a.mon_n + 1;
     const int first = a.mon_csr[inst], items = a.mon_csr[inst + 1] - first;
     const int nsub = items < kMonSub ? items : kMonSub;
@@ -811,7 +800,7 @@ __device__ __forceinline__ void mon_block_store(const MonAcc<R>& acc, const Step
         // orders after this thread's acquire
         flag = atom_add_acq_rel_gpu(cnt + s * kCounterStride, 1) == in_sub - 1;
     }
-    group_sync(bar, nthr);
+    __syncthreads();
     if (!flag) return;
     // the sub-group's slots, in order
     double w[4] = {0.0, 0.0, 0.0, 0.0};
@@ -822,7 +811,7 @@ __device__ __forceinline__ void mon_block_store(const MonAcc<R>& acc, const Step
         w[2] = fmax(w[2], __ldcg(p + 2));
         w[3] += __ldcg(p + 3);
     }
-    group_reduce4(w, tid, nthr, bar, red);
+    block_reduce4(w, tid, nthr, red);
     if (tid == 0) {
         double* sub = a.mon_sub + ((long long)inst * kMonSub + s) * kMonQ;
         sub[0] = w[0];
@@ -832,10 +821,10 @@ __device__ __forceinline__ void mon_block_store(const MonAcc<R>& acc, const Step
         cnt[s * kCounterStride] = 0;                      // ready for the next monitored step
         flag = atom_add_acq_rel_gpu(cnt + kMonSub * kCounterStride, 1) == nsub - 1;
     }
-    group_sync(bar, nthr);   // (every thread read the first flag before group_reduce4's barriers)
+    __syncthreads();   // (every thread read the first flag before block_reduce4's barriers)
     if (!flag || tid >= 32) return;
     // the instance's record from its sub-group slots: lane q < nsub of the
-    // group's first warp loads slot q (the loads in parallel), lane 0 adds them
+    // block's first warp loads slot q (the loads in parallel), lane 0 adds them
     // in order q = 0, 1, ...
     double sv[4] = {0.0, 0.0, 0.0, 0.0};
     if (tid < nsub) {
@@ -870,7 +859,7 @@ __device__ __forceinline__ void mon_block_store(const MonAcc<R>& acc, const Step
 
 // Monitor of every step of a persistent launch (step_kernel_x2_multi with the
 // record of each step), the two-level tree of mon_block_store kept per step s
-// of the launch: the group reduces its item's sums into slot
+// of the launch: the block reduces its item's sums into slot
 // a.mon[(s * a.ndesc + item) * kMonQ] and counts itself in its sub-group's
 // counter (sub-group = its position pos within the instance's items modulo
 // kMonSub; counters a.mon_count[(s * a.mon_n + inst) * (kMonSub + 1) + ...],
@@ -884,15 +873,13 @@ __device__ __forceinline__ void mon_block_store(const MonAcc<R>& acc, const Step
 // that finishes a step last short, since its neighbours wait for it.
 template <typename R>
 __device__ __forceinline__ void mon_step_store(const MonAcc<R>& acc, const StepArgs& a, int inst, int item,
-                                               int pos, int tid, int nthr, int bar, int grp, int s) {
-    __shared__ double sred_all[4][4][8];
-    __shared__ int sflag_all[4];
-    double (*red)[8] = sred_all[grp];
-    int& flag = sflag_all[grp];
+                                               int pos, int tid, int nthr, int s) {
+    __shared__ double red[4][8];
+    __shared__ int flag;
     double v[4];
     acc.result(v[0], v[1], v[2]);
     v[3] = 0.0;
-    group_reduce4(v, tid, nthr, bar, red);
+    block_reduce4(v, tid, nthr, red);
     const int* idx = a.mon_csr + a.mon_n + 1;
     const int first = a.mon_csr[inst], items = a.mon_csr[inst + 1] - first;
     const int nsub = items < kMonSub ? items : kMonSub;
@@ -909,7 +896,7 @@ __device__ __forceinline__ void mon_step_store(const MonAcc<R>& acc, const StepA
         out[3] = (isfinite(v[0]) && isfinite(v[1])) ? 0.0 : 1.0;
         flag = atom_add_acq_rel_gpu(cnt + sg, 1) == in_sub - 1;
     }
-    group_sync(bar, nthr);
+    __syncthreads();
     if (!flag) return;
     double w[4] = {0.0, 0.0, 0.0, 0.0};
     for (int j = tid; j < in_sub; j += nthr) {
@@ -919,7 +906,7 @@ __device__ __forceinline__ void mon_step_store(const MonAcc<R>& acc, const StepA
         w[2] = fmax(w[2], __ldcg(p + 2));
         w[3] += __ldcg(p + 3);
     }
-    group_reduce4(w, tid, nthr, bar, red);
+    block_reduce4(w, tid, nthr, red);
     double* subs = a.mon_sub + si * kMonSub * kMonQ;
     if (tid == 0) {
         double* sub = subs + sg * kMonQ;
@@ -929,7 +916,7 @@ __device__ __forceinline__ void mon_step_store(const MonAcc<R>& acc, const StepA
         sub[3] = w[3];
         flag = atom_add_acq_rel_gpu(cnt + kMonSub, 1) == nsub - 1;
     }
-    group_sync(bar, nthr);   // (every thread read the first flag before group_reduce4's barriers)
+    __syncthreads();   // (every thread read the first flag before block_reduce4's barriers)
     if (!flag || tid >= 32) return;
     // the record from the sub-group slots: lane q < nsub loads slot q, lane 0
     // adds them in order q = 0, 1, ...
@@ -1359,7 +1346,7 @@ __global__ void __launch_bounds__(TX, StepOcc<FORM, TX>::value) step_kernel(cons
         __syncthreads();
         collide_row(Y, g, pux, puy);
     }
-    if constexpr (MON) mon_block_store(mon, a, wk.inst, blockIdx.x, wk.pad, threadIdx.x, TX, 0, 0);
+    if constexpr (MON) mon_block_store(mon, a, wk.inst, blockIdx.x, wk.pad, threadIdx.x, TX);
 }
 
 }  // namespace lbm

@@ -200,22 +200,19 @@ __device__ __forceinline__ void x2_collide_push(const Consts<float>& C, const X2
 }
 
 // One work item (a strip of 2 TX columns of one instance, a run of rows) marched
-// by a group of TX threads (32, 64 or 128): a whole thread block in every kernel
-// here (barrier 0, the one __syncthreads uses; TX its compile-time block size, so
-// the layout below folds to constants). smem_raw is the group's region in the
-// X2Smem<FORM, TX> layout, tid the thread's index in the group, item the work
-// item's index in StepArgs::work (and of its monitor slot); swap: the step reads
-// the *_out buffers of a and writes the *_in ones (odd steps of a launch of
-// several).
+// by a block of TX threads (32, 64 or 128; the caller's compile-time block size, so
+// the layout below folds to constants). smem_raw is the block's region in the
+// X2Smem<FORM, TX> layout, tid the thread's index, item the work item's index in
+// StepArgs::work (and of its monitor slot); swap: the step reads the *_out buffers
+// of a and writes the *_in ones (odd steps of a launch of several).
 template <int FORM, int MON>
 __device__ __forceinline__ void x2_item(const StepArgs& a, int item, unsigned char* smem_raw, int tid,
-                                        int bar, int grp, const int TX, const bool swap = false,
-                                        const int step = 0) {
+                                        const int TX, const bool swap = false, const int step = 0) {
     using F = Form<FORM>;
     using HT = typename F::HT;
     using GT = typename F::GT;
     static_assert(sizeof(typename F::R) == 4, "the paired kernel serves the FP32-arithmetic forms");
-    // X2Smem<FORM, TX>'s layout for this group width
+    // X2Smem<FORM, TX>'s layout for this width
     const int SW = 2 * TX, RW = SW + 8;
     const size_t H0B = F::cons ? (size_t)RW * sizeof(float2) : 0;
     const size_t HPB = (size_t)RW * sizeof(HT);
@@ -461,18 +458,18 @@ __device__ __forceinline__ void x2_item(const StepArgs& a, int item, unsigned ch
             if (ghost(Y0 + k * d) == (pass == 1)) lead_row(Y0 + k * d);
     p_row(Y0 - d);
     p_row(Y0);
-    group_sync(bar, TX);
+    __syncthreads();
     mu_row(Y0);
     mu_row(Y0 - d);
     if constexpr (F::comp) {
         // mu of row Y0 - d read the low parts of phi from the h slot of row
         // Y0 - 2d: every thread must be done with it before it is refilled
-        group_sync(bar, TX);
+        __syncthreads();
         prefetch(Y0 + 2 * d, Y0 + d);   // the slot of row Y0 - 2d takes the first lead row
     } else {
         // (issued before the barrier: the slot of row Y0 - 2d was read only above)
         prefetch(Y0 + 2 * d, Y0 + d);
-        group_sync(bar, TX);
+        __syncthreads();
     }
     for (int k = 0; k < wk.nrows; ++k) {
         const int Y = Y0 + k * d;
@@ -493,32 +490,32 @@ __device__ __forceinline__ void x2_item(const StepArgs& a, int item, unsigned ch
         if constexpr (!F::h16)
             if (k + 1 < wk.nrows) l2_prefetch_row(Y + d);
         lead_row_async(Y + 2 * d);
-        group_sync(bar, TX);
+        __syncthreads();
         // every thread is past the collision of row Y - d: the h slot of row Y - d
         // and the p slot of row Y - 2d are free for the next iteration's rows
         if (k + 1 < wk.nrows) prefetch(Y + 3 * d, Y + 2 * d);
         mu_row(Y + d);
-        group_sync(bar, TX);
+        __syncthreads();
         collide_row(Y, g, pux, puy);
     }
-    if constexpr (MON == 1) mon_block_store(mon, a, wk.inst, item, wk.pad, tid, TX, bar, grp);
+    if constexpr (MON == 1) mon_block_store(mon, a, wk.inst, item, wk.pad, tid, TX);
     if constexpr (MON == 2) {
         // persistent launch: publish this item's step first (the monitor's tree
         // reads only the monitor buffers), so the neighbour items' next step
         // need not wait for the reduction
-        group_sync(bar, TX);
+        __syncthreads();
         if (tid == 0) {
             __threadfence();
             atomicAdd(a.done + item, 1);
         }
-        mon_step_store(mon, a, wk.inst, item, wk.pad, tid, TX, bar, grp, step);
+        mon_step_store(mon, a, wk.inst, item, wk.pad, tid, TX, step);
     }
 }
 
 template <int FORM, int TX, bool MON = false>
 __global__ void __launch_bounds__(TX, X2Occ<FORM, TX>::value) step_kernel_x2(const StepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    x2_item<FORM, MON>(a, blockIdx.x, smem_raw, threadIdx.x, 0, 0, TX);
+    x2_item<FORM, MON>(a, blockIdx.x, smem_raw, threadIdx.x, TX);
 }
 
 // ---------------------------------------------------------------------------
@@ -555,7 +552,7 @@ __global__ void __launch_bounds__(TX, X2Occ<FORM, TX>::value) step_kernel_x2_mul
         if (s > 0 && !tile_wait(a.done, a.nbr + b * kMaxTileNbr, s + a.wait_extra, a.wait_limit, a.status, abort_flag,
                                 &s_bad, tid))
             return;
-        x2_item<FORM, MON ? 2 : 0>(a, item, smem_raw, tid, 0, 0, TX, (s & 1) != 0, s);
+        x2_item<FORM, MON ? 2 : 0>(a, item, smem_raw, tid, TX, (s & 1) != 0, s);
         __syncthreads();   // every thread's stores of step s issued
         if (!MON && tid == 0) {   // (the monitored item publishes itself, before its monitor tree)
             __threadfence();
@@ -626,7 +623,7 @@ __global__ void __launch_bounds__(kBatchedTX, X2Occ<FORM, kBatchedTX>::value) st
         const int gq = s_next;
         if (s_abort) break;
         const int s = gq / a.ndesc, item = gq - s * a.ndesc;
-        x2_item<FORM, MON>(a, item, smem_raw, tid, 0, 0, TX, !MON && (s & 1) != 0);
+        x2_item<FORM, MON>(a, item, smem_raw, tid, TX, !MON && (s & 1) != 0);
         __syncthreads();   // every thread's stores issued; the rings and s_next free
         if (tid == 0) {    // publish: one more item of this instance finished
             __threadfence();
