@@ -368,17 +368,18 @@ bool use_batched(const lbm_ctx* c, bool f_pairs, bool f_async, bool f_tma) {
 // prologue), waves of `target` blocks counted whole -- one exact wave where the
 // strips allow it; runs of at least 8 rows. *cost: that product.
 int march_rows(int ny, int strips, long long target, long long* cost) {
-    long long best = -1, best_cost = 0;
-    for (long long r = 1; r <= ny; ++r) {
-        const long long rr = (ny + r - 1) / r;
-        if (rr < 8 && r > 1) break;
-        const long long runs = (ny + rr - 1) / rr;
+    int best = 0;
+    long long best_cost = 0;
+    lbm::each_run_length(ny, [&](int rr) {
+        if (rr < 8 && rr < ny) return false;
+        const long long runs = ((long long)ny + rr - 1) / rr;
         const long long waves = (strips * runs + target - 1) / target;
         const long long k = waves * (rr + 3);
-        if (best < 0 || k < best_cost) { best = rr; best_cost = k; }
-    }
+        if (best == 0 || k < best_cost) { best = rr; best_cost = k; }
+        return true;
+    });
     if (cost) *cost = best_cost;
-    return (int)best;
+    return best;
 }
 
 lbm_status plan(lbm_ctx* c) {

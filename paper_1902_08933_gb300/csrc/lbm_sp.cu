@@ -837,15 +837,16 @@ lbm_status sp_plan(lbm_sp_ctx* c) {
         for (int threads = 64; threads <= kSpThreads; threads += 32) {
             const int strips = (units + threads - 3) / (threads - 2), w = (units + strips - 1) / strips;
             const long long target = slots(c->kernel, threads);
-            for (int r = 1; r <= c->p.ny; ++r) {
-                const int rows = (c->p.ny + r - 1) / r, runs = (c->p.ny + rows - 1) / rows;
+            lbm::each_run_length(c->p.ny, [&](int rows) {
+                const int runs = (c->p.ny + rows - 1) / rows;
                 const long long cost = ((long long)strips * runs + target - 1) / target * (rows + 2);
                 if (best < 0 || cost < best) {
                     best = cost;
                     c->threads = threads;
                     c->run = SpRun{rows, strips, w * c->cells};
                 }
-            }
+                return true;
+            });
         }
     }
     // Tiles, several steps a launch, while every tile is resident at once: a step of

@@ -96,6 +96,18 @@ bool march_neighbours(const WorkItem* items, int count, int tx, Dom&& dom, std::
     return true;
 }
 
+// Calls f(rows) for each run length that cuts ny rows into equal runs, the longest
+// (one run) first, until it returns false: the different values of ceil(ny / r),
+// about 2 sqrt(ny) of them.
+template <typename F>
+void each_run_length(int ny, F&& f) {
+    for (long long r = 1; r <= ny;) {
+        const int rows = (int)((ny + r - 1) / r);
+        if (!f(rows) || rows == 1) return;
+        r = (ny + (long long)rows - 2) / (rows - 1);   // the first r of a shorter run
+    }
+}
+
 // The smallest of 8 x 4, 8 x 8 and 16 x 8 units whose tiles (count(U, R) of them)
 // leave no SM with two; else 16 x 8.
 template <typename Count>

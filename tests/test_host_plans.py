@@ -151,3 +151,29 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_run_lengths_are_those_of_every_number_of_runs(tmp_path):
+    # the different ceil(ny / r) in order; the tallest grids accepted take few calls
+    run_cpp(tmp_path, r"""
+#include "lbm_tileplan.h"
+int main() {
+    for (int ny = 1; ny < 2000; ++ny) {
+        std::vector<int> want, got;
+        for (int r = 1; r <= ny; ++r)
+            if (want.empty() || want.back() != (ny + r - 1) / r) want.push_back((ny + r - 1) / r);
+        lbm::each_run_length(ny, [&](int rows) { got.push_back(rows); return true; });
+        if (got != want) return 1;
+    }
+    for (int ny : {79536431, 715827882, 2147483647}) {
+        long long calls = 0;
+        int last = 0;
+        lbm::each_run_length(ny, [&](int rows) { ++calls; last = rows; return true; });
+        if (last != 1 || calls > 100000) return 2;
+        calls = 0;
+        lbm::each_run_length(ny, [&](int rows) { ++calls; return rows >= 8; });
+        if (calls > 100000) return 3;
+    }
+    return 0;
+}
+""")
