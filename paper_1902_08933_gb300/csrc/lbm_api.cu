@@ -175,16 +175,12 @@ struct lbm_ctx {
     bool multi = false;            // persistent plan: several steps a launch
     long long step_launches = 0;   // kernel launches lbm_step has issued (graph nodes counted)
     int graph_launches = 0;        // kernel nodes of the captured graph
-    int* d_nbr = nullptr;          // persistent plan: neighbour items, kMaxTileNbr an item
-    int* d_multi_done = nullptr;   // persistent plan: steps finished per item, then the abort flag
+    lbm::ItemBuffers multi_buf;    // persistent plan: neighbours, step counters
     lbm::MultiMonitor mon_multi;   // persistent plan, every step of a launch monitored (kMultiSteps of them)
-    // tile plan (plan_tile): items, neighbours and step counters in one allocation
+    // tile plan (plan_tile)
     int tile_items = 0, tile_grid = 0, tile_ulog = 0, tile_occ = 0;
     bool tile_pair = false;
-    void* d_tile = nullptr;
-    WorkItem* d_tile_work = nullptr;
-    int* d_tile_nbr = nullptr;
-    int* d_tile_done = nullptr;
+    lbm::ItemBuffers tile_buf;     // its items, neighbours and step counters
     bool plan_dirty = true;
     // CUDA graph of 2 * graph_pairs steps starting from cur == 0 (built on first use,
     // dropped when the plan changes)
@@ -331,9 +327,11 @@ void choose(const lbm_ctx* c, const lbm_params& p, bool f_pairs, bool f_async, b
     *variant = v;
     if (c->tile_req) *tile = c->tile_req;
     else *tile = v == lbm::kPairs ? default_tile_pairs(p.nx) : default_tile(p.nx);
-    // one cell a thread, state well inside L2: narrow strips where they pad less (517
-    // x 1033 f32, 0.6 of L2, 29.2 -> 26.1 us a step; 701 x 1500 FP16 g, 0.96 of L2,
-    // 50.7 and 53.0)
+    // one cell a thread, state well inside L2: narrow strips where they pad less. us a
+    // step with strips of 128 and 32 columns, at the state's share of L2: f32 517 wide
+    // 31.5 and 28.8 (0.6), 42.0 and 39.2 (0.85), 49.7 and 50.9 (1.04), 55.0 and 57.7
+    // (1.2); 651 wide 34.9 and 30.8 (0.7); f32_c 517 wide 32.8 and 30.8 (0.7), 43.7 and
+    // 41.1 (0.94), 57.2 and 59.9 (1.35); FP16 g 41.2 and 36.6 (0.65), 54.2 and 56.8 (0.93)
     if (!c->tile_req && v == lbm::kAsync && c->l2_share <= 0.75 &&
         (p.nx + 31) / 32 * 32 * 1.05 < (p.nx + *tile - 1) / *tile * *tile)
         *tile = 32;
@@ -572,15 +570,11 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
         return lbm::Domain{c->params[k].nx, c->params[k].ny, c->params[k].bc_y != LBM_BC_BOUNCEBACK};
     };
     if (!lbm::march_neighbours(c->work.data() + L.offset, L.count, L.tx, domain, nbr)) return LBM_OK;
-    cudaFree(c->d_nbr);
-    c->d_nbr = nullptr;
-    cudaFree(c->d_multi_done);
-    c->d_multi_done = nullptr;
     cudaFree(c->mon_multi.slots);
     c->mon_multi = lbm::MultiMonitor();
-    LBM_CK(c, cudaMalloc(&c->d_nbr, nbr.size() * sizeof(int)));
-    LBM_CK(c, cudaMemcpy(c->d_nbr, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LBM_CK(c, cudaMalloc(&c->d_multi_done, ((size_t)L.count + 1) * sizeof(int)));
+    const cudaError_t e = c->multi_buf.upload({}, nbr);
+    if (e == cudaErrorMemoryAllocation) return LBM_OK;   // as PAIRS
+    if (e != cudaSuccess) return cuda_fail(c, e, "persistent plan upload");
     c->multi = true;
     if (c->monitor) multi_monitor(c);
     return LBM_OK;
@@ -603,9 +597,12 @@ lbm_status plan_multi(lbm_ctx* c, int sms) {
 // 1024 (4) 26 and 27.5, 1024 x 1024 (7) 58 and 41: up to 3 rounds. One cell a
 // thread in FP32: 513 x 513 (3) 16.5 and 25.0, 517 x 1033 (6) 33 and 31: up to 4.
 // FP64 is bound by its arithmetic either way, so the tile wins by balance: 512 x
-// 512 121 and 146, 517 x 1033 (5 strips of 128 for 4.04) 248 and 308, 1024 x 1024
-// 471 and 456: taken while 1.2 x rounds x blocks stays below the march's waves x
-// (rows + 3) x blocks, both in units of 128 cells.
+// 512 121 and 146, 517 x 1033 (5 strips of 128 for 4.04) 248 and 308, the same far
+// beyond L2 (517 x 16 000 3755 and 4274, 130 x 40 000 2452 and 3321), 1024 x 1024 471
+// and 456: taken while 1.2 x rounds x blocks stays below the march's waves x (rows +
+// 3) x blocks, both in units of 128 cells. Several FP64 instances, 16 rounds: 4 x 64^2
+// 12.5 and 18.7, 64 x 64^2 122 and 178, 32 x 128^2 (15 rounds) 245 and 281, 8 x 256^2
+// (14) 245 and 284, 60 x 128^2 (28; the march) 476.
 lbm_status plan_tile(lbm_ctx* c, int sms) {
     c->tile_items = 0;
     if (c->d3 || c->pipeline != LBM_PIPELINE_AUTO || c->tile_req || c->rows_req) return LBM_OK;
@@ -657,21 +654,10 @@ lbm_status plan_tile(lbm_ctx* c, int sms) {
         const lbm_params& p = c->params[k];
         lbm::add_tiles(list, k, p.nx, p.ny, cpt, p.bc_y != LBM_BC_BOUNCEBACK, U, R);
     }
-    const std::vector<WorkItem>& items = list.items;
-    const std::vector<int>& nbr = list.nbr;
-    const size_t wb = (items.size() * sizeof(WorkItem) + 255) & ~size_t(255);
-    const size_t nb = (nbr.size() * sizeof(int) + 255) & ~size_t(255);
-    const size_t db = (items.size() + 1) * sizeof(int);
-    cudaFree(c->d_tile);
-    c->d_tile = nullptr;
-    LBM_CK(c, cudaMalloc(&c->d_tile, wb + nb + db));
-    c->d_tile_work = static_cast<WorkItem*>(c->d_tile);
-    c->d_tile_nbr = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb);
-    c->d_tile_done = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb + nb);
-    LBM_CK(c, cudaMemcpy(c->d_tile_work, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-    LBM_CK(c, cudaMemcpy(c->d_tile_nbr, nbr.data(), nbr.size() * sizeof(int), cudaMemcpyHostToDevice));
-    LBM_CK(c, cudaMemset(c->d_tile_done, 0, db));
-    c->tile_items = (int)items.size();
+    const cudaError_t e = c->tile_buf.upload(list.items, list.nbr);
+    if (e == cudaErrorMemoryAllocation) return LBM_OK;   // the march serves every step
+    if (e != cudaSuccess) return cuda_fail(c, e, "tile plan upload");
+    c->tile_items = (int)list.items.size();
     c->tile_grid = (int)std::min<long long>(c->tile_items, slots);
     c->tile_occ = occ;
     c->tile_ulog = ulog;
@@ -837,9 +823,8 @@ void release(lbm_ctx* c) {
     cudaFree(c->d_work);
     cudaFree(c->d_queue);
     cudaFree(c->d_done);
-    cudaFree(c->d_nbr);
-    cudaFree(c->d_multi_done);
-    cudaFree(c->d_tile);
+    c->multi_buf.release();
+    c->tile_buf.release();
     cudaFree(c->mon_multi.slots);
     cudaFree(c->d_tmp);
     cudaFree(c->d_out);
@@ -1100,7 +1085,7 @@ bool multi_plan(const lbm_ctx* c) {
 cudaError_t enqueue_multi(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, int wait_limit = lbm::kWaitLimit,
                           lbm::MonRecord* host_records = nullptr) {
     const auto& L = c->launches[0];
-    cudaError_t e = cudaMemsetAsync(c->d_multi_done, 0, ((size_t)L.count + 1) * sizeof(int), c->stream);
+    cudaError_t e = cudaMemsetAsync(c->multi_buf.done, 0, ((size_t)L.count + 1) * sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
     const bool monitor = host_records != nullptr;
     if (monitor) {
@@ -1111,8 +1096,8 @@ cudaError_t enqueue_multi(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, in
     }
     StepArgs a = step_args(c, in);
     a.work = c->d_work + L.offset;
-    a.nbr = c->d_nbr;
-    a.done = c->d_multi_done;
+    a.nbr = c->multi_buf.nbr;
+    a.done = c->multi_buf.done;
     a.ndesc = L.count;
     a.nsteps = nsteps;
     a.wait_extra = wait_extra;
@@ -1141,13 +1126,13 @@ bool tile_plan(const lbm_ctx* c) { return !c->d3 && c->tile_items > 0; }
 // wait_extra / wait_limit as in StepArgs.
 cudaError_t enqueue_tile(lbm_ctx* c, int in, int nsteps, int wait_extra = 0, int wait_limit = lbm::kWaitLimit) {
     if (nsteps > 1) {
-        cudaError_t e = cudaMemsetAsync(c->d_tile_done, 0, ((size_t)c->tile_items + 1) * sizeof(int), c->stream);
+        cudaError_t e = cudaMemsetAsync(c->tile_buf.done, 0, ((size_t)c->tile_items + 1) * sizeof(int), c->stream);
         if (e != cudaSuccess) return e;
     }
     StepArgs a = step_args(c, in);
-    a.work = c->d_tile_work;
-    a.nbr = c->d_tile_nbr;
-    a.done = c->d_tile_done;
+    a.work = c->tile_buf.work;
+    a.nbr = c->tile_buf.nbr;
+    a.done = c->tile_buf.done;
     a.ndesc = c->tile_items;
     a.nsteps = nsteps;
     a.wait_extra = wait_extra;

@@ -748,10 +748,7 @@ struct lbm_sp_ctx {
     int threads = kSpThreads;
     const void* tile = nullptr;        // small domains: several steps a launch (null: not taken)
     int tile_items = 0, tile_grid = 0, tile_ulog = 0;
-    void* d_tile = nullptr;            // items, neighbours, step counters and abort flag
-    lbm::WorkItem* d_tile_work = nullptr;
-    int* d_tile_nbr = nullptr;
-    int* d_tile_done = nullptr;
+    lbm::ItemBuffers tile_buf;         // items, neighbours, step counters and abort flag
     int* d_status = nullptr;           // set by a bounded wait that ran out
     std::string err;
 };
@@ -773,7 +770,7 @@ void sp_release(lbm_sp_ctx* c) {
     cudaFree(c->g[1]);
     cudaFree(c->src);
     cudaFree(c->ufield);
-    cudaFree(c->d_tile);
+    c->tile_buf.release();
     cudaFree(c->d_status);
     cudaFree(c->d_tmp);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -868,18 +865,12 @@ lbm_status sp_plan(lbm_sp_ctx* c) {
     }
     lbm::TileList list;
     lbm::add_tiles(list, 0, c->p.nx, c->p.ny, c->cells, c->p.bc_y != LBM_BC_BOUNCEBACK, U, R);
-    const size_t wb = (list.items.size() * sizeof(lbm::WorkItem) + 255) & ~size_t(255);
-    const size_t nb = (list.nbr.size() * sizeof(int) + 255) & ~size_t(255);
-    const size_t db = (list.items.size() + 1) * sizeof(int);
-    cudaError_t r = cudaMalloc(&c->d_tile, wb + nb + db);
-    if (r != cudaSuccess) return r == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
-    c->d_tile_work = static_cast<lbm::WorkItem*>(c->d_tile);
-    c->d_tile_nbr = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb);
-    c->d_tile_done = reinterpret_cast<int*>(static_cast<char*>(c->d_tile) + wb + nb);
-    if (cudaMemcpy(c->d_tile_work, list.items.data(), list.items.size() * sizeof(lbm::WorkItem),
-                   cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(c->d_tile_nbr, list.nbr.data(), list.nbr.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
-        return LBM_ECUDA;
+    const cudaError_t e = c->tile_buf.upload(list.items, list.nbr);
+    if (e == cudaErrorMemoryAllocation) {   // no room: a launch a step
+        c->tile = nullptr;
+        return LBM_OK;
+    }
+    if (e != cudaSuccess) return LBM_ECUDA;
     c->tile_items = (int)list.items.size();
     c->tile_grid = c->tile_items;
     while ((1 << c->tile_ulog) < U) ++c->tile_ulog;
@@ -916,9 +907,9 @@ cudaError_t sp_step_tiles(lbm_sp_ctx* c, int n, int wait_extra = 0, int wait_lim
     a.ulog = c->tile_ulog;
     a.wait_limit = wait_limit;
     a.wait_extra = wait_extra;
-    a.work = c->d_tile_work;
-    a.nbr = c->d_tile_nbr;
-    a.done = c->d_tile_done;
+    a.work = c->tile_buf.work;
+    a.nbr = c->tile_buf.nbr;
+    a.done = c->tile_buf.done;
     a.status = c->d_status;
     if (n > 1) {
         const cudaError_t e = cudaMemsetAsync(a.done, 0, ((size_t)c->tile_items + 1) * sizeof(int), c->stream);

@@ -12,8 +12,8 @@
 //      of the tile and its halo into shared memory, p with a 1-cell halo;
 //   B. mu (Eq. 8) of the tile and a 1-cell ring;
 //   C. the collision and push of the tile's cells.
-// The halo costs 1.7 to 3 loads of h a cell, from L2 (the grids this serves fit
-// there). The arithmetic is that of the marches, cell by cell (phi in the same
+// The halo costs 1.7 to 3 loads of h a cell, from L2 where the grid fits there; FP64
+// runs larger grids on tiles too, bound by its operations either way. The arithmetic is that of the marches, cell by cell (phi in the same
 // order of summation, chem_pot, macroscopic, collide_emit).
 //
 // One cooperative launch runs several steps: block b takes items b, b + gridDim,

@@ -56,6 +56,49 @@ inline void add_tiles(TileList& out, int inst, int nx, int ny, int cpt, bool per
         }
 }
 
+// What a launch of several steps keeps on the device: its items (those of a row march
+// are the context's, nwork = 0), their neighbours, and the steps finished per item
+// followed by the abort flag. One allocation or none.
+struct ItemBuffers {
+    void* base = nullptr;
+    WorkItem* work = nullptr;
+    int *nbr = nullptr, *done = nullptr;
+    // alloc(void**, bytes): whether it was had
+    template <typename Alloc>
+    bool allocate(size_t nwork, size_t items, Alloc&& alloc) {
+        auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+        const size_t wb = up(nwork * sizeof(WorkItem)), nb = up(items * kMaxTileNbr * sizeof(int));
+        void* p = nullptr;
+        *this = ItemBuffers();
+        if (!alloc(&p, wb + nb + (items + 1) * sizeof(int)) || !p) return false;
+        base = p;
+        work = reinterpret_cast<WorkItem*>(p);
+        nbr = reinterpret_cast<int*>(static_cast<char*>(p) + wb);
+        done = reinterpret_cast<int*>(static_cast<char*>(p) + wb + nb);
+        return true;
+    }
+    void release() {
+        cudaFree(base);
+        *this = ItemBuffers();
+    }
+    // Allocates and fills them. cudaErrorMemoryAllocation (cleared): there is no room,
+    // and the plan that wanted them is not made.
+    cudaError_t upload(const std::vector<WorkItem>& items, const std::vector<int>& neighbours) {
+        release();
+        const size_t n = neighbours.size() / kMaxTileNbr;
+        cudaError_t e = cudaSuccess;
+        if (!allocate(items.size(), n, [&e](void** p, size_t b) { return (e = cudaMalloc(p, b)) == cudaSuccess; })) {
+            cudaGetLastError();
+            return e;
+        }
+        if (!items.empty()) e = cudaMemcpy(work, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(nbr, neighbours.data(), neighbours.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemset(done, 0, (n + 1) * sizeof(int));
+        if (e != cudaSuccess) release();
+        return e;
+    }
+};
+
 struct Domain {
     int nx, ny;
     bool per_y;   // periodic in y (in x always)

@@ -177,3 +177,27 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_item_buffers_come_all_or_not_at_all(tmp_path):
+    run_cpp(tmp_path, r"""
+#include <cstdint>
+#include <cstdlib>
+#include "lbm_tileplan.h"
+extern "C" cudaError_t cudaFree(void*) { return cudaSuccess; }
+int main() {
+    for (size_t nwork : {0, 1, 11, 456}) for (size_t items : {1, 11, 456}) {
+        lbm::ItemBuffers b;
+        if (b.allocate(nwork, items, [](void**, size_t) { return false; }) || b.base || b.work || b.nbr || b.done) return 1;
+        size_t bytes = 0;
+        if (!b.allocate(nwork, items, [&](void** p, size_t n) { *p = std::malloc(bytes = n); return true; })) return 2;
+        const char *w = (char*)b.work, *n = (char*)b.nbr, *d = (char*)b.done;
+        if (w != b.base || n < w + nwork * sizeof(lbm::WorkItem) || d < n + items * lbm::kMaxTileNbr * sizeof(int)) return 3;
+        if (d + (items + 1) * sizeof(int) > w + bytes || (uintptr_t)n % 4 || (uintptr_t)d % 4) return 4;
+        std::free(b.base);
+        b.release();
+        if (b.base || b.work || b.nbr || b.done) return 5;
+    }
+    return 0;
+}
+""")
