@@ -1252,7 +1252,7 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
     const bool mon_last = c->monitor && nsteps > 0;
     int left = mon_last ? nsteps - 1 : nsteps;
     while (left > 0 && tile_plan(c)) {   // launches of up to 256 steps
-        const int n = std::min(left, 256);
+        const int n = std::min(left, lbm::kLaunchSteps);
         cudaError_t e = enqueue_tile(c, c->cur, n);
         if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
         ++c->step_launches;
@@ -1279,7 +1279,7 @@ lbm_status lbm_step(lbm_ctx* c, int nsteps) {
         }
     }
     while (left > 0 && (batched_plan(c) || (multi_plan(c) && left > 1))) {   // launches of up to 256 steps
-        const int n = std::min(left, 256);
+        const int n = batched_plan(c) ? lbm::batched_steps(left, c->ndesc) : std::min(left, lbm::kLaunchSteps);
         cudaError_t e = batched_plan(c) ? enqueue_batched(c, c->cur, n) : enqueue_multi(c, c->cur, n);
         if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
         ++c->step_launches;

@@ -1045,7 +1045,7 @@ lbm_status lbm_sp_step(lbm_sp_ctx* c, int nsteps) {
     if (nsteps < 0) return sp_fail(c, LBM_EINVAL, "nsteps < 0");
     if (!c->ready) return sp_fail(c, LBM_ESTATE, "not initialised");
     for (int s = 0; s < nsteps;) {
-        const int n = c->tile ? (nsteps - s < 256 ? nsteps - s : 256) : 1;
+        const int n = c->tile ? std::min(nsteps - s, lbm::kLaunchSteps) : 1;
         const cudaError_t e = c->tile ? sp_step_tiles(c, n) : sp_step_once(c);
         if (e != cudaSuccess) return sp_cuda(c, e, "step kernel");
         s += n;

@@ -139,6 +139,14 @@ bool march_neighbours(const WorkItem* items, int count, int tx, Dom&& dom, std::
     return true;
 }
 
+// Steps of one launch: 256 at most, and what the batched queue can count -- steps x
+// items, past which every block counts on once, stay below 2^31.
+constexpr int kLaunchSteps = 256;
+inline int batched_steps(int left, int items) {
+    constexpr int kMost = 0x7fffffff - (1 << 20);   // (1 << 20: more blocks than are ever resident)
+    return std::max(1, std::min(std::min(left, kLaunchSteps), kMost / std::max(1, items)));
+}
+
 // Calls f(rows) for each run length that cuts ny rows into equal runs, the longest
 // (one run) first, until it returns false: the different values of ceil(ny / r),
 // about 2 sqrt(ny) of them.

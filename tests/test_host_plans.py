@@ -201,3 +201,20 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_batched_queue_counts_stay_below_2_31(tmp_path):
+    # 1.1e9 cells in items of 128 x 1 (run length 1 asked for) are 8.6 million items a step
+    run_cpp(tmp_path, r"""
+#include "lbm_tileplan.h"
+int main() {
+    for (long long items : {1LL, 700LL, 8000000LL, 8388608LL, 8600000LL, 16777216LL, 2000000000LL})
+        for (int left : {1, 2, 255, 256, 257, 100000}) {
+            const int n = lbm::batched_steps(left, (int)items);
+            if (n < 1 || n > left || n > 256) return 1;
+            if (n * items + (1 << 20) > 0x7fffffffLL) return 2;
+            if (items < 8000000 && n != (left < 256 ? left : 256)) return 3;
+        }
+    return 0;
+}
+""")
