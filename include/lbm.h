@@ -341,6 +341,12 @@ lbm_status lbm_set_launch(lbm_ctx* ctx, int tile_x, int rows);
  *                      launch in which a tile's step waits (bounded) for the
  *                      tiles within 3 cells of it only, while the launch shape
  *                      is the built-in one (lbm_set_launch(ctx, 0, 0)).
+ * A launch of several steps is cooperative and keeps its share of every SM from
+ * its first step to its last (a 1024 x 4096 FP32 domain: up to 256 steps, 30 ms).
+ * Kernels that do not fit beside it -- of other streams, other contexts' steps
+ * among them -- run before or after it, not at its step boundaries. Where other
+ * work must get in between, take fewer steps a call, or a plan of a launch a step:
+ * LBM_PIPELINE_PAIRS (ASYNC for nx odd, PLAIN for FP64).
  * An instance that cannot use a variant falls back to PLAIN. Takes effect at
  * the next lbm_step. LBM_EINVAL for an unknown mode.
  * D3Q15 contexts: PLAIN runs the unfused step (phi, mu and the collision as
@@ -526,7 +532,9 @@ void lbm_destroy(lbm_ctx* ctx);
  * div u (as printed); the source field is S_1, (force_x, force_y) is F_1, p0 > 0.
  * One kernel a step; domains whose tiles fit on the GPU at once run up to 256
  * steps in one cooperative launch with bounded waits between tiles: one that ran
- * out makes the read-backs return LBM_ETIMEOUT until lbm_sp_init. */
+ * out makes the read-backs return LBM_ETIMEOUT until lbm_sp_init. Such a launch
+ * keeps its SMs for all its steps (a 256 x 256 domain: about 1 ms in FP32); fewer
+ * steps a call let other streams' kernels in sooner. */
 enum { LBM_SP_INCOMPRESSIBLE_SOURCE = 0, LBM_SP_NEARLY_INCOMPRESSIBLE = 1, LBM_SP_HE_INCOMPRESSIBLE = 2 };
 /* scheme LBM_SP_SCHEME_REMARK4 (with model LBM_SP_INCOMPRESSIBLE_SOURCE only)
  * evolves the Remark 3 model with the explicit discretization of D_i G_i of
